@@ -323,15 +323,26 @@ cudaError_t ensure_scratch(Call &c, size_t *summ_off) {
   return ensure_giant(*c.ctx, counters + pw * (rp >> 10), c.st);
 }
 
-// Per-CTA scratch of the giant bin: 4 ints per wedge of the largest row.
-cudaError_t giant_scratch(Call &c, int32_t max_work, WalkLaunch *L) {
+// Scratch of the giant and dense bins (their kernels run one after the other
+// and share it): 4 ints per wedge of the largest giant row and giant CTA;
+// the dense bin's per-CTA need for its largest row.  Sets L's dense_pairs,
+// dense_size and giant_stride and returns the ints.
+size_t scratch_ints(WalkLaunch *L, int32_t max_giant, long long pairs_big, long long pairs_small,
+                    int32_t dense_size) {
+  L->giant_stride = 4ll * max_giant;
+  L->dense_pairs[0] = pairs_big;
+  L->dense_pairs[1] = pairs_small;
+  L->dense_size = dense_size;
+  return std::max((size_t)giant_ctas() * (size_t)L->giant_stride,
+                  (size_t)dense_ints(pairs_big, pairs_small, dense_size));
+}
+
+cudaError_t giant_scratch(Call &c, int32_t max_giant, long long pairs_big, long long pairs_small,
+                          int32_t dense_size, WalkLaunch *L) {
   L->giant_scratch = nullptr;
-  L->giant_stride = 0;
-  if (max_work <= 0) return cudaSuccess;
-  const long long stride = 4ll * max_work;
-  cudaError_t e = c.pool->get(&L->giant_scratch, (size_t)giant_ctas() * (size_t)stride);
-  if (e == cudaSuccess) L->giant_stride = stride;
-  return e;
+  const size_t n = scratch_ints(L, max_giant, pairs_big, pairs_small, dense_size);
+  L->scratch_ints = (long long)n;
+  return n ? c.pool->get(&L->giant_scratch, n) : cudaSuccess;
 }
 
 thread_local int32_t t_err_where = 0;  // kWhere* of the last device-raised error
@@ -349,7 +360,6 @@ WalkLaunch walk_launch(Call &c, int mode, int32_t smin, int32_t list_base) {
   L.a.unweighted = c.unweighted;
   L.a.row_s = c.sd.row_s;
   L.a.row_fhi = c.sd.row_fhi;
-  L.a.dense_ratio = t_bins.dense;
   L.a.smin = smin;
   L.a.row_begin = list_base;
   L.a.n_e = c.w.n_e;
@@ -508,7 +518,15 @@ int run_binned(Call &c, int64_t *result) {
   const unsigned giant_rest0 = mp.giant_rest;
   WalkLaunch L = walk_launch(c, c.op == kOpBuild ? kStage : kCount, c.smin, c.row_begin);
   L.a.core = core;
-  SLG_TRY(giant_scratch(c, max_giant, &L));
+  // pairs of a dense row: every one has s wedges or a tile count
+  auto dense_pairs = [&](unsigned rows, int32_t work) -> long long {
+    if (!rows) return 0;
+    const long long p = work / c.smin + (core.T ? core.n_core : 0);
+    return std::max(std::min<long long>(p, c.sd.R), 1ll);
+  };
+  SLG_TRY(giant_scratch(c, max_giant, dense_pairs(mp.dense_huge, mp.max_dense_work[0]),
+                        dense_pairs(mp.dense_rest, mp.max_dense_work[1]), mp.max_dense_size,
+                        &L));
   L.w.r_off = c.sd.r_off;
   L.w.r_idx = c.sd.r_idx;
   L.w.c_idx_s = w.c_idx_s;
@@ -539,6 +557,10 @@ int run_binned(Call &c, int64_t *result) {
     } else {
       // Staging too small: walk again, writing straight to the output.
       SLG_TRY(cudaMemsetAsync(&w.meta->giant_ticket, 0, sizeof(unsigned int), c.st));
+      static_assert(offsetof(Meta, dense_ticket_rest) ==
+                        offsetof(Meta, dense_ticket) + sizeof(unsigned int),
+                    "the two dense ticket counters are cleared together");
+      SLG_TRY(cudaMemsetAsync(&w.meta->dense_ticket, 0, 2 * sizeof(unsigned int), c.st));
       static_assert(offsetof(Meta, sparse_ticket_rest) ==
                         offsetof(Meta, sparse_ticket) + sizeof(unsigned int),
                     "the two sparse ticket counters are cleared together");
@@ -650,7 +672,10 @@ int run_spgemm(Call &c, int64_t *result) {
   w.stage_cap = budget;
   WalkLaunch Lg = walk_launch(c, kStage, 1, c.row_begin);
   Lg.a.full_rows = 1;
-  SLG_TRY(giant_scratch(c, max_row > kCtaLMaxWork ? (int32_t)max_row : 0, &Lg));
+  SLG_TRY(giant_scratch(c, max_row > kCtaLMaxWork ? (int32_t)max_row : 0,
+                        max_row > kDenseMinWork ? std::min<long long>(max_row, c.sd.R) : 0,
+                        max_row > kDenseMinWork ? std::min<long long>(max_row, c.sd.R) : 0,
+                        c.meta_host->max_row_size, &Lg));
   long long total_out = 0, products = 0;
   int32_t r0 = 0;
   if (c.evs->on) cudaEventRecord(c.evs->ev[kEvWalk], c.st);
@@ -709,7 +734,8 @@ int run(const slg_hypergraph *h, int32_t smin, uint32_t flags, int32_t row_begin
         int32_t row_end, Op op, int32_t *out_i, int32_t *out_j, int32_t *out_w,
         int64_t capacity, int64_t *result, cudaStream_t st, const int32_t *row_s = nullptr,
         int32_t *max_row_work = nullptr, long long *row_ptr_out = nullptr,
-        int32_t *row_work_out = nullptr, const int32_t *row_fhi = nullptr) {
+        int32_t *row_work_out = nullptr, const int32_t *row_fhi = nullptr,
+        int32_t *max_row_size = nullptr) {
   int rc = check_args(h, smin, flags);
   if (rc != SLG_OK) return rc;
   if (!result) return SLG_ERR_INVALID;
@@ -773,7 +799,7 @@ int run(const slg_hypergraph *h, int32_t smin, uint32_t flags, int32_t row_begin
   SLG_TRY(pool.get(&w.tail_beg, (size_t)nnz));
   SLG_TRY(pool.get(&w.tail_end, (size_t)nnz));
   SLG_TRY(pool.get(&w.tile, (size_t)ntiles + 1));
-  SLG_TRY(pool.get(&w.bin_rows, (size_t)kNumBins * (c.rows > 0 ? c.rows : 1)));
+  SLG_TRY(pool.get(&w.bin_rows, (size_t)kNumLists * (c.rows > 0 ? c.rows : 1)));
   SLG_TRY(pool.get(&w.n_e, (size_t)c.rows + 1));
   SLG_TRY(pool.get(&w.row_work, (size_t)c.rows + 1));
   SLG_TRY(pool.get(&w.stage_pos, (size_t)c.rows + 1));
@@ -852,7 +878,13 @@ int run(const slg_hypergraph *h, int32_t smin, uint32_t flags, int32_t row_begin
     stats.incid_bin[b] = (int64_t)m.incid_bin[b];
     stats.pairs_bin[b] = (int64_t)m.pairs_bin[b];
   }
+  // the dense bin's rows are reported as giant ones
+  stats.rows_bin[kBinGiant] += (int64_t)m.rows_bin[kBinDense];
+  stats.wedges_bin[kBinGiant] += (int64_t)m.wedges_bin[kBinDense];
+  stats.incid_bin[kBinGiant] += (int64_t)m.incid_bin[kBinDense];
+  stats.pairs_bin[kBinGiant] += (int64_t)m.pairs_bin[kBinDense];
   if (max_row_work) *max_row_work = m.max_row_work;
+  if (max_row_size) *max_row_size = m.max_row_size;
   stats.kernel_launches = c.launches;
   stats.core_rows = c.core_rows;
   stats.core_cols = c.core_cols;
@@ -922,7 +954,7 @@ struct slg_plan {
   int32_t *row_base = nullptr;     // [count + 1] first row of each member (side)
   slg::Work w = {};
   int32_t *giant = nullptr;
-  long long giant_stride = 0;
+  slg::WalkLaunch scratch = {};    // giant_stride, dense_pairs, dense_size, scratch_ints
   int32_t *out_i = nullptr, *out_j = nullptr, *out_w = nullptr;
   long long *offsets = nullptr;    // [count + 1]
   int64_t pairs = 0;
@@ -962,7 +994,6 @@ cudaError_t enqueue_plan(slg_plan *p, const Bins &bins, cudaStream_t st, int32_t
   L.a.unweighted = (p->flags & SLG_UNWEIGHTED) != 0;
   L.a.row_s = sd.row_s;
   L.a.row_fhi = sd.row_fhi;
-  L.a.dense_ratio = bins.dense;
   L.a.smin = 1;
   L.a.row_begin = 0;
   L.a.n_e = w.n_e;
@@ -977,7 +1008,11 @@ cudaError_t enqueue_plan(slg_plan *p, const Bins &bins, cudaStream_t st, int32_t
   L.rows = sd.R;
   L.R = sd.R;
   L.giant_scratch = p->giant;
-  L.giant_stride = p->giant_stride;
+  L.giant_stride = p->scratch.giant_stride;
+  L.dense_pairs[0] = p->scratch.dense_pairs[0];
+  L.dense_pairs[1] = p->scratch.dense_pairs[1];
+  L.dense_size = p->scratch.dense_size;
+  L.scratch_ints = p->scratch.scratch_ints;
   int32_t n = 0;
   if (sd.R > 0) PLAN_TRY(launch_walk(L, st, &n));
   PLAN_TRY(launch_row_scan(sd.R, w, st));
@@ -1661,9 +1696,9 @@ extern "C" int slg_plan_create(const slg_hypergraph *hs, const int32_t *s, int32
   p->sd.row_fhi = dual ? p->row_fhi_v : p->row_fhi_e;
   // 2. sizes: one counting pass over the union (per-row thresholds)
   int64_t pairs = 0;
-  int32_t max_work = 0;
+  int32_t max_work = 0, max_size = 0;
   int rc = run(&p->u, 1, flags, 0, p->sd.R, kOpCount, nullptr, nullptr, nullptr, 0, &pairs, st,
-               p->sd.row_s, &max_work, nullptr, nullptr, p->sd.row_fhi);
+               p->sd.row_s, &max_work, nullptr, nullptr, p->sd.row_fhi, &max_size);
   if (rc != SLG_OK) return rc;
   p->pairs = pairs;
   // 3. persistent buffers
@@ -1677,7 +1712,7 @@ extern "C" int slg_plan_create(const slg_hypergraph *hs, const int32_t *s, int32
   SLG_TRY(p->mem.get(&w.tail_beg, (size_t)nnz));
   SLG_TRY(p->mem.get(&w.tail_end, (size_t)nnz));
   SLG_TRY(p->mem.get(&w.tile, (size_t)((nnz + 4095) / 4096) + 1));
-  SLG_TRY(p->mem.get(&w.bin_rows, (size_t)kNumBins * (R > 0 ? R : 1)));
+  SLG_TRY(p->mem.get(&w.bin_rows, (size_t)kNumLists * (R > 0 ? R : 1)));
   SLG_TRY(p->mem.get(&w.n_e, (size_t)R + 1));
   SLG_TRY(p->mem.get(&w.row_work, (size_t)R + 1));
   SLG_TRY(p->mem.get(&w.stage_pos, (size_t)R + 1));
@@ -1691,12 +1726,14 @@ extern "C" int slg_plan_create(const slg_hypergraph *hs, const int32_t *s, int32
   SLG_TRY(p->mem.get(&p->out_w, (size_t)std::max<int64_t>(pairs, 1)));
   SLG_TRY(p->mem.get(&p->offsets, (size_t)count + 1));
   if (max_work > 0) {
-    p->giant_stride = 4ll * max_work;
-    SLG_TRY(p->mem.get(&p->giant, (size_t)giant_ctas() * (size_t)p->giant_stride));
+    const size_t n = scratch_ints(&p->scratch, max_work, std::min<long long>(max_work, R),
+                                  std::min<long long>(max_work, R), max_size);
+    p->scratch.scratch_ints = (long long)n;
+    SLG_TRY(p->mem.get(&p->giant, n));
   }
   // 4. autotuner: bin thresholds, timed on this batch
   // candidates: CTA-bin limits, the sparse bin's range (0: off) and the
-  // dense-row ratio of the giant bin
+  // dense-row ratio
   const Bins cands[] = {Bins{},
                         Bins{64, 1024, 4096},
                         Bins{128, 512, 4096},
@@ -1704,9 +1741,9 @@ extern "C" int slg_plan_create(const slg_hypergraph *hs, const int32_t *s, int32
                         Bins{128, 1024, 4096, 8192},
                         Bins{128, 1024, 4096, 0},
                         Bins{128, 1024, 2048, 16384, 2048},
-                        Bins{128, 1024, 4096, 16384, 4096, 4},
-                        Bins{128, 1024, 4096, 16384, 4096, 16},
-                        Bins{128, 1024, 4096, 16384, 4096, 8}};
+                        Bins{128, 1024, 4096, 16384, 1024, kDenseRatio / 2},
+                        Bins{128, 1024, 4096, 16384, 1024, kDenseRatio * 2},
+                        Bins{128, 1024, 4096, 16384, 4096}};
   cudaEvent_t t0, t1;
   SLG_TRY(cudaEventCreate(&t0));
   SLG_TRY(cudaEventCreate(&t1));

@@ -19,13 +19,15 @@ namespace slg {
 constexpr int kWarp = 32;
 constexpr int32_t kEmpty = -1;
 
-// Row bins by wedge work (the degree-binned scheduler).  Rows with s >= 2
-// from Bins::bloom up to Bins::sparse wedges go to the sparse bin, the ones
-// above the CTA bins only when their far ends are sparse in their id span
-// (fewer than one wedge per kDenseRatio ids); the other rows above the CTA
-// bins go to the giant bin (dense rows, s = 1, dense-core rows).
+// Row bins by wedge work (the degree-binned scheduler).  Rows above
+// kDenseMinWork wedges whose far ends are dense in their id span (is_dense)
+// go to the dense bin; of the others, rows with s >= 2 from Bins::bloom up to
+// Bins::sparse wedges go to the sparse bin and the rest above the CTA bins to
+// the giant bin.  The statistics count the dense bin's rows as giant ones
+// (kNumBins bins are reported, kNumLists lists are kept).
 enum Bin : int {
-  kBinWarp = 0, kBinCtaS = 1, kBinCtaL = 2, kBinGiant = 3, kBinSparse = 4, kNumBins = 5
+  kBinWarp = 0, kBinCtaS = 1, kBinCtaL = 2, kBinGiant = 3, kBinSparse = 4, kNumBins = 5,
+  kBinDense = 5, kNumLists = 6
 };
 
 // Upper bounds on a row's wedge count for each non-giant bin.  The hash tables
@@ -52,20 +54,41 @@ constexpr int32_t kGiantHugeWork = SLG_GIANT_HUGE_WORK;
 #endif
 constexpr int32_t kSparseBigWork = SLG_SP_BIG_WORK > 0 ? SLG_SP_BIG_WORK : kGiantHugeWork;
 // A row is dense when it has at least one wedge per this many ids of its far
-// ends' span (swept: 8 best for the giant bin's dense windows).
+// ends' span, for 16-bit counters (see is_dense).  Step of four builds on
+// chung_lu_1m: 137.2, 134.8, 137.1, 180 ms with 8, 16, 24, 48.
 #ifndef SLG_DENSE_RATIO
-#define SLG_DENSE_RATIO 8
+#define SLG_DENSE_RATIO 16
 #endif
 constexpr int kDenseRatio = SLG_DENSE_RATIO;
+#ifndef SLG_DENSE_MIN_WORK
+#define SLG_DENSE_MIN_WORK 1024
+#endif
+constexpr int32_t kDenseMinWork = SLG_DENSE_MIN_WORK;
+// Dense rows of more vertices (16-bit counters and up) take the instance of
+// the dense kernel with the larger windows.
+constexpr int32_t kDenseBigSize = 255;
+
+// log2 of the dense bin's counter width for a row of `size` vertices: a
+// count |e ∩ f| is at most `size`.
+__host__ __device__ __forceinline__ int dense_lg_bits(int32_t size) {
+  return size <= 15 ? 2 : size <= 255 ? 3 : size <= 65535 ? 4 : 5;
+}
+
+// Dense rows: the dense bin's cost per row is its wedges plus its counters
+// (span x bits), so the line is drawn at a number of wedges per counter byte.
+__host__ __device__ __forceinline__ bool is_dense(int32_t work, int32_t size, int32_t span,
+                                                  int32_t ratio) {
+  return ((long long)work * ratio << 4) >= ((long long)span << dense_lg_bits(size));
+}
 
 // Counters the device writes and the host reads once per call.
 struct Meta {
   int32_t err;                         // first slg_status raised on the device
   int32_t err_where;                   // which check raised it
-  unsigned long long rows_bin[kNumBins];
-  unsigned long long wedges_bin[kNumBins];
-  unsigned long long incid_bin[kNumBins];
-  unsigned long long pairs_bin[kNumBins];
+  unsigned long long rows_bin[kNumLists];
+  unsigned long long wedges_bin[kNumLists];
+  unsigned long long incid_bin[kNumLists];
+  unsigned long long pairs_bin[kNumLists];
   unsigned long long wedges;           // W_s
   unsigned long long active;           // rows with size >= s in range
   unsigned long long pairs;            // |L_s| over the row range
@@ -78,12 +101,19 @@ struct Meta {
   unsigned int sparse_ticket_rest;     // the small-table sparse kernel's own tickets
   unsigned int sparse_huge;
   unsigned int sparse_rest;
+  unsigned int dense_ticket;           // the same four for the dense bin (huge: kDenseBigSize)
+  unsigned int dense_ticket_rest;
+  unsigned int dense_huge;
+  unsigned int dense_rest;
+  int32_t max_dense_work[2];           // largest work of a dense-bin row: big instance, other
+  int32_t max_dense_size;              // most vertices of a dense-bin row
+  int32_t max_row_size;                // most vertices of a row with work
   int32_t max_sparse_work;             // largest work of a sparse-bin row
   int32_t kept;                        // entries of the filtered CSC
   int32_t max_giant_work;              // largest work of a giant-bin row
   unsigned long long nnz_core;         // incidences of the dense core
   int32_t max_row_work;                // largest work of any row
-  unsigned long long giant_cycles[4];  // giant bin: SM cycles in walk, partition, buckets
+  unsigned long long giant_cycles[4];  // giant bin: SM cycles in walk, partition, buckets; dense bin
   unsigned long long sparse_cycles[5]; // sparse bin: row set-up, walk, collect, emit, staging
 };
 
@@ -361,7 +391,7 @@ __device__ __forceinline__ int32_t s_of(const int32_t *row_s, int32_t smin, int3
 #define SLG_BLOOM_MIN_WORK 1024
 #endif
 // `dense`: a row with at least one wedge per `dense` ids of its far ends'
-// span is dense (the giant bin counts it in dense windows).
+// span is dense, for 16-bit counters (see is_dense).
 struct Bins {
   int32_t warp = kWarpMaxWork, ctas = kCtaSMaxWork, ctal = kCtaLMaxWork;
   int32_t sparse = SLG_SPARSE_MAX_WORK;
@@ -394,7 +424,7 @@ struct Work {
   int32_t *tail_beg;   // [nnz] tail of each incidence: [tail_beg, tail_end)
   int32_t *tail_end;   // [nnz]
   int32_t *tile;       // [ntiles + 1] scan scratch
-  int32_t *bin_rows;   // [kNumBins][R] row lists
+  int32_t *bin_rows;   // [kNumLists][R] row lists
   int32_t *n_e;        // [R] pairs per row
   int32_t *row_work;   // [R] wedges per row
   long long *stage_pos;// [R] staging offset per row, -1 = not staged
@@ -447,7 +477,6 @@ struct EmitArgs {
   int unweighted;
   const int32_t *row_s;               // per-row threshold, or null: smin
   const int32_t *row_fhi;             // per-row far-end bound, or null: R
-  int32_t dense_ratio;                // Bins::dense
   int full_rows;                      // 1: tails are whole columns, far ends in [0, R)
   const int32_t *row_work;            // [rows] wedges per row (giant bin)
   CoreInfo core;                      // dense core (tile counts added by the giant bin)
@@ -465,17 +494,22 @@ struct EmitArgs {
 struct WalkLaunch {
   Walk w;
   EmitArgs a;
-  const int32_t *bin_rows;  // [kNumBins][rows] row lists
+  const int32_t *bin_rows;  // [kNumLists][rows] row lists
   const int32_t *row_work;  // [rows] wedges per row
   int32_t rows;             // rows in the range (list stride)
   int32_t *giant_scratch;   // [giant_ctas][4 * max giant work] wedge ends + pairs
   long long giant_stride;   // ints per giant CTA
   int32_t R;                // rows of the side (far ends lie in [0, R))
+  long long scratch_ints;   // of giant_scratch
+  long long dense_pairs[2]; // most pairs a dense-bin row can have: big instance, other (0: no row)
+  int32_t dense_size;       // most vertices of a dense-bin row
 };
 
-// CTAs of the giant kernel (two per SM) and of the sparse kernel.
+// CTAs of the giant kernel (two per SM) and of the sparse kernel, and the
+// scratch ints of the dense kernels.
 int giant_ctas();
 int sparse_ctas();
+long long dense_ints(long long pairs_big, long long pairs_small, int32_t size_big);
 // The largest side (rows) a build supports: row ids and the giant bin's
 // super-chunk bounds stay below 2^31.
 constexpr int32_t kMaxRows = (int32_t)((1u << 31) - (1u << 23));
@@ -488,6 +522,8 @@ constexpr int32_t kComponentsMaxR = 1 << 24;
 constexpr int kWalkEv[kNumBins] = {0, 1, 2, 4, 3};
 cudaError_t launch_walk(const WalkLaunch &L, cudaStream_t st, int32_t *launches,
                         cudaEvent_t *ev = nullptr);
+cudaError_t launch_walk_sparse(const WalkLaunch &L, cudaStream_t st, int32_t *launches);
+cudaError_t launch_walk_dense(const WalkLaunch &L, cudaStream_t st, int32_t *launches);
 cudaError_t launch_row_scan(int32_t rows, const Work &w, cudaStream_t st);
 // The device Meta into host memory the device can address (mapped pinned
 // memory), by a kernel: no copy engine involved.

@@ -193,22 +193,23 @@ __global__ __launch_bounds__(kRowsNT) void k_rows_work(Side s, int32_t smin, int
                                                        Meta *meta) {
   if (meta->err) return;
   __shared__ int32_t s_work[kRowsPerBlock];
-  // block maxima of the row work (all rows, giant-bin rows, sparse-bin rows):
-  // one global atomicMax each per block instead of one per row
-  __shared__ int32_t s_max[3];
+  // block maxima of the row work (all rows, giant-bin, sparse-bin, the dense
+  // bin's two instances' rows) and size (dense-bin rows, all rows): one global atomicMax each per
+  // block instead of one per row
+  __shared__ int32_t s_max[7];
   __shared__ int32_t s_act;  // active rows (size >= s) of the block
-  __shared__ int32_t s_cnt[kNumBins], s_base[kNumBins];
-  __shared__ int32_t s_hcnt[2], s_hbase[2];  // giant / sparse rows handed out first
-  __shared__ unsigned long long s_w[kNumBins], s_k[kNumBins];
+  __shared__ int32_t s_cnt[kNumLists], s_base[kNumLists];
+  __shared__ int32_t s_hcnt[3], s_hbase[3];  // giant / sparse / dense rows handed out first
+  __shared__ unsigned long long s_w[kNumLists], s_k[kNumLists];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int32_t r0 = row_begin + blockIdx.x * kRowsPerBlock;
-  if (threadIdx.x < kNumBins) {
+  if (threadIdx.x < kNumLists) {
     s_cnt[threadIdx.x] = 0;
     s_w[threadIdx.x] = 0;
     s_k[threadIdx.x] = 0;
   }
-  if (threadIdx.x < 2) s_hcnt[threadIdx.x] = 0;
-  if (threadIdx.x < 3) s_max[threadIdx.x] = 0;
+  if (threadIdx.x < 3) s_hcnt[threadIdx.x] = 0;
+  if (threadIdx.x < 7) s_max[threadIdx.x] = 0;
   if (threadIdx.x == 0) s_act = 0;
   __syncthreads();
   for (int i = warp; i < kRowsPerBlock; i += kRowsNT / 32) {
@@ -249,7 +250,10 @@ __global__ __launch_bounds__(kRowsNT) void k_rows_work(Side s, int32_t smin, int
         n_e[e - row_begin] = 0;
         stage_pos[e - row_begin] = -1;
         row_work[e - row_begin] = work;
-        if (work) atomicMax(&s_max[0], work);
+        if (work) {
+          atomicMax(&s_max[0], work);
+          atomicMax(&s_max[5], hi - lo);
+        }
         if (active) atomicAdd(&s_act, 1);
       }
     }
@@ -272,35 +276,45 @@ __global__ __launch_bounds__(kRowsNT) void k_rows_work(Side s, int32_t smin, int
     if (my_work > 0 || forced) {
       const int32_t e = r0 + threadIdx.x;
       my_bin = forced ? (int)kBinGiant : bin_of(my_work, bins);
-      // a row with s >= 2 from bins.bloom up to bins.sparse wedges takes the
-      // sparse bin; above the CTA bins only when its far ends are sparse in
-      // its span (f in (e, R))
-      if (!forced && my_work > bins.bloom && my_work <= bins.sparse &&
-          s_of(s.row_s, smin, e) >= 2 &&
-          (my_bin != kBinGiant ||
-           (long long)my_work * bins.dense < (long long)((s.row_fhi ? s.row_fhi[e] : s.R) - 1 - e)))
+      const int32_t size = s.r_off[e + 1] - s.r_off[e];
+      const int32_t se = s_of(s.row_s, smin, e);
+      const int32_t span = (s.row_fhi ? s.row_fhi[e] : s.R) - 1 - e;  // far ends: (e, e + span]
+      // a row whose far ends are dense in its span takes the dense bin; else
+      // one with s >= 2 from bins.bloom up to bins.sparse wedges the sparse bin
+      if ((forced || my_work > kDenseMinWork) && is_dense(my_work, size, span, bins.dense))
+        my_bin = kBinDense;
+      else if (!forced && my_work > bins.bloom && my_work <= bins.sparse && se >= 2)
         my_bin = kBinSparse;
       if (my_bin == kBinGiant) atomicMax(&s_max[1], my_work);
       if (my_bin == kBinSparse) atomicMax(&s_max[2], my_work);
-      huge = (my_bin == kBinGiant && my_work > kGiantHugeWork) ||
+      if (my_bin == kBinDense) {
+        atomicMax(&s_max[size > kDenseBigSize ? 3 : 6], my_work);
+        atomicMax(&s_max[4], size);
+      }
+      huge = (my_bin == kBinDense && size > kDenseBigSize) ||
+             (my_bin == kBinGiant && my_work > kGiantHugeWork) ||
              (my_bin == kBinSparse && my_work > kSparseBigWork);
-      my_slot = huge ? atomicAdd(&s_hcnt[my_bin == kBinSparse], 1) : atomicAdd(&s_cnt[my_bin], 1);
+      my_slot = huge ? atomicAdd(&s_hcnt[my_bin - kBinGiant], 1) : atomicAdd(&s_cnt[my_bin], 1);
       atomicAdd(&s_w[my_bin], (unsigned long long)my_work);
-      atomicAdd(&s_k[my_bin], (unsigned long long)(s.r_off[e + 1] - s.r_off[e]));
+      atomicAdd(&s_k[my_bin], (unsigned long long)size);
     }
   }
   __syncthreads();
-  if (threadIdx.x < kNumBins) {
+  if (threadIdx.x < kNumLists) {
     const int b = threadIdx.x;
-    if (b != kBinGiant && b != kBinSparse) {
+    if (b < kBinGiant) {
       s_base[b] = s_cnt[b] ? (int32_t)atomicAdd(&meta->rows_bin[b], (unsigned long long)s_cnt[b]) : 0;
     } else {
-      // the huge rows of the giant and sparse bins fill their list from the
-      // front, the others from the back (the kernels hand out the huge ones
-      // first); rows_bin counts both
-      const int q = b == kBinSparse;
-      unsigned *rest = q ? &meta->sparse_rest : &meta->giant_rest;
-      unsigned *hge = q ? &meta->sparse_huge : &meta->giant_huge;
+      // the huge rows of the giant, sparse and dense bins fill their list from
+      // the front, the others from the back (the kernels hand out the huge
+      // ones first); rows_bin counts both
+      const int q = b - kBinGiant;
+      unsigned *rest = q == 0   ? &meta->giant_rest
+                       : q == 1 ? &meta->sparse_rest
+                                : &meta->dense_rest;
+      unsigned *hge = q == 0   ? &meta->giant_huge
+                      : q == 1 ? &meta->sparse_huge
+                               : &meta->dense_huge;
       if (s_cnt[b] + s_hcnt[q])
         atomicAdd(&meta->rows_bin[b], (unsigned long long)(s_cnt[b] + s_hcnt[q]));
       s_base[b] = s_cnt[b] ? (int32_t)atomicAdd(rest, (unsigned)s_cnt[b]) : 0;
@@ -312,18 +326,22 @@ __global__ __launch_bounds__(kRowsNT) void k_rows_work(Side s, int32_t smin, int
       atomicAdd(&meta->incid_bin[b], s_k[b]);
     }
   }
-  if (threadIdx.x == kNumBins && s_act) atomicAdd(&meta->active, (unsigned long long)s_act);
+  if (threadIdx.x == kNumLists && s_act) atomicAdd(&meta->active, (unsigned long long)s_act);
   __syncthreads();
   if (threadIdx.x == 0) {
     if (s_max[0]) atomicMax(&meta->max_row_work, s_max[0]);
     if (s_max[1]) atomicMax(&meta->max_giant_work, s_max[1]);
     if (s_max[2]) atomicMax(&meta->max_sparse_work, s_max[2]);
+    if (s_max[3]) atomicMax(&meta->max_dense_work[0], s_max[3]);
+    if (s_max[6]) atomicMax(&meta->max_dense_work[1], s_max[6]);
+    if (s_max[4]) atomicMax(&meta->max_dense_size, s_max[4]);
+    if (s_max[5]) atomicMax(&meta->max_row_size, s_max[5]);
   }
   if (my_bin >= 0) {
     const int64_t len = row_end - row_begin;
     int64_t pos = s_base[my_bin] + my_slot;
-    if (huge) pos = s_hbase[my_bin == kBinSparse] + my_slot;
-    else if (my_bin == kBinGiant || my_bin == kBinSparse) pos = len - 1 - pos;
+    if (huge) pos = s_hbase[my_bin - kBinGiant] + my_slot;
+    else if (my_bin >= kBinGiant) pos = len - 1 - pos;
     bin_rows[(int64_t)my_bin * len + pos] = r0 + threadIdx.x;
   }
 }

@@ -15,7 +15,9 @@ namespace {
 constexpr int kNT = 256;
 constexpr int kRowsPerBlock = 64;
 
-__device__ __forceinline__ int bin_of_full(int32_t work) {
+// (full columns: far ends lie anywhere in [0, R), threshold 1)
+__device__ __forceinline__ int bin_of_full(int32_t work, int32_t size, int32_t R) {
+  if (work > kDenseMinWork && is_dense(work, size, R, kDenseRatio)) return kBinDense;
   if (work <= kWarpMaxWork) return kBinWarp;
   if (work <= kCtaSMaxWork) return kBinCtaS;
   if (work <= kCtaLMaxWork) return kBinCtaL;
@@ -35,10 +37,13 @@ __global__ __launch_bounds__(kNT) void k_rows_full(Side s, int32_t row_begin, in
                                                    int32_t list_stride, Meta *meta) {
   if (meta->err) return;
   __shared__ int32_t s_work[kRowsPerBlock];
-  __shared__ int32_t s_cnt[kNumBins], s_base[kNumBins];
+  __shared__ int32_t s_size;  // most vertices of a row of the block
+  __shared__ int32_t s_cnt[kNumLists], s_base[kNumLists];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int32_t r0 = row_begin + blockIdx.x * kRowsPerBlock;
-  if (threadIdx.x < kNumBins) s_cnt[threadIdx.x] = 0;
+  if (threadIdx.x < kNumLists) s_cnt[threadIdx.x] = 0;
+  if (threadIdx.x == 0) s_size = 0;
+  __syncthreads();
   for (int i = warp; i < kRowsPerBlock; i += kNT / 32) {
     const int32_t e = r0 + i;
     int32_t work = 0;
@@ -56,6 +61,7 @@ __global__ __launch_bounds__(kNT) void k_rows_full(Side s, int32_t row_begin, in
 #pragma unroll
       for (int d = 16; d > 0; d >>= 1) work += __shfl_xor_sync(0xffffffffu, work, d);
       if (lane == 0) {
+        atomicMax(&s_size, hi - lo);
         if (work_out) work_out[e - list_base] = work;
         if (bin_rows) {
           n_e[e - list_base] = 0;
@@ -65,24 +71,32 @@ __global__ __launch_bounds__(kNT) void k_rows_full(Side s, int32_t row_begin, in
     }
     if (lane == 0) s_work[i] = (e < row_end) ? work : 0;
   }
-  if (!bin_rows) return;
   __syncthreads();
+  if (threadIdx.x == 0 && s_size) atomicMax(&meta->max_row_size, s_size);
+  if (!bin_rows) return;
   int my_bin = -1, my_slot = 0;
   if (threadIdx.x < kRowsPerBlock && s_work[threadIdx.x] > 0) {
-    my_bin = bin_of_full(s_work[threadIdx.x]);
-    my_slot = atomicAdd(&s_cnt[my_bin], 1);
-    if (my_bin == kBinGiant) atomicMax(&meta->max_giant_work, s_work[threadIdx.x]);
+    const int32_t e = r0 + (int32_t)threadIdx.x;
+    my_bin = bin_of_full(s_work[threadIdx.x], s.r_off[e + 1] - s.r_off[e], s.R);
+    if (my_bin == kBinDense && s.r_off[e + 1] - s.r_off[e] > kDenseBigSize)
+      my_slot = -1 - (int)atomicAdd(&meta->dense_huge, 1u);
+    else my_slot = atomicAdd(&s_cnt[my_bin], 1);
   }
   __syncthreads();
-  if (threadIdx.x < kNumBins && s_cnt[threadIdx.x])
+  if (threadIdx.x < kNumLists && s_cnt[threadIdx.x])
     s_base[threadIdx.x] =
-        (int32_t)atomicAdd(&meta->rows_bin[threadIdx.x], (unsigned long long)s_cnt[threadIdx.x]);
+        threadIdx.x == kBinDense
+            ? (int32_t)atomicAdd(&meta->dense_rest, (unsigned)s_cnt[threadIdx.x])
+            : (int32_t)atomicAdd(&meta->rows_bin[threadIdx.x],
+                                 (unsigned long long)s_cnt[threadIdx.x]);
   __syncthreads();
   if (my_bin >= 0) {
-    // giant rows fill their list from the back: k_walk_giant hands out the
-    // rows at its front (none here) first, then the back ones
+    // giant and dense rows fill their list from the back (the giant kernel
+    // hands out the rows at its front, none here, first); the dense rows of
+    // the big instance fill it from the front
     int64_t pos = s_base[my_bin] + my_slot;
-    if (my_bin == kBinGiant) pos = list_stride - 1 - pos;
+    if (my_slot < 0) pos = -1 - my_slot;
+    else if (my_bin >= kBinGiant) pos = list_stride - 1 - pos;
     bin_rows[(int64_t)my_bin * list_stride + pos] = r0 + threadIdx.x;
   }
 }

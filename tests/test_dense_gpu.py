@@ -1,0 +1,79 @@
+"""The dense bin (rows counted in windows of packed counters): counter widths
+at their largest value, window edges, every list of tails it keeps."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+import hypergen as hg  # noqa: E402
+import oracle  # noqa: E402
+import paper_2010_11448_gb300 as slg  # noqa: E402
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2010_11448_gb300 import build_lib
+    build_lib.build()
+    slg.load()
+
+
+def hub_rows(k, m, n=700, seed=3):
+    """Row 0 holds vertices 0 .. k-1 and so do the last two rows (weights k:
+    the largest a counter of the row has to hold); the rows between hold 1 to
+    4 random vertices, so that row 0's far ends cover ids up to m."""
+    rng = np.random.default_rng(seed + k)
+    size = rng.integers(1, 5, m - 3)
+    r = np.concatenate([np.zeros(k, np.int64), np.repeat(np.arange(1, m - 2), size),
+                        np.full(k, m - 2), np.full(k, m - 1)])
+    hub = np.arange(k)
+    c = np.concatenate([hub, rng.integers(0, n, int(size.sum())), hub, hub])
+    return hg.from_pairs(r, c, m, n)
+
+
+def as_np(t):
+    return np.stack([x.cpu().numpy() for x in t], 1).astype(np.int64)
+
+
+# 4-, 8- and 16-bit counters at both ends of their range; 600 tails: the list
+# beyond shared memory.  120,000 ids cross a window of every width.
+@pytest.mark.parametrize("k,m", [(15, 120_000), (16, 120_000), (255, 60_000), (256, 120_000),
+                                 (600, 110_000), (15, 3_001)])
+def test_counter_widths_and_windows(k, m):
+    h = hub_rows(k, m)
+    dh = slg.to_device(h)
+    for s in (1, 2, 3, k):
+        want = oracle.canonical(*oracle.line_graph_of(h, s, threads=8))
+        got = as_np(slg.build(dh, s))
+        st = slg.last_stats()
+        if m > 10_000 and s <= 2:  # (fewer far ends are left at larger s)
+            assert st["rows_bin"][3] > 0
+        assert np.array_equal(got, want), s
+        assert (0, m - 1, k) in map(tuple, got[got[:, 0] == 0])
+        i, j, w = slg.build(dh, s, unweighted=True)
+        assert w is None and np.array_equal(
+            np.stack([i.cpu().numpy(), j.cpu().numpy()], 1), want[:, :2])
+        assert slg.count(dh, s) == want.shape[0]
+
+
+def test_long_tails_are_cut():
+    # two tails of 60,000 entries in one window: each is swept as several
+    m = 60_000
+    rng = np.random.default_rng(1)
+    r = np.concatenate([np.arange(m), np.arange(m), np.arange(m)])
+    c = np.concatenate([np.zeros(m, np.int64), np.ones(m, np.int64),
+                        rng.integers(2, 5_000, m)])
+    keep = (r < 3) | (rng.random(r.shape[0]) < 0.6)
+    h = hg.from_pairs(r[keep], c[keep], m, 5_000)
+    rows = np.array([0, 1, 2, 777, 30_000, m - 2], np.int32)
+    mm, n, off, idx = oracle.side(h, False)
+    for s in (1, 2):
+        want = oracle.canonical(*oracle.line_graph(mm, n, off, idx, s, rows=rows, threads=8))
+        ptr = slg.row_offsets(slg.to_device(h), s).cpu().numpy()
+        for e in rows:
+            n_e = int(ptr[e + 1] - ptr[e])
+            i, j, w = slg.build_rows(slg.to_device(h), s, int(e), int(e) + 1,
+                                     capacity=max(n_e, 1))
+            assert np.array_equal(as_np((i, j, w)), want[want[:, 0] == e]), (s, e)
