@@ -24,13 +24,13 @@
 // of 26K ids) take an instance with one CTA of 1,024 threads per SM and a
 // window of 96K ids; the others one with three CTAs of 512 threads.
 //
-// Measured on chung_lu_1m (1M x 2M, s = 2) against the partitioned hash
-// buckets and dense windows of the giant bin that these rows took before
-// (dense rows, 8 ids per wedge; the others hashed): giant bin on H 12.1 ms ->
-// big 5.0, small 1.7, giant 2.4 ms; on H* 47.7 ms -> big 8.7, small 10.7,
-// giant 17.3 ms.  With a scan of the counters instead of the survivor bits
-// (full test of every counter word) the dense rows took 1.5 times as long;
-// with three CTAs of 26K-id windows for every row, 1.5 times on H.
+// Measured on chung_lu_1m (1M x 2M) against the partitioned hash buckets and
+// dense windows of the giant bin that these rows took before: L_8 of H, giant
+// bin 8.8 ms -> big 4.1, small 1.1, giant 1.5 ms; L_2 of H*, 47.7 ms -> big
+// 8.7, small 10.7, giant 17.3 ms.  A scan of the counters in place of the
+// survivor bits cost 26 instead of 13 x 10^9 CTA cycles on L_2(H*) (rows down
+// to one wedge per 32 ids); windows of 26K ids for every row took 13.9
+// instead of 9.2 ms on L_2(H).
 #include <algorithm>
 #include <mutex>
 

@@ -54,8 +54,8 @@ constexpr int32_t kGiantHugeWork = SLG_GIANT_HUGE_WORK;
 #endif
 constexpr int32_t kSparseBigWork = SLG_SP_BIG_WORK > 0 ? SLG_SP_BIG_WORK : kGiantHugeWork;
 // A row is dense when it has at least one wedge per this many ids of its far
-// ends' span, for 16-bit counters (see is_dense).  Step of four builds on
-// chung_lu_1m: 137.2, 134.8, 137.1, 180 ms with 8, 16, 24, 48.
+// ends' span, for 16-bit counters (see is_dense).  L_8(H), L_2(H*) and L_8(H*)
+// of chung_lu_1m together: 119.0, 121.5, 163.6 ms with 16, 24, 48.
 #ifndef SLG_DENSE_RATIO
 #define SLG_DENSE_RATIO 16
 #endif
