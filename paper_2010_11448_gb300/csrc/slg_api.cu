@@ -323,24 +323,25 @@ cudaError_t ensure_scratch(Call &c, size_t *summ_off) {
   return ensure_giant(*c.ctx, counters + pw * (rp >> 10), c.st);
 }
 
-// Scratch of the giant and dense bins (their kernels run one after the other
-// and share it): 4 ints per wedge of the largest giant row and giant CTA;
+// Scratch of the sparse, giant and dense bins (their kernels run one after the
+// other and share it): 4 ints per wedge of the largest giant row and giant CTA;
 // the dense bin's per-CTA need for its largest row.  Sets L's dense_pairs,
 // dense_size and giant_stride and returns the ints.
-size_t scratch_ints(WalkLaunch *L, int32_t max_giant, long long pairs_big, long long pairs_small,
-                    int32_t dense_size) {
+size_t scratch_ints(WalkLaunch *L, int32_t max_giant, int32_t max_sparse, long long pairs_big,
+                    long long pairs_small, int32_t dense_size) {
   L->giant_stride = 4ll * max_giant;
   L->dense_pairs[0] = pairs_big;
   L->dense_pairs[1] = pairs_small;
   L->dense_size = dense_size;
-  return std::max((size_t)giant_ctas() * (size_t)L->giant_stride,
+  const size_t sp = max_sparse > 0 ? (size_t)sparse_ints(max_sparse) : 0;
+  return std::max(std::max((size_t)giant_ctas() * (size_t)L->giant_stride, sp),
                   (size_t)dense_ints(pairs_big, pairs_small, dense_size));
 }
 
-cudaError_t giant_scratch(Call &c, int32_t max_giant, long long pairs_big, long long pairs_small,
-                          int32_t dense_size, WalkLaunch *L) {
+cudaError_t giant_scratch(Call &c, int32_t max_giant, int32_t max_sparse, long long pairs_big,
+                          long long pairs_small, int32_t dense_size, WalkLaunch *L) {
   L->giant_scratch = nullptr;
-  const size_t n = scratch_ints(L, max_giant, pairs_big, pairs_small, dense_size);
+  const size_t n = scratch_ints(L, max_giant, max_sparse, pairs_big, pairs_small, dense_size);
   L->scratch_ints = (long long)n;
   return n ? c.pool->get(&L->giant_scratch, n) : cudaSuccess;
 }
@@ -524,7 +525,8 @@ int run_binned(Call &c, int64_t *result) {
     const long long p = work / c.smin + (core.T ? core.n_core : 0);
     return std::max(std::min<long long>(p, c.sd.R), 1ll);
   };
-  SLG_TRY(giant_scratch(c, max_giant, dense_pairs(mp.dense_huge, mp.max_dense_work[0]),
+  SLG_TRY(giant_scratch(c, max_giant, mp.max_sparse_work,
+                        dense_pairs(mp.dense_huge, mp.max_dense_work[0]),
                         dense_pairs(mp.dense_rest, mp.max_dense_work[1]), mp.max_dense_size,
                         &L));
   L.w.r_off = c.sd.r_off;
@@ -672,7 +674,7 @@ int run_spgemm(Call &c, int64_t *result) {
   w.stage_cap = budget;
   WalkLaunch Lg = walk_launch(c, kStage, 1, c.row_begin);
   Lg.a.full_rows = 1;
-  SLG_TRY(giant_scratch(c, max_row > kCtaLMaxWork ? (int32_t)max_row : 0,
+  SLG_TRY(giant_scratch(c, max_row > kCtaLMaxWork ? (int32_t)max_row : 0, 0,
                         max_row > kDenseMinWork ? std::min<long long>(max_row, c.sd.R) : 0,
                         max_row > kDenseMinWork ? std::min<long long>(max_row, c.sd.R) : 0,
                         c.meta_host->max_row_size, &Lg));
@@ -1726,7 +1728,7 @@ extern "C" int slg_plan_create(const slg_hypergraph *hs, const int32_t *s, int32
   SLG_TRY(p->mem.get(&p->out_w, (size_t)std::max<int64_t>(pairs, 1)));
   SLG_TRY(p->mem.get(&p->offsets, (size_t)count + 1));
   if (max_work > 0) {
-    const size_t n = scratch_ints(&p->scratch, max_work, std::min<long long>(max_work, R),
+    const size_t n = scratch_ints(&p->scratch, max_work, max_work, std::min<long long>(max_work, R),
                                   std::min<long long>(max_work, R), max_size);
     p->scratch.scratch_ints = (long long)n;
     SLG_TRY(p->mem.get(&p->giant, n));
@@ -1738,12 +1740,12 @@ extern "C" int slg_plan_create(const slg_hypergraph *hs, const int32_t *s, int32
                         Bins{64, 1024, 4096},
                         Bins{128, 512, 4096},
                         Bins{128, 1024, 2048},
-                        Bins{128, 1024, 4096, 8192},
+                        Bins{128, 1024, 4096, 16384},
                         Bins{128, 1024, 4096, 0},
-                        Bins{128, 1024, 2048, 16384, 2048},
-                        Bins{128, 1024, 4096, 16384, 1024, kDenseRatio / 2},
-                        Bins{128, 1024, 4096, 16384, 1024, kDenseRatio * 2},
-                        Bins{128, 1024, 4096, 16384, 4096}};
+                        Bins{128, 1024, 2048, 65536, 2048},
+                        Bins{128, 1024, 4096, 65536, 1024, kDenseRatio / 2},
+                        Bins{128, 1024, 4096, 65536, 1024, kDenseRatio * 2},
+                        Bins{128, 1024, 4096, 65536, 4096}};
   cudaEvent_t t0, t1;
   SLG_TRY(cudaEventCreate(&t0));
   SLG_TRY(cudaEventCreate(&t1));

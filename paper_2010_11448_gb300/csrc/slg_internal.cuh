@@ -45,14 +45,17 @@ constexpr int32_t kCtaLMaxWork = 4096;
 #define SLG_GIANT_HUGE_WORK 32768
 #endif
 constexpr int32_t kGiantHugeWork = SLG_GIANT_HUGE_WORK;
-// Sparse rows above this work are handed out first, to the sparse kernel
-// with the larger candidate table; the others go to the one with the smaller
-// table and one more CTA per SM (0: a single sparse kernel, and no sparse
-// row is handed out first).
+// Sparse rows above this work take the instance of the sparse kernel with
+// the larger table.
 #ifndef SLG_SP_BIG_WORK
 #define SLG_SP_BIG_WORK 8192
 #endif
-constexpr int32_t kSparseBigWork = SLG_SP_BIG_WORK > 0 ? SLG_SP_BIG_WORK : kGiantHugeWork;
+constexpr int32_t kSparseBigWork = SLG_SP_BIG_WORK;
+// Largest row of the sparse bin (Bins::sparse is at most this).
+#ifndef SLG_SPARSE_MAX_WORK
+#define SLG_SPARSE_MAX_WORK 65536
+#endif
+constexpr int32_t kSparseMaxWork = SLG_SPARSE_MAX_WORK;
 // A row is dense when it has at least one wedge per this many ids of its far
 // ends' span, for 16-bit counters (see is_dense).  L_8(H), L_2(H*) and L_8(H*)
 // of chung_lu_1m together: 119.0, 121.5, 163.6 ms with 16, 24, 48.
@@ -98,7 +101,7 @@ struct Meta {
   unsigned int giant_huge;             // giant rows above kGiantHugeWork (front of the list)
   unsigned int giant_rest;             // the other giant rows (back of the list)
   unsigned int sparse_ticket;          // the same three for the sparse bin
-  unsigned int sparse_ticket_rest;     // the small-table sparse kernel's own tickets
+  unsigned int sparse_ticket_rest;
   unsigned int sparse_huge;
   unsigned int sparse_rest;
   unsigned int dense_ticket;           // the same four for the dense bin (huge: kDenseBigSize)
@@ -384,9 +387,6 @@ __device__ __forceinline__ int32_t s_of(const int32_t *row_s, int32_t smin, int3
 // and the giant bin's partition serves them better); 0 turns the bin off.
 // `bloom`: rows with s >= 2 above this work (and at most `sparse`) take the
 // sparse bin also when they are dense or fit a CTA bin.
-#ifndef SLG_SPARSE_MAX_WORK
-#define SLG_SPARSE_MAX_WORK 16384
-#endif
 #ifndef SLG_BLOOM_MIN_WORK
 #define SLG_BLOOM_MIN_WORK 1024
 #endif
@@ -394,7 +394,7 @@ __device__ __forceinline__ int32_t s_of(const int32_t *row_s, int32_t smin, int3
 // span is dense, for 16-bit counters (see is_dense).
 struct Bins {
   int32_t warp = kWarpMaxWork, ctas = kCtaSMaxWork, ctal = kCtaLMaxWork;
-  int32_t sparse = SLG_SPARSE_MAX_WORK;
+  int32_t sparse = kSparseMaxWork;
   int32_t bloom = SLG_BLOOM_MIN_WORK;
   int32_t dense = kDenseRatio;
 };
@@ -505,10 +505,10 @@ struct WalkLaunch {
   int32_t dense_size;       // most vertices of a dense-bin row
 };
 
-// CTAs of the giant kernel (two per SM) and of the sparse kernel, and the
-// scratch ints of the dense kernels.
+// CTAs of the giant kernel (two per SM); scratch ints of the sparse and dense
+// kernels.
 int giant_ctas();
-int sparse_ctas();
+long long sparse_ints(int32_t max_work);
 long long dense_ints(long long pairs_big, long long pairs_small, int32_t size_big);
 // The largest side (rows) a build supports: row ids and the giant bin's
 // super-chunk bounds stay below 2^31.

@@ -1,34 +1,40 @@
-// The sparse bin of the s-overlap walk.
+// The sparse bin of the s-overlap walk: rows with s >= 2 whose far ends are
+// sparse in their id span.
 //
-// Large rows whose far ends are sparse in their id span, with s >= 2.  Almost
-// every far end of such a row occurs once (on the Chung-Lu workloads about
-// 96 % of the wedges of these rows are the only wedge to their far end), and
-// a far end with a single wedge can never reach s >= 2.  The row is counted
-// in two passes with little shared memory, so that several rows are in
-// flight on each SM (the walk's far-end gathers are latency-bound: a row at
-// a time per SM leaves the memory system idle):
-//   1. every wedge sets its far end's bit in a one-hash Bloom filter (one
-//      shared atomicOr); a wedge that finds the bit already set makes f a
-//      candidate: f is claimed in a small shared table (key, count 0) and
-//      marked in a second filter.  Every f with two or more wedges becomes
-//      a candidate (its second wedge finds the bit set); so may a few
-//      single-wedge f whose bit another f had set;
-//   2. a second pass counts, exactly, every wedge whose far end is a
-//      candidate (the second filter screens out almost all others before
-//      the table is probed).  The count of f is then |e ∩ f|.  It reads the
-//      row's far ends from a copy the first walk wrote to global scratch
-//      (or, for a row of at most kSpCache wedges, to shared memory), or
-//      walks the tails again when there is no room for the copy.
-// The candidates with count >= s are sorted and emitted.  A row whose
-// candidates overflow the table (a probe sequence longer than kSpMaxProbe)
-// is handed to the giant bin, which runs after this one.
-// Two instances of the kernel share the bin: rows above kSparseBigWork go
-// to one with a 2^SLG_SP_LGT-slot table, the rest to one with a
-// 2^SLG_SP_SMALL_LGT-slot table, whose smaller shared memory leaves room for
-// one more resident CTA per SM.  Rows of up to 8192 wedges seldom have more
-// candidates or survivors than the smaller table holds (the overflow would
-// send them to the giant bin); rows of up to 16384 do.
-
+// Almost every far end of such a row occurs once (on the Chung-Lu workloads
+// about 96 % of the wedges are the only wedge to their far end), and a far
+// end with a single wedge can never reach s >= 2.  Moreover a far end f with
+// |e ∩ f| >= s meets e outside any s - 1 of e's vertices: with the row's t <=
+// s - 1 longest tails set aside, f still has s - t wedges in the others.  The
+// tails are very unequal (on L_8 of the dual of chung_lu_1m the six longest
+// hold nine tenths of such a row's wedges), so most wedges are only looked
+// up, never inserted anywhere:
+//   1. every wedge of the inserted tails sets its far end's bit in a Bloom
+//      filter `once` (one shared atomicOr); a wedge that finds the bit set
+//      also sets it in a second filter `twice`;
+//   2. s <= 3, one tail set aside: a far end of that tail whose bit is set
+//      in `once` is marked in `twice` and counted in a small shared table
+//      (a tail holds each far end at most once);
+//   3. the inserted tails are read again; a far end whose bit is set in
+//      `twice` is counted in the table.  s > 3, s - 2 tails set aside: theirs
+//      are read too.  Every f with |e ∩ f| >= s passes in each of its wedges
+//      (it has s - t >= 2 inserted wedges, or, s <= 3, one and one in the
+//      tail set aside), so its count is exact;
+//   4. the far ends whose count reached s, listed as they did, are ranked
+//      and written.
+// A warp takes a segment of a tail at a time (consecutive far ends: no
+// search for a wedge's tail); the few far ends that pass a filter are queued
+// and counted by whole warps.
+//
+// Rows above kSpChunk (s > 3: kSpChunkAside) wedges are processed in several ranges of ids, so that
+// a range's far ends fit the filter and the table.  A range that overflows
+// the table (a probe sequence longer than kSpMaxProbe) is repeated with the
+// largest one; one that overflows that, or has more survivors than can be
+// ordered, with half the ids (a row that still fails with 64 ids would be
+// handed to the giant bin, which runs after this one).
+//
+// Bound by instruction issue (70 % of issue slots) and the latency of the
+// dependent steps of a row, with five rows in flight per SM.
 #include <algorithm>
 #include <mutex>
 
@@ -38,198 +44,210 @@ namespace slg {
 
 namespace {
 
+#ifndef SLG_SP_LOGB
+#define SLG_SP_LOGB 16
+#endif
 #ifndef SLG_SP_NT
 #define SLG_SP_NT 256
 #endif
-#ifndef SLG_SP_LOGB
-#define SLG_SP_LOGB 17
+#ifndef SLG_SP_MINB
+#define SLG_SP_MINB 5
 #endif
 #ifndef SLG_SP_LGT
-#define SLG_SP_LGT 12
+#define SLG_SP_LGT 11
 #endif
-#ifndef SLG_SP_CACHE
-#define SLG_SP_CACHE 0
+#ifndef SLG_SP_BIG_NT
+#define SLG_SP_BIG_NT 512
 #endif
-#ifndef SLG_SP_MINB
-#define SLG_SP_MINB 4
-#endif
-#ifndef SLG_SP_SMALL_LGT
-#define SLG_SP_SMALL_LGT 11
-#endif
-#ifndef SLG_SP_SMALL_MINB
-#define SLG_SP_SMALL_MINB 5
+#ifndef SLG_SP_BIG_MINB
+#define SLG_SP_BIG_MINB 3
 #endif
 #ifndef SLG_SP_G
-#define SLG_SP_G 6
+#define SLG_SP_G 4
 #endif
-#ifndef SLG_SP_RUNS
-#define SLG_SP_RUNS 1  // order survivor sets above 64 by sorted warp runs
+#ifndef SLG_SP_CHUNK
+#define SLG_SP_CHUNK 12288
 #endif
-constexpr int kSpNT = SLG_SP_NT;
-constexpr int kSpLogB = SLG_SP_LOGB;          // Bloom filter bits (log2)
+#ifndef SLG_SP_CHUNK_ASIDE
+#define SLG_SP_CHUNK_ASIDE 32768
+#endif
+#ifndef SLG_SP_DROP
+#define SLG_SP_DROP 16
+#endif
+constexpr int kSpLogB = SLG_SP_LOGB;          // bits of each filter (log2)
 constexpr int kSpWords = 1 << (kSpLogB - 5);
-constexpr int kSpCWords = kSpWords / 4;       // candidate filter words
-constexpr int kSpLgT = SLG_SP_LGT;            // candidate table slots (log2)
-constexpr int kSpSmallLgT = SLG_SP_SMALL_LGT;  // the same, rows up to kSparseBigWork
-constexpr int kSpCache = SLG_SP_CACHE;        // far ends kept of a small row
 constexpr int kSpMaxProbe = 32;
-constexpr int kSpG = SLG_SP_G;                // wedges per thread per walk step
-static_assert((1 << kSpSmallLgT) >= kSpNT && kSpSmallLgT <= kSpLgT &&
-                  kSpWords % (4 * kSpNT) == 0 && kSpCWords % 4 == 0,
-              "sparse bin geometry");
+constexpr int kSpG = SLG_SP_G;                // wedges per thread per step
+constexpr int kSpSeg = 32 * kSpG;             // far ends per segment of a tail
+constexpr int32_t kSpChunk = SLG_SP_CHUNK;    // a row's wedges per id range, about
+constexpr int32_t kSpChunkAside = SLG_SP_CHUNK_ASIDE;  // s > 3 (most wedges are set aside)
+constexpr int kSpDrop = SLG_SP_DROP;          // tails set aside, at most
+constexpr int kSpQ = 32 + kSpSeg;             // queued far ends per warp
+constexpr int kSpList = kSpWords;             // listed survivors, at most (in `once`)
+constexpr int kSpSortMax = kSpWords / 2 - 32;  // of which ordered in `twice`
+constexpr int kSpRegQ = 4;                    // more: ordered in the table, 4 per thread
 
-// [s_base 8][s_ovf 4][s_row 4][pad 16][filter kSpWords x 4]
-// [candidate filter kSpCWords x 4][table 2^lgt x 8][cache kSpCache x 4]
-// [s_beg NT][s_pref NT+1][ws NT/32+1]
-constexpr size_t sparse_smem(int lgt) {
-  return 32 + (size_t)kSpWords * 4 + (size_t)kSpCWords * 4 + ((size_t)8 << lgt) +
-         (size_t)kSpCache * 4 + (size_t)(2 * kSpNT + 1 + kSpNT / 32 + 1) * 4;
+// The two instances of the kernel: NT threads, tables of up to 2^LGT slots,
+// MINB CTAs per SM, tails of up to MAXW wedges in all.
+struct SpSmall {  // rows of at most kSparseBigWork wedges
+  static constexpr int NT = SLG_SP_NT, LGT = SLG_SP_LGT, MINB = SLG_SP_MINB;
+  static constexpr int32_t MAXW = kSparseBigWork;
+};
+struct SpBig {
+  static constexpr int NT = SLG_SP_BIG_NT, LGT = 12, MINB = SLG_SP_BIG_MINB;
+  static constexpr int32_t MAXW = kSparseMaxWork;
+};
+template <class C>
+constexpr int sp_max_seg() {  // segments of a batch of NT tails
+  return C::MAXW / kSpSeg + C::NT;
 }
 
-// A row's filter has 2^lgb bits (its candidate filter 2^(lgb - 2)) and its
-// table 2^lgt slots, sized by the row's work (see sp_sizes).
-__device__ __forceinline__ uint32_t sp_h1(int32_t f, int lgb) {  // Bloom filter bit
+// [s_base 8][s_ovf 4][s_row 4][s_any 4][s_sum 4][s_nsurv 4][pad 4][s_cyc 6 x 8][once][twice]
+// [table x 8][segments x 8][lengths NT][ws NT/32+1][queues]
+template <class C>
+constexpr size_t sparse_smem() {
+  static_assert(kSpWords % (4 * C::NT) == 0 && sp_max_seg<C>() < 65536 &&
+                    kSpList <= 2 * (1 << C::LGT) && 2 * C::NT * kSpRegQ <= (1 << C::LGT),
+                "sparse bin geometry");
+  return 80 + (size_t)kSpWords * 8 + (size_t)((1 << C::LGT) + 32) * 8 +
+         (size_t)sp_max_seg<C>() * 8 +
+         (size_t)(C::NT + C::NT / 32 + 1 + C::NT / 32 * kSpQ) * 4;
+}
+
+__device__ __forceinline__ uint32_t sp_bit(int32_t f, int lgb) {  // filter bit
   return ((uint32_t)f * 0x9E3779B1u) >> (32 - lgb);
 }
-__device__ __forceinline__ uint32_t sp_h2(int32_t f, int lgb) {  // candidate filter bit
-  return ((uint32_t)f * 0x85EBCA6Bu) >> (34 - lgb);
-}
-__device__ __forceinline__ uint32_t sp_ht(int32_t f, int lgt) {  // candidate table slot
-  return ((uint32_t)f * 0xC2B2AE35u) >> (32 - lgt);
-}
 
-// Per-row sizes: a filter of >= 32 bits per wedge (so that a single-wedge
-// far end finds its bit set by another with probability below 1/64 on
-// average) and a table of >= one slot per wedge (every candidate has two
-// wedges or is such a collision), within the shared-memory maxima (a table
-// of at most 2^max_lgt slots).
-__device__ __forceinline__ void sp_sizes(int32_t work, int max_lgt, int *lgb, int *lgt) {
-  const int lw = ceil_log2(work > 1 ? work : 2);
-  *lgb = min(max(lw + 5, 12), kSpLogB);
-  *lgt = min(max(lw, 7), max_lgt);
-}
-
-// Pass 1: f is a candidate (its filter bit was already set).  Claims f's
-// table slot (32-bit CAS on the key word; the count word stays 0) unless it
-// is there already, and marks it in the candidate filter.  A probe sequence
-// longer than kSpMaxProbe marks the row as overflowed.
-__device__ __forceinline__ void sp_candidate(unsigned long long *tab, uint32_t *cand, int32_t f,
-                                             int32_t *s_ovf, int lgb, int lgt) {
-  if (*(volatile int32_t *)s_ovf) return;
+// One wedge to f, counted in the table: the key word is claimed with a 32-bit
+// CAS and the claim stands for one wedge (the count word holds count - 1).  A
+// far end whose count reaches s (>= 2) appends its slot to the survivors.
+// Unweighted: a count that reached s is not raised further.  A probe sequence
+// longer than kSpMaxProbe marks the range as overflowed.
+__device__ __forceinline__ void sp_insert(unsigned long long *tab, int32_t f, int32_t smin,
+                                          bool unweighted, int lgt, int32_t *s_ovf,
+                                          int32_t *list, int32_t *s_nsurv) {
   const uint32_t mask = (1u << lgt) - 1u;
-  uint32_t h = sp_ht(f, lgt);
+  uint32_t h = ((uint32_t)f * 0xC2B2AE35u) >> (32 - lgt);
   for (int probe = 0; probe < kSpMaxProbe; ++probe) {
-    const uint32_t k = atomicCAS(count_word(tab, h) + 1, 0xFFFFFFFFu, (uint32_t)f);
-    if (k == 0xFFFFFFFFu) {
-      const uint32_t c = sp_h2(f, lgb);
-      atomicOr(cand + (c >> 5), 1u << (c & 31));
+    uint32_t *cw = count_word(tab, h);
+    const uint32_t k = atomicCAS(cw + 1, 0xFFFFFFFFu, (uint32_t)f);
+    if (k == 0xFFFFFFFFu) return;
+    if (k == (uint32_t)f) {
+      if (unweighted && (int32_t)*(volatile uint32_t *)cw + 1 >= smin) return;
+      if ((int32_t)atomicAdd(cw, 1u) == smin - 2) {
+        const int32_t p = atomicAdd(s_nsurv, 1);
+        if (p < kSpList) list[p] = (int32_t)h;
+      }
       return;
     }
-    if (k == (uint32_t)f) return;
     h = (h + 1) & mask;
   }
   *(volatile int32_t *)s_ovf = 1;
 }
 
-// Pass 2, for an f that passed the candidate filter: counted if it is in
-// the table.  Unweighted: a count that reached s is not raised further.
-__device__ __forceinline__ void sp_count_listed(unsigned long long *tab, int32_t f, int32_t smin,
-                                                bool unweighted, int lgt) {
-  const uint32_t mask = (1u << lgt) - 1u;
-  uint32_t h = sp_ht(f, lgt);
-  for (int probe = 0; probe < kSpMaxProbe; ++probe) {
-    uint32_t *cw = count_word(tab, h);
-    const uint32_t k = cw[1];
-    if (k == (uint32_t)f) {
-      if (!unweighted || (int32_t)*(volatile uint32_t *)cw < smin) atomicAdd(cw, 1u);
-      return;
-    }
-    if (k == 0xFFFFFFFFu) return;
-    h = (h + 1) & mask;
+// A warp's queue of far ends to count (a few per hundred wedges).  They are
+// gathered in shared memory and handled 32 at a time, so that the counting
+// runs with whole warps; its code is there once per pass (the unrolled steps
+// only append), which keeps the passes within the instruction cache.
+struct SpQueue {
+  int32_t *q;  // kSpQ entries of this warp
+  int n;       // queued (warp-uniform), below 32 between steps
+  __device__ __forceinline__ void push(bool c, int32_t f) {
+    const unsigned bal = __ballot_sync(0xffffffffu, c);
+    if (c) q[n + __popc(bal & ((1u << (threadIdx.x & 31)) - 1u))] = f;
+    n += __popc(bal);
   }
+  // fn(f) for whole warps of queued far ends; with `all`, for every one
+  template <class Fn>
+  __device__ __forceinline__ void drain(bool all, Fn &&fn) {
+    if (n < (all ? 1 : 32)) return;
+    __syncwarp();
+    const int lane = threadIdx.x & 31;
+    do {
+      const int take = min(n, 32);
+      n -= take;
+      if (lane < take) fn(q[n + lane]);
+    } while (n >= (all ? 1 : 32));
+    __syncwarp();
+  }
+};
+
+// First position in the ascending a[lo, hi) with a value >= x.
+__device__ __forceinline__ int32_t lower_pos(const int32_t *__restrict__ a, int32_t lo, int32_t hi,
+                                             int32_t x) {
+  while (lo < hi) {
+    const int32_t mid = lo + ((hi - lo) >> 1);
+    if (__ldg(a + mid) < x) lo = mid + 1;
+    else hi = mid;
+  }
+  return lo;
 }
 
-// Pass 2: one wedge to f; counted when f is a candidate.
-__device__ __forceinline__ void sp_count(unsigned long long *tab, const uint32_t *cand,
-                                         int32_t f, int32_t smin, bool unweighted, int lgb,
-                                         int lgt) {
-  const uint32_t c = sp_h2(f, lgb);
-  if (!(cand[c >> 5] & (1u << (c & 31)))) return;
-  sp_count_listed(tab, f, smin, unweighted, lgt);
-}
-
-// A lane's few wedges of a walk step that take the slow path (candidate
-// claims in pass 1, counts in pass 2: a small fraction of the wedges) are
-// gathered in registers and handled in rounds, the q-th round taking every
-// lane's q-th one, so that a warp runs max over its lanes rounds instead of
-// one round per wedge slot of the step with a lane or two active.
-#ifndef SLG_SP_DEFER
-#define SLG_SP_DEFER 1
-#endif
-template <int G>
-__device__ __forceinline__ void pend_push(int32_t (&pend)[G], int &np, bool c, int32_t f, int g) {
-#pragma unroll
-  for (int q = 0; q < G; ++q)  // selects: no local memory
-    if (q <= g) pend[q] = (c && q == np) ? f : pend[q];
-  np += c;
-}
-
-// The first walk also copies the row's far ends (in flattened wedge order) to
-// the CTA's part of the giant bin's scratch (free while this kernel runs:
-// the giant bin runs after it), so that the second pass reads them in order
-// instead of walking the tails again.  buf_stride: ints per CTA (0: none).
-#ifndef SLG_SP_GBUF
-#define SLG_SP_GBUF 1
-#endif
-// part: 0 every row of the bin, 1 the rows handed out first (the front of
-// the list), 2 the others (the back of the list, on their own ticket).
-template <int LGT, int MINB>
-__global__ __launch_bounds__(kSpNT, MINB) void k_walk_sparse(
+// part 0: the rows above kSparseBigWork wedges (the front of the list), 1: the
+// others (its back), each on its own ticket.  buf: the CTA's share of the
+// giant bin's scratch (free while this kernel runs), for the pairs of rows of
+// several ranges: buf_stride ints, at least the largest row's work.
+template <class C>
+__global__ __launch_bounds__(C::NT, C::MINB) void k_walk_sparse(
     Walk w, const int32_t *__restrict__ rows, EmitArgs a, int32_t *__restrict__ giant_rows,
-    int32_t list_len, int32_t *__restrict__ buf, long long buf_stride, int part) {
-  constexpr int kT = 1 << LGT;        // candidate table slots
-  constexpr int kSPT = kT / kSpNT;    // table slots per thread
+    int32_t list_len, int32_t *__restrict__ buf, long long buf_stride, int32_t R, int part) {
+  constexpr int NT = C::NT, NW = NT / 32, kSpT = 1 << C::LGT;
   Meta *meta = a.meta;
   if (meta->err) return;
   extern __shared__ __align__(16) unsigned char smem[];
   long long *s_base = reinterpret_cast<long long *>(smem);
   int32_t *s_ovf = reinterpret_cast<int32_t *>(smem + 8);
   int32_t *s_row = reinterpret_cast<int32_t *>(smem + 12);
-  uint32_t *filt = reinterpret_cast<uint32_t *>(smem + 32);
-  uint32_t *cand = filt + kSpWords;
-  unsigned long long *tab = reinterpret_cast<unsigned long long *>(cand + kSpCWords);
-  int32_t *cache = reinterpret_cast<int32_t *>(tab + kT);
-  int32_t *s_beg = cache + kSpCache;
-  int32_t *s_pref = s_beg + kSpNT;
-  int32_t *ws = s_pref + kSpNT + 1;
-  const int32_t tid = (int32_t)threadIdx.x;
-  // clears the first 2^(lgb - 5) filter words and 2^(lgb - 7) candidate
-  // filter words (>= 128 and 32: whole uint4 groups)
-  auto clear_filters = [&](int lgb) {
-    uint4 *f4 = reinterpret_cast<uint4 *>(filt);
-    for (int i = tid; i < (1 << (lgb - 7)); i += kSpNT) f4[i] = make_uint4(0, 0, 0, 0);
-    uint4 *c4 = reinterpret_cast<uint4 *>(cand);
-    for (int i = tid; i < (1 << (lgb - 9)); i += kSpNT) c4[i] = make_uint4(0, 0, 0, 0);
+  int32_t *s_any = reinterpret_cast<int32_t *>(smem + 16);
+  int32_t *s_sum = reinterpret_cast<int32_t *>(smem + 20);
+  int32_t *s_nsurv = reinterpret_cast<int32_t *>(smem + 24);
+  // SM cycles of the CTA's first thread: row set-up, first pass, second
+  // pass, order and write, clear; the last lap's time
+  long long *s_cyc = reinterpret_cast<long long *>(smem + 32);
+  uint32_t *once = reinterpret_cast<uint32_t *>(smem + 80);
+  uint32_t *twice = once + kSpWords;
+  unsigned long long *tab = reinterpret_cast<unsigned long long *>(twice + kSpWords);
+  int2 *s_seg = reinterpret_cast<int2 *>(tab + kSpT + 32);  // (first far end, how many)
+  int32_t *s_len = reinterpret_cast<int32_t *>(s_seg + sp_max_seg<C>());
+  int32_t *ws = s_len + NT;
+  const int32_t tid = (int32_t)threadIdx.x, lane = tid & 31, wq = tid >> 5;
+  SpQueue q = {ws + NW + 1 + wq * kSpQ, 0};
+  // the survivors' slots, in `once` (not read any more when they are listed),
+  // and their keys, in `twice` (the same)
+  int32_t *list = reinterpret_cast<int32_t *>(once);
+  unsigned long long *keys = reinterpret_cast<unsigned long long *>(twice);
+  auto zero = [&](uint32_t *p, int n) {  // words, rounded up to four
+    uint4 *p4 = reinterpret_cast<uint4 *>(p);
+    for (int i = tid; i < (n + 3) >> 2; i += NT) p4[i] = make_uint4(0, 0, 0, 0);
   };
-  clear_filters(kSpLogB);
-  for (int i = tid; i < kT; i += kSpNT) tab[i] = kEmpty64;
-  const unsigned nrows = (unsigned)meta->rows_bin[kBinSparse];
-  const unsigned nhuge = meta->sparse_huge;
-  unsigned *ticket = part == 2 ? &meta->sparse_ticket_rest : &meta->sparse_ticket;
-  const unsigned t_first = part == 2 ? nhuge : 0u;
-  const unsigned t_end = part == 1 ? nhuge : nrows;
+  zero(once, 2 * kSpWords);
+  clear_slots<NT>(tab, kSpT + 32);
+  const unsigned nrows = part ? meta->sparse_rest : meta->sparse_huge;
+  unsigned *ticket = part ? &meta->sparse_ticket_rest : &meta->sparse_ticket;
   const bool unweighted = a.unweighted != 0;
   const bool emit = a.mode != kCount;
-  // SM cycles of the CTA's first thread: row set-up, first walk, second
-  // walk, collect and order, emit and clear
-  long long cyc[5] = {0, 0, 0, 0, 0};
-  for (;;) {
-    long long t0 = clock64();
-    __syncthreads();  // the previous row's clears done
+  // pairs of a row of several ranges: at most work / 2 (s >= 2)
+  int32_t *pj = buf + (long long)blockIdx.x * buf_stride, *pw = pj + buf_stride / 2;
+  if (tid == 0) {
+    for (int i = 0; i < 5; ++i) s_cyc[i] = 0;
+    s_cyc[5] = clock64();
+  }
+  auto lap = [&](int i) {
     if (tid == 0) {
-      const unsigned t = t_first + atomicAdd(ticket, 1u);
+      const long long t1 = clock64();
+      s_cyc[i] += t1 - s_cyc[5];
+      s_cyc[5] = t1;
+    }
+  };
+  for (;;) {
+    __syncthreads();  // the previous row is done
+    if (tid == 0) {
+      const unsigned t = atomicAdd(ticket, 1u);
+      *s_row = t >= nrows ? -1 : rows[part ? list_len - 1 - t : t];
       *s_ovf = 0;
-      *s_row = t >= t_end ? -1 : rows[t < nhuge ? t : list_len - 1 - (t - nhuge)];
+      *s_any = 0;
+      *s_sum = 0;
+      *s_nsurv = 0;
     }
     __syncthreads();
     const int32_t e = *s_row;
@@ -237,179 +255,276 @@ __global__ __launch_bounds__(kSpNT, MINB) void k_walk_sparse(
     const int32_t smin = s_of(a.row_s, a.smin, e);
     const int32_t work = a.row_work[e - a.row_begin];
     const int32_t k0 = w.r_off[e], k1 = w.r_off[e + 1];
-    const bool cached = work <= kSpCache;
-    // the far ends kept in global scratch for the second pass (uniform)
-    int32_t *gbuf = (SLG_SP_GBUF && !cached && (long long)work <= buf_stride)
-                        ? buf + (long long)blockIdx.x * buf_stride
-                        : nullptr;
-    int lgb, lgt;
-    sp_sizes(work, LGT, &lgb, &lgt);
-    const int32_t T = 1 << lgt;
-    {
-      const long long t1 = clock64();
-      cyc[0] += t1 - t0;
-      t0 = t1;
-    }
-    // 1. filter; candidates (a thread's G filter updates are in flight together)
-    cta_walk_batched<kSpNT, kSpG>(
-        w, k0, k1, s_beg, s_pref, ws, [&](const int32_t(&f)[kSpG], int32_t i0) {
-          uint32_t old[kSpG], m[kSpG];
-#pragma unroll
-          for (int g = 0; g < kSpG; ++g) {
-            if (cached && f[g] >= 0) cache[i0 + 32 * g] = f[g];
-            if (gbuf && f[g] >= 0) gbuf[i0 + 32 * g] = f[g];
-            const uint32_t h = sp_h1(f[g], lgb);
-            m[g] = f[g] >= 0 ? 1u << (h & 31) : 0u;
-            old[g] = f[g] >= 0 ? atomicOr(filt + (h >> 5), m[g]) : 0u;
+    const bool single = k1 - k0 <= NT;  // one batch of tails: the longest are set aside
+    const int32_t nset = smin <= 3 ? 1 : min(smin - 2, kSpDrop);
+    // the ids of a range: the whole span for rows of up to `chunk` wedges
+    const int32_t f_hi = a.row_fhi ? a.row_fhi[e] : R;
+    const int32_t chunk = smin <= 3 ? kSpChunk : kSpChunkAside;
+    int32_t step = (f_hi - (e + 1)) / ((work + chunk - 1) / chunk) + 1;
+    bool multi = work > chunk;  // several ranges: the row's pairs are gathered in scratch
+    // (both by the planning: cannot happen)
+    bool hand_over = work > C::MAXW || work > buf_stride;
+    bool full = false;  // the largest table, after an overflow
+    int32_t out = 0;    // pairs of the earlier ranges
+    int32_t next = 0, upto = 0;  // single: where the thread's tail goes on
+    lap(0);
+    for (int32_t Fa = e + 1; Fa < f_hi && !hand_over;) {
+      const int32_t Fb = f_hi - Fa > step ? Fa + step : f_hi;
+      int lgb = kSpLogB, lgt = C::LGT;
+      // The range's tails of incidences [base, base + NT) as segments of at
+      // most kSpSeg far ends: s_seg[0, nA) those to insert, s_seg[nA, nA + nD)
+      // those of the tails set aside.
+      int32_t nA = 0, nD = 0;
+      auto load_batch = [&](int32_t base) {
+        const int32_t k = base + tid;
+        int32_t b = 0, len = 0;
+        if (k < k1) {
+          b = __ldg(w.tail_beg + k);
+          int32_t end = __ldg(w.tail_end + k);
+          if (multi) {
+            // (one batch: the last range's end is kept)
+            if (Fa > e + 1) b = single ? next : lower_pos(w.c_idx_s, b, end, Fa);
+            if (Fb < f_hi) end = lower_pos(w.c_idx_s, b, end, Fb);
+            upto = end;
           }
-#if SLG_SP_DEFER
-          int32_t pend[kSpG] = {};
-          int np = 0;
-#pragma unroll
-          for (int g = 0; g < kSpG; ++g) pend_push(pend, np, (old[g] & m[g]) != 0, f[g], g);
-#pragma unroll
-          for (int q = 0; q < kSpG; ++q) {
-            if (!__any_sync(0xffffffffu, q < np)) break;
-            if (q < np) sp_candidate(tab, cand, pend[q], s_ovf, lgb, lgt);
+          len = end - b;
+        }
+        bool aside = false;
+        if (single) {
+          // a tail's rank by length (ties: the earlier one first)
+          s_len[tid] = len;
+          __syncthreads();
+          if (len > 0) {
+            int32_t r = 0;
+            const int32_t n = k1 - k0;
+            for (int32_t j = 0; j < n; ++j) {
+              const int32_t x = s_len[j];
+              r += x > len || (x == len && j < tid);
+            }
+            aside = r < nset;
           }
-#else
+          const int32_t sum = __reduce_add_sync(0xffffffffu, aside ? 0 : len);
+          if (lane == 0 && sum) atomicAdd(s_sum, sum);
+        }
+        const int32_t n = (len + kSpSeg - 1) / kSpSeg;
+        const int32_t packed = aside ? n << 16 : n;
+        int32_t total;
+        const int32_t pos = block_inclusive_scan<NT>(packed, ws, &total) - packed;
+        nA = total & 0xFFFF;
+        nD = total >> 16;
+        int2 *dst = s_seg + (aside ? nA + (pos >> 16) : pos & 0xFFFF);
+        for (int32_t i = 0; i < n; ++i)
+          dst[i] = make_int2(b + i * kSpSeg, min(kSpSeg, len - i * kSpSeg));
+        __syncthreads();
+      };
+      // step(f, last) for every segment of s_seg[x0, x1): a warp each
+      auto for_segments = [&](int32_t x0, int32_t x1, auto &&step) {
+        for (int32_t x = x0 + wq; x < x1; x += NW) {
+          const int2 sg = s_seg[x];
+          int32_t f[kSpG];
 #pragma unroll
           for (int g = 0; g < kSpG; ++g)
-            if (old[g] & m[g]) sp_candidate(tab, cand, f[g], s_ovf, lgb, lgt);
-#endif
-        });
-    __syncthreads();  // candidates final
-    {
-      const long long t1 = clock64();
-      cyc[1] += t1 - t0;
-      t0 = t1;
-    }
-    if (*s_ovf) {  // uniform: too many candidates for the table
-      if (tid == 0) {
-        // hand the row to the giant bin (launched after this kernel)
-        const unsigned pos = atomicAdd(&meta->giant_rest, 1u);
-        giant_rows[list_len - 1 - pos] = e;
-        atomicAdd(&meta->rows_bin[kBinGiant], 1ull);
-      }
-      clear_filters(lgb);
-      for (int i = tid; i < T; i += kSpNT) tab[i] = kEmpty64;
-      continue;
-    }
-    // 2. exact counts of the candidates
-    // (the deferred slow path, as in the walk below)
-    auto count_step = [&](const int32_t(&f)[kSpG]) {
-      uint32_t word[kSpG], bit[kSpG];
-#pragma unroll
-      for (int g = 0; g < kSpG; ++g) {  // the candidate filter, loads in flight together
-        const uint32_t c = sp_h2(f[g], lgb);
-        bit[g] = 1u << (c & 31);
-        word[g] = f[g] >= 0 ? cand[c >> 5] : 0u;
-      }
-      int32_t pend[kSpG] = {};
-      int np = 0;
-#pragma unroll
-      for (int g = 0; g < kSpG; ++g) pend_push(pend, np, (word[g] & bit[g]) != 0, f[g], g);
-#pragma unroll
-      for (int q = 0; q < kSpG; ++q) {
-        if (!__any_sync(0xffffffffu, q < np)) break;
-        if (q < np) sp_count_listed(tab, pend[q], smin, unweighted, lgt);
-      }
-    };
-    if (gbuf) {
-      // warp-uniform steps over the copy, 32 consecutive far ends per load
-      const int32_t lane = tid & 31;
-      for (int32_t b0 = (tid >> 5) * 32 * kSpG; b0 < work; b0 += kSpNT * kSpG) {
-        int32_t f[kSpG];
-#pragma unroll
-        for (int g = 0; g < kSpG; ++g) {
-          const int32_t i = b0 + 32 * g + lane;
-          f[g] = i < work ? gbuf[i] : -1;
+            f[g] = 32 * g + lane < sg.y ? __ldg(w.c_idx_s + sg.x + 32 * g + lane) : -1;
+          step(f, x + NW >= x1);
         }
-        count_step(f);
+      };
+      auto count = [&](int32_t x) {
+        sp_insert(tab, x, smin, unweighted, lgt, s_ovf, list, s_nsurv);
+      };
+      // 1. the inserted tails
+      bool hit = false;
+      for (int32_t base = k0; base < k1; base += NT) {
+        if (base > k0) __syncthreads();  // the previous batch's segments are read
+        load_batch(base);
+        if (base == k0) {
+          // a filter of >= 32 bits per inserted wedge (a single-wedge far end
+          // finds its bit set by another with probability below 1/64), and a
+          // table of half a slot per inserted wedge, within the maxima
+          const int32_t ins = single ? *s_sum : min(work, 2 * chunk);
+          lgb = min(max(ceil_log2(ins > 1 ? ins : 2) + 5, 12), kSpLogB);
+          if (!full) lgt = min(max(ceil_log2(ins / 2 + 1), 8), C::LGT);
+        }
+        for_segments(0, nA, [&](const int32_t(&f)[kSpG], bool) {
+          uint32_t old[kSpG], h[kSpG];
+#pragma unroll
+          for (int g = 0; g < kSpG; ++g) {
+            h[g] = sp_bit(f[g], lgb);
+            old[g] = f[g] >= 0 ? atomicOr(once + (h[g] >> 5), 1u << (h[g] & 31)) : 0u;
+          }
+#pragma unroll
+          for (int g = 0; g < kSpG; ++g)
+            if ((old[g] >> (h[g] & 31)) & 1u) {
+              atomicOr(twice + (h[g] >> 5), 1u << (h[g] & 31));
+              hit = true;
+            }
+        });
       }
-      __syncthreads();  // every read of the copy done
-      l2_discard(gbuf, work);
-    } else if (cached) {
-      for (int32_t i = tid; i < work; i += kSpNT)
-        sp_count(tab, cand, cache[i], smin, unweighted, lgb, lgt);
-    } else {
-      cta_walk_batched<kSpNT, kSpG>(
-          w, k0, k1, s_beg, s_pref, ws, [&](const int32_t(&f)[kSpG], int32_t) {
-#if SLG_SP_DEFER
-            uint32_t word[kSpG], bit[kSpG];
+      if (hit) *s_any = 1;
+      __syncthreads();  // both filters as far as the inserted tails go
+      // 2. one tail set aside (s <= 3)
+      if (smin <= 3 && nA > 0 && nD > 0) {  // uniform
+        bool in = false;
+        for_segments(nA, nA + nD, [&](const int32_t(&f)[kSpG], bool last) {
 #pragma unroll
-            for (int g = 0; g < kSpG; ++g) {  // the candidate filter, loads in flight together
-              const uint32_t c = sp_h2(f[g], lgb);
-              bit[g] = 1u << (c & 31);
-              word[g] = f[g] >= 0 ? cand[c >> 5] : 0u;
+          for (int g = 0; g < kSpG; ++g) {
+            const uint32_t h = sp_bit(f[g], lgb);
+            const bool c = f[g] >= 0 && ((once[h >> 5] >> (h & 31)) & 1u);
+            if (c) {
+              atomicOr(twice + (h >> 5), 1u << (h & 31));
+              in = true;
             }
-            int32_t pend[kSpG] = {};
-            int np = 0;
-#pragma unroll
-            for (int g = 0; g < kSpG; ++g) pend_push(pend, np, (word[g] & bit[g]) != 0, f[g], g);
-#pragma unroll
-            for (int q = 0; q < kSpG; ++q) {
-              if (!__any_sync(0xffffffffu, q < np)) break;
-              if (q < np) sp_count_listed(tab, pend[q], smin, unweighted, lgt);
-            }
-#else
-#pragma unroll
-            for (int g = 0; g < kSpG; ++g)
-              if (f[g] >= 0) sp_count(tab, cand, f[g], smin, unweighted, lgb, lgt);
-#endif
+            q.push(c, f[g]);
+          }
+          q.drain(last, [&](int32_t x) {
+            // (nothing is listed here: a first wedge, and s >= 2)
+            sp_insert(tab, x, 0x7fffffff, unweighted, lgt, s_ovf, list, s_nsurv);
           });
-    }
-    __syncthreads();  // counts final
-    {
-      const long long t1 = clock64();
-      cyc[2] += t1 - t0;
-      t0 = t1;
-    }
-    // 3. candidates with count >= s, in ascending f at tab[at, at + n)
-    int32_t at = 0, used = T;
-    // (ordering n survivors needs 2 n + 32 slots of the table)
-    const int32_t n = table_collect<kSpNT, kSPT, (SLG_SP_RUNS != 0)>(
-        tab, T, smin, emit, ws, &at, &used, (T - 32) / 2);
-    if (n < 0) {  // uniform: hand the row to the giant bin, as for an overflow
+        });
+        if (in) *s_any = 1;
+        __syncthreads();  // `twice` is final, `once` is not read any more
+      }
+      lap(1);
+      const int32_t T = 1 << lgt;
+      int32_t n = 0, dirty_once = 1 << (lgb - 5), dirty_twice = dirty_once;
+      bool redo = false;
+      if (*s_any) {  // uniform: else no far end has two wedges
+        // 3. counts
+        for (int32_t base = k0; base < k1; base += NT) {
+          if (!single) {
+            if (base > k0) __syncthreads();
+            load_batch(base);
+          }
+          for_segments(0, smin > 3 ? nA + nD : nA, [&](const int32_t(&f)[kSpG], bool last) {
+            uint32_t word[kSpG], h[kSpG];
+#pragma unroll
+            for (int g = 0; g < kSpG; ++g) {  // loads in flight together
+              h[g] = sp_bit(f[g], lgb);
+              word[g] = f[g] >= 0 ? twice[h[g] >> 5] : 0u;
+            }
+#pragma unroll
+            for (int g = 0; g < kSpG; ++g) q.push((word[g] >> (h[g] & 31)) & 1u, f[g]);
+            q.drain(last, count);
+          });
+        }
+        __syncthreads();  // counts and survivors final
+        lap(2);
+        n = *s_nsurv;
+        dirty_once = max(dirty_once, min(n, kSpList));  // the list
+        // 4. survivors in ascending f.  Those that fit are ranked in `twice`
+        // while the table is cleared; more of them are ordered in the table.
+        const bool small = n <= kSpSortMax;
+        if (*s_ovf || (emit && !small && (n > NT * kSpRegQ || n > kSpList))) {
+          redo = true;
+        } else if (emit && n > 0) {
+          long long base = -1;
+          if (!multi && tid == 0) *s_base = reserve(a, e, n, kBinSparse);
+          auto write = [&](int32_t i, unsigned long long x) {
+            const int32_t f = (int32_t)(x >> 32), c = (int32_t)(uint32_t)x;
+            if (multi) {
+              pj[out + i] = f;
+              if (!unweighted) pw[out + i] = c;
+            } else if (base >= 0) {
+              put(a, base, i, e, f, c);
+            }
+          };
+          if (small) {
+            dirty_twice = max(dirty_twice, 2 * ((n + 31) & ~31));
+            for (int32_t i = tid; i < n; i += NT)
+              keys[i] = tab[list[i]] + 1ull;  // the count word holds count - 1
+            __syncthreads();  // keys and base in place, the table is read
+            base = *s_base;
+            clear_slots<NT>(tab, T);
+            rank_keys<NT>(keys, n, write);
+          } else {
+            unsigned long long x[kSpRegQ];
+#pragma unroll
+            for (int i = 0; i < kSpRegQ; ++i)
+              x[i] = tid + i * NT < n ? tab[list[tid + i * NT]] + 1ull : 0ull;
+            __syncthreads();  // keys read, base in place
+            base = *s_base;
+            clear_slots<NT>(tab, T);
+            __syncthreads();
+#pragma unroll
+            for (int i = 0; i < kSpRegQ; ++i)
+              if (tid + i * NT < n) tab[tid + i * NT] = x[i];
+            __syncthreads();
+            int32_t used = 0;
+            const int32_t at = sort_survivors<NT, true>(tab, n, &used);
+            for (int32_t i = tid; i < n; i += NT) write(i, tab[at + i]);
+            __syncthreads();  // the sorted keys are written
+            clear_slots<NT>(tab, used);
+          }
+        } else {
+          if (!multi && tid == 0) reserve(a, e, n, kBinSparse);
+          clear_slots<NT>(tab, T);
+        }
+      } else {
+        lap(2);
+      }
+      __syncthreads();  // every shared value of the range is read
+      lap(3);
+      if (redo) {
+        const bool over = *s_ovf != 0;
+        __syncthreads();  // s_ovf is read
+        if (over && lgt < C::LGT) {
+          full = true;
+        } else {  // half the ids at a time
+          multi = true;
+          hand_over = step <= 64;
+          step = (step + 1) / 2;
+        }
+        clear_slots<NT>(tab, T);
+      } else {
+        out += n;
+        next = upto;
+        Fa = Fb;
+        full = false;
+      }
+      zero(once, dirty_once);
+      zero(twice, dirty_twice);
+      if (tid == 0) {
+        *s_ovf = 0;
+        *s_any = 0;
+        *s_sum = 0;
+        *s_nsurv = 0;
+      }
       __syncthreads();
+      lap(4);
+    }
+    if (hand_over) {
+      // to the giant bin (launched after this kernel)
       if (tid == 0) {
         const unsigned pos = atomicAdd(&meta->giant_rest, 1u);
         giant_rows[list_len - 1 - pos] = e;
         atomicAdd(&meta->rows_bin[kBinGiant], 1ull);
       }
-      clear_filters(lgb);
-      for (int i = tid; i < T; i += kSpNT) tab[i] = kEmpty64;
-      continue;
+    } else if (multi) {
+      if (tid == 0) *s_base = reserve(a, e, out, kBinSparse);
+      __syncthreads();
+      const long long base = *s_base;
+      if (emit && base >= 0)
+        for (int32_t i = tid; i < out; i += NT)
+          put(a, base, i, e, pj[i], unweighted ? 0 : pw[i]);
     }
-    if (tid == 0) *s_base = reserve(a, e, n, kBinSparse);
-    __syncthreads();
-    {
-      const long long t1 = clock64();
-      cyc[3] += t1 - t0;
-      t0 = t1;
-    }
-    const long long base = *s_base;
-    if (emit && base >= 0)
-      for (int32_t i = tid; i < n; i += kSpNT) {
-        const unsigned long long x = tab[at + i];
-        const int32_t f = (int32_t)(x >> 32), c = (int32_t)(uint32_t)x;
-        put(a, base, i, e, f, c);
-      }
-    clear_filters(lgb);  // nothing reads the filters after the second pass
-    table_reset_front<kSpNT>(tab, used);
-    cyc[4] += clock64() - t0;
+    lap(4);
   }
   if (tid == 0)
-    for (int q = 0; q < 5; ++q) atomicAdd(&meta->sparse_cycles[q], (unsigned long long)cyc[q]);
+    for (int i = 0; i < 5; ++i) atomicAdd(&meta->sparse_cycles[i], (unsigned long long)s_cyc[i]);
 }
 
-#define K_SP_BIG k_walk_sparse<kSpLgT, SLG_SP_MINB>
-#define K_SP_SMALL k_walk_sparse<kSpSmallLgT, SLG_SP_SMALL_MINB>
-
 struct SpOcc {
-  int big = 0, small = 0;  // CTAs
+  int small = 0, big = 0;  // CTAs
   int dev = -1;
 };
+
+template <class C>
+int sp_ctas(int sms) {
+  int nb = 0;
+  cudaFuncSetAttribute(k_walk_sparse<C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)sparse_smem<C>());
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_walk_sparse<C>, C::NT, sparse_smem<C>());
+  return sms * std::max(nb, 1);
+}
 
 SpOcc &sp_occ() {
   static SpOcc occ[64];
@@ -419,45 +534,39 @@ SpOcc &sp_occ() {
   SpOcc &o = occ[dev & 63];
   std::lock_guard<std::mutex> lock(mu);
   if (o.dev != dev) {
-    int sms = 0, nb = 0;
+    int sms = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaFuncSetAttribute(K_SP_BIG, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)sparse_smem(kSpLgT));
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, K_SP_BIG, kSpNT, sparse_smem(kSpLgT));
-    o.big = sms * std::max(nb, 1);
-    cudaFuncSetAttribute(K_SP_SMALL, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)sparse_smem(kSpSmallLgT));
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, K_SP_SMALL, kSpNT,
-                                                  sparse_smem(kSpSmallLgT));
-    o.small = sms * std::max(nb, 1);
+    o.small = sp_ctas<SpSmall>(sms);
+    o.big = sp_ctas<SpBig>(sms);
     o.dev = dev;
   }
   return o;
 }
 
+template <class C>
+void sp_launch(const WalkLaunch &L, int ctas, int part, cudaStream_t st) {
+  const int64_t stride = L.rows;
+  k_walk_sparse<C><<<ctas, C::NT, sparse_smem<C>(), st>>>(
+      L.w, L.bin_rows + (int64_t)kBinSparse * stride, L.a,
+      const_cast<int32_t *>(L.bin_rows) + (int64_t)kBinGiant * stride, (int32_t)stride,
+      L.giant_scratch, (L.scratch_ints / (long long)ctas) & ~31ll, L.R, part);
+}
+
 }  // namespace
 
-int sparse_ctas() { return std::max(sp_occ().big, sp_occ().small); }
+// Scratch ints for rows of up to `max_work` wedges.
+long long sparse_ints(int32_t max_work) {
+  SpOcc &o = sp_occ();
+  return std::max((long long)o.small * (std::min(max_work, kSparseBigWork) + 128ll),
+                  (long long)o.big * (max_work + 128ll));
+}
 
 cudaError_t launch_walk_sparse(const WalkLaunch &L, cudaStream_t st, int32_t *launches) {
+  if (!L.giant_scratch) return cudaSuccess;  // no row in the bin
   SpOcc &o = sp_occ();
-  const int64_t stride = L.rows;
-  // the CTAs share the giant bin's scratch out (it holds at least
-  // 4 x max(giant, sparse row work) ints per giant CTA)
-  auto buf_stride = [&](int ctas) -> long long {
-    return L.giant_scratch ? (L.scratch_ints / (long long)ctas) & ~31ll : 0;
-  };
-  const int32_t *rows = L.bin_rows + (int64_t)kBinSparse * stride;
-  int32_t *giant_list = const_cast<int32_t *>(L.bin_rows) + (int64_t)kBinGiant * stride;
-  K_SP_BIG<<<o.big, kSpNT, sparse_smem(kSpLgT), st>>>(L.w, rows, L.a, giant_list, (int32_t)stride,
-                                                      L.giant_scratch, buf_stride(o.big),
-                                                      SLG_SP_BIG_WORK > 0 ? 1 : 0);
-  ++*launches;
-  if (SLG_SP_BIG_WORK > 0) {
-    K_SP_SMALL<<<o.small, kSpNT, sparse_smem(kSpSmallLgT), st>>>(
-        L.w, rows, L.a, giant_list, (int32_t)stride, L.giant_scratch, buf_stride(o.small), 2);
-    ++*launches;
-  }
+  sp_launch<SpBig>(L, o.big, 0, st);
+  sp_launch<SpSmall>(L, o.small, 1, st);
+  *launches += 2;
   return cudaGetLastError();
 }
 

@@ -138,3 +138,76 @@ def test_two_instances_and_hand_off(s):
     assert w is None
     assert np.array_equal(np.stack([i.cpu().numpy(), j.cpu().numpy()], 1), want[:, :2])
     assert slg.count(dh, s) == want.shape[0]
+
+
+def aside_rows(m=500_000, n=900_000, seed=15, small=(1, 4)):
+    """Three rows sparse in 500,000 ids, the other rows of small[0] to
+    small[1] - 1 random vertices.  Row 0: two vertices with the same
+    6,000 other hyperedges (more survivors than one range can order) and 18
+    rare ones.  Row 1: 600 vertices of 40 hyperedges (more tails than a batch
+    holds, nothing set aside), 100 hyperedges holding seven of them.  Row 2:
+    12 vertices of 100 to 4,000 hyperedges (all but a few of its wedges are in
+    the longest tails), 50 hyperedges holding nine of them."""
+    rng = np.random.default_rng(seed)
+    size = rng.integers(*small, m)
+    r = [np.repeat(np.arange(m), size)]
+    c = [rng.integers(10_000, n, int(size.sum()))]
+
+    def add(row, col):
+        r.append(np.broadcast_to(row, np.broadcast(row, col).shape).ravel())
+        c.append(np.broadcast_to(col, np.broadcast(row, col).shape).ravel())
+
+    f = rng.choice(np.arange(3, m), 6_000, replace=False)
+    add(f, 0)
+    add(f, 1)
+    add(0, np.arange(20))
+    for v in range(600):
+        add(rng.choice(np.arange(3, m), 40, replace=False), 1_000 + v)
+    add(1, np.arange(1_000, 1_600))
+    for x in rng.choice(np.arange(3, m), 100, replace=False):
+        add(x, 1_000 + rng.choice(600, 7, replace=False))
+    for v in range(12):
+        add(rng.choice(np.arange(3, m), 100 if v < 6 else 4_000, replace=False), 3_000 + v)
+    add(2, np.arange(3_000, 3_012))
+    for x in rng.choice(np.arange(3, m), 50, replace=False):
+        add(x, 3_000 + rng.choice(12, 9, replace=False))
+    return hg.from_pairs(np.concatenate(r), np.concatenate(c), m, n)
+
+
+@pytest.fixture(scope="module")
+def aside():
+    h = aside_rows()
+    return h, slg.to_device(h)
+
+
+@pytest.mark.parametrize("s", [2, 3, 4, 5, 6, 9, 12])
+def test_tails_set_aside_and_split_ranges(aside, s):
+    h, dh = aside
+    want = oracle.canonical(*oracle.line_graph_of(h, s, threads=8))
+    got = as_np(slg.build(dh, s))
+    if s <= 3:  # (the small rows leave at larger s)
+        assert slg.last_stats()["rows_bin"][4] > 0
+    assert np.array_equal(got, want)
+    i, j, w = slg.build(dh, s, unweighted=True)
+    assert w is None and np.array_equal(
+        np.stack([i.cpu().numpy(), j.cpu().numpy()], 1), want[:, :2])
+    assert slg.count(dh, s) == want.shape[0]
+
+
+@pytest.fixture(scope="module")
+def aside_large():
+    h = aside_rows(small=(12, 15))
+    return h, slg.to_device(h)
+
+
+@pytest.mark.parametrize("s", [4, 6, 9, 12])
+def test_tails_set_aside_large_rows(aside_large, s):
+    # rows of 12 and more vertices: the far ends stay at these thresholds
+    h, dh = aside_large
+    rows = np.unique(np.concatenate([np.arange(3), np.arange(0, h.m, 53)])).astype(np.int32)
+    m, n, off, idx = oracle.side(h, False)
+    want = oracle.canonical(*oracle.line_graph(m, n, off, idx, s, rows=rows, threads=8))
+    got = as_np(slg.build(dh, s))
+    assert slg.last_stats()["rows_bin"][4] > 0
+    assert np.array_equal(got[np.isin(got[:, 0], rows)], want)
+    assert slg.count(dh, s) == got.shape[0]
