@@ -22,7 +22,8 @@
 // fewer windows a row has the better: rows of more than kDenseBigSize
 // vertices (short pieces of many tails: 3 to 8 entries of a tail in a window
 // of 26K ids) take an instance with one CTA of 1,024 threads per SM and a
-// window of 96K ids; the others one with three CTAs of 512 threads.
+// window of 96K ids; the others one with four CTAs of 256 threads and windows
+// of 80K (4-bit) or 40K ids (8-bit counters).
 //
 // Measured on chung_lu_1m (1M x 2M) against the partitioned hash buckets and
 // dense windows of the giant bin that these rows took before: L_8 of H, giant
@@ -30,7 +31,12 @@
 // 8.7, small 10.7, giant 17.3 ms.  A scan of the counters in place of the
 // survivor bits cost 26 instead of 13 x 10^9 CTA cycles on L_2(H*) (rows down
 // to one wedge per 32 ids); windows of 26K ids for every row took 13.9
-// instead of 9.2 ms on L_2(H).
+// instead of 9.2 ms on L_2(H).  The small instance with three CTAs of 512
+// threads and windows of 104K / 52K ids, as it first was: half of its warps'
+// time went on barriers (few tails per window and warp); L_8 of a 300K x 600K
+// dual 10.98 -> 9.53 ms, step of chung_lu_1m 118.4 -> 115.1 ms with four
+// of 256 threads (five with 8,192 words: 9.83, 117.6; eight of 128 threads
+// with 4,608 words: 8.86, 118.8).
 #include <algorithm>
 #include <mutex>
 
@@ -40,11 +46,11 @@ namespace slg {
 
 namespace {
 
-#ifndef SLG_DN_WORDS
-#define SLG_DN_WORDS 13312
+#ifndef SLG_DN_NT
+#define SLG_DN_NT 256
 #endif
-#ifndef SLG_DN_BIG_WORDS
-#define SLG_DN_BIG_WORDS 48128
+#ifndef SLG_DN_MINB
+#define SLG_DN_MINB 4
 #endif
 #ifndef SLG_DN_LONG
 #define SLG_DN_LONG 16
@@ -58,28 +64,29 @@ namespace {
 #ifndef SLG_DN_UL
 #define SLG_DN_UL 2
 #endif
-constexpr int kDnEntExtra = 512;              // list entries beyond one per tail, at most
 constexpr int kDnSeg = SLG_DN_SEG;            // a tail's entries per window and list entry, about
-constexpr int kDnSmemEnt = kDnEntExtra * 2;   // list entries held in shared memory
 constexpr int kDnUS = SLG_DN_US;              // short entries in flight per 8 lanes
 constexpr int kDnUL = SLG_DN_UL;              // long entries in flight per warp
 
 // The two instances of the kernel: NT threads, WORDS counter words per
 // window, MAP words of survivor bits (counters of at least 32 WORDS / (32
-// MAP) bits), MINB CTAs per SM.
+// MAP) bits), MINB CTAs per SM, ENT list entries in shared memory, EXTRA of
+// them beyond one per tail.
 struct DnSmall {
-  static constexpr int NT = 512, MINB = 3, WORDS = SLG_DN_WORDS, MAP = WORDS / 4;
+  static constexpr int NT = SLG_DN_NT, MINB = SLG_DN_MINB, WORDS = SLG_DN_WORDS, MAP = WORDS / 4;
+  static constexpr int EXTRA = 128, ENT = kDenseBigSize + EXTRA + 1;
 };
 struct DnBig {
   static constexpr int NT = 1024, MINB = 1, WORDS = SLG_DN_BIG_WORDS, MAP = WORDS / 16;
+  static constexpr int EXTRA = 512, ENT = 1024;
 };
 
-// [counters][survivor bits][entries kDnSmemEnt x 8][totals 2 x 32 x 4]
+// [counters][survivor bits][entries C::ENT x 8][totals 2 x 32 x 4]
 // [n_long, n_short, row, pad][base 8]
 template <class C>
 constexpr size_t dense_smem() {
   static_assert(C::WORDS % 64 == 0, "16-byte alignment of the parts");
-  return (size_t)C::WORDS * 4 + (size_t)C::MAP * 4 + (size_t)kDnSmemEnt * 8 + 2 * 32 * 4 + 16 + 16;
+  return (size_t)C::WORDS * 4 + (size_t)C::MAP * 4 + (size_t)C::ENT * 8 + 2 * 32 * 4 + 16 + 16;
 }
 
 // Adds n to counter o (2^LB bits wide, packed in 32-bit words) and marks o in
@@ -193,7 +200,7 @@ __global__ __launch_bounds__(C::NT, C::MINB) void k_walk_dense(
   uint4 *cnt4 = reinterpret_cast<uint4 *>(smem);
   uint32_t *map = cnt + C::WORDS;
   int2 *s_ent = reinterpret_cast<int2 *>(map + C::MAP);
-  int32_t *s_tot = reinterpret_cast<int32_t *>(s_ent + kDnSmemEnt);
+  int32_t *s_tot = reinterpret_cast<int32_t *>(s_ent + C::ENT);
   int32_t *s_n = s_tot + 64;  // [0] long entries, [1] short entries, [2] row
   long long *s_base = reinterpret_cast<long long *>(s_n + 4);
   // per-CTA global scratch: staged pairs (j, w), then the list entries of
@@ -239,16 +246,16 @@ __global__ __launch_bounds__(C::NT, C::MINB) void k_walk_dense(
     // with many entries per window from the front (a warp sweeps one), the
     // others from the back (8 lanes sweep one).  A tail with more than seg
     // entries is cut into several, so that no warp sweeps far more of a
-    // window than the others: at most (k1 - k0) + kDnEntExtra entries.
-    const bool in_smem = k1 - k0 <= kDnSmemEnt - kDnEntExtra;
+    // window than the others: at most (k1 - k0) + C::EXTRA entries.
+    const bool in_smem = k1 - k0 <= C::ENT - C::EXTRA;
     int2 *ent = in_smem ? s_ent : g_ent;
-    const int32_t ecap = in_smem ? kDnSmemEnt : ent_cap;
-    if (!in_smem && k1 - k0 + kDnEntExtra > ent_cap) {  // sized by the planning: cannot happen
+    const int32_t ecap = in_smem ? C::ENT : ent_cap;
+    if (!in_smem && k1 - k0 + C::EXTRA > ent_cap) {  // sized by the planning: cannot happen
       if (tid == 0) raise_error(meta, SLG_ERR_INVALID, kWhereGiant);
       break;
     }
     const int32_t work = a.row_work[e - a.row_begin];
-    const int32_t seg = max(kDnSeg * min(nwin, 1 << 20), work / (kDnEntExtra - 1) + 1);
+    const int32_t seg = max(kDnSeg * min(nwin, 1 << 20), work / (C::EXTRA - 1) + 1);
     const int32_t long_min = SLG_DN_LONG * min(nwin, 1 << 24);
     for (int32_t k = k0 + tid; k < k1; k += NT) {
       int32_t b = __ldg(w.tail_beg + k);
@@ -423,10 +430,11 @@ DnOcc &dn_occ() {
 
 // Ints per CTA: pairs of the largest row (two arrays) and the entries of the
 // row with the most tails.
+template <class C>
 long long dense_stride(long long max_pairs, int32_t max_size, long long *pair_cap,
                        int32_t *ent_cap) {
   *pair_cap = (max_pairs + 31) & ~31ll;
-  *ent_cap = max_size > kDnSmemEnt - kDnEntExtra ? (max_size + kDnEntExtra + 15) & ~15 : 0;
+  *ent_cap = max_size > C::ENT - C::EXTRA ? (max_size + C::EXTRA + 15) & ~15 : 0;
   return 2 * *pair_cap + 2ll * *ent_cap;
 }
 
@@ -437,9 +445,9 @@ long long dense_ints(long long pairs_big, long long pairs_small, int32_t size_bi
   DnOcc &o = dn_occ();
   long long pc = 0;
   int32_t ec = 0;
-  const long long b = pairs_big > 0 ? o.big * dense_stride(pairs_big, size_big, &pc, &ec) : 0;
+  const long long b = pairs_big > 0 ? o.big * dense_stride<DnBig>(pairs_big, size_big, &pc, &ec) : 0;
   const long long s = pairs_small > 0
-                          ? o.small * dense_stride(pairs_small, kDenseBigSize, &pc, &ec)
+                          ? o.small * dense_stride<DnSmall>(pairs_small, kDenseBigSize, &pc, &ec)
                           : 0;
   return std::max(b, s);
 }
@@ -450,13 +458,13 @@ cudaError_t launch_walk_dense(const WalkLaunch &L, cudaStream_t st, int32_t *lau
   long long pc = 0;
   int32_t ec = 0;
   if (L.dense_pairs[0] > 0) {
-    const long long stride = dense_stride(L.dense_pairs[0], L.dense_size, &pc, &ec);
+    const long long stride = dense_stride<DnBig>(L.dense_pairs[0], L.dense_size, &pc, &ec);
     k_walk_dense<DnBig><<<o.big, DnBig::NT, dense_smem<DnBig>(), st>>>(
         L.w, rows, L.a, L.giant_scratch, stride, pc, ec, L.R, L.rows, 0);
     ++*launches;
   }
   if (L.dense_pairs[1] > 0) {
-    const long long stride = dense_stride(L.dense_pairs[1], kDenseBigSize, &pc, &ec);
+    const long long stride = dense_stride<DnSmall>(L.dense_pairs[1], kDenseBigSize, &pc, &ec);
     k_walk_dense<DnSmall><<<o.small, DnSmall::NT, dense_smem<DnSmall>(), st>>>(
         L.w, rows, L.a, L.giant_scratch, stride, pc, ec, L.R, L.rows, 1);
     ++*launches;

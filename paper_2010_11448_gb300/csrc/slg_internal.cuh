@@ -56,15 +56,8 @@ constexpr int32_t kSparseBigWork = SLG_SP_BIG_WORK;
 #define SLG_SPARSE_MAX_WORK 65536
 #endif
 constexpr int32_t kSparseMaxWork = SLG_SPARSE_MAX_WORK;
-// A row is dense when it has at least one wedge per this many ids of its far
-// ends' span, for 16-bit counters (see is_dense).  L_8(H), L_2(H*) and L_8(H*)
-// of chung_lu_1m together: 119.0, 121.5, 163.6 ms with 16, 24, 48.
-#ifndef SLG_DENSE_RATIO
-#define SLG_DENSE_RATIO 16
-#endif
-constexpr int kDenseRatio = SLG_DENSE_RATIO;
 #ifndef SLG_DENSE_MIN_WORK
-#define SLG_DENSE_MIN_WORK 1024
+#define SLG_DENSE_MIN_WORK 256
 #endif
 constexpr int32_t kDenseMinWork = SLG_DENSE_MIN_WORK;
 // Dense rows of more vertices (16-bit counters and up) take the instance of
@@ -77,11 +70,54 @@ __host__ __device__ __forceinline__ int dense_lg_bits(int32_t size) {
   return size <= 15 ? 2 : size <= 255 ? 3 : size <= 65535 ? 4 : 5;
 }
 
-// Dense rows: the dense bin's cost per row is its wedges plus its counters
-// (span x bits), so the line is drawn at a number of wedges per counter byte.
-__host__ __device__ __forceinline__ bool is_dense(int32_t work, int32_t size, int32_t span,
-                                                  int32_t ratio) {
-  return ((long long)work * ratio << 4) >= ((long long)span << dense_lg_bits(size));
+// Counter words of a window of the dense bin's two instances.
+#ifndef SLG_DN_WORDS
+#define SLG_DN_WORDS 10240
+#endif
+#ifndef SLG_DN_BIG_WORDS
+#define SLG_DN_BIG_WORDS 48128
+#endif
+// Wedges per window and row from which a row is dense, by what else would
+// count it (see is_dense): s = 1 (CTA bins or giant bin; L_1 of 100K x 200K
+// 4.12, 3.84, 3.15 ms with 700, 200 from 1,024 wedges and 200 from 256); rows
+// of up to kDenseFew vertices per vertex beyond two of the threshold, whose
+// wedges the sparse bin mostly sets aside (L_8 of a 300K x 600K dual 7.48,
+// 6.83, 7.06 ms with 2,000, 3,000, 4,500; 10.0 with one line for all s); the
+// other rows (L_2 and more of a 150K x 300K dual 14.1, 13.8, 13.2 ms, step of
+// chung_lu_1m 118.5, 118.4, 120.0 with 1,000, 1,300, 1,800); rows of the
+// large-window instance (118.5, 117.8, 121.9 ms with 5,000, 3,500, 8,000,
+// and 115.0, 115.3 with 2,500, 1,500 and the rest as here).
+#ifndef SLG_DENSE_T1
+#define SLG_DENSE_T1 200
+#endif
+#ifndef SLG_DENSE_T2
+#define SLG_DENSE_T2 1300
+#endif
+#ifndef SLG_DENSE_T4
+#define SLG_DENSE_T4 3000
+#endif
+#ifndef SLG_DENSE_KF
+#define SLG_DENSE_KF 10
+#endif
+constexpr int32_t kDenseFew = SLG_DENSE_KF;
+#ifndef SLG_DENSE_TB
+#define SLG_DENSE_TB 2000
+#endif
+constexpr int kDenseRatio = 16;
+
+// Dense rows: the dense bin's cost per row is its wedges plus so much per
+// window (sweep latency, survivors, clear), the other bins' is their cost per
+// wedge; so the line is drawn at a number of wedges per window.
+__host__ __device__ __forceinline__ bool is_dense(int32_t work, int32_t size, int32_t s,
+                                                  int32_t span, int32_t ratio) {
+  const int lw = 5 - dense_lg_bits(size);
+  const bool big = size > kDenseBigSize;
+  const int32_t nwin = span / ((big ? SLG_DN_BIG_WORDS : SLG_DN_WORDS) << lw) + 1;
+  const int32_t per = big                                          ? SLG_DENSE_TB
+                      : s == 1                                     ? SLG_DENSE_T1
+                      : size <= (long long)kDenseFew * (s - 2) ? SLG_DENSE_T4
+                                                                   : SLG_DENSE_T2;
+  return (long long)work * ratio >= (long long)per * 16 * nwin;
 }
 
 // Counters the device writes and the host reads once per call.
@@ -390,8 +426,8 @@ __device__ __forceinline__ int32_t s_of(const int32_t *row_s, int32_t smin, int3
 #ifndef SLG_BLOOM_MIN_WORK
 #define SLG_BLOOM_MIN_WORK 1024
 #endif
-// `dense`: a row with at least one wedge per `dense` ids of its far ends'
-// span is dense, for 16-bit counters (see is_dense).
+// `dense`: scales the dense bin's threshold (see is_dense; 16: as stated there,
+// more: more rows are dense).
 struct Bins {
   int32_t warp = kWarpMaxWork, ctas = kCtaSMaxWork, ctal = kCtaLMaxWork;
   int32_t sparse = kSparseMaxWork;

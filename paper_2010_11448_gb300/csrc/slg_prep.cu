@@ -281,7 +281,7 @@ __global__ __launch_bounds__(kRowsNT) void k_rows_work(Side s, int32_t smin, int
       const int32_t span = (s.row_fhi ? s.row_fhi[e] : s.R) - 1 - e;  // far ends: (e, e + span]
       // a row whose far ends are dense in its span takes the dense bin; else
       // one with s >= 2 from bins.bloom up to bins.sparse wedges the sparse bin
-      if ((forced || my_work > kDenseMinWork) && is_dense(my_work, size, span, bins.dense))
+      if ((forced || my_work > kDenseMinWork) && is_dense(my_work, size, se, span, bins.dense))
         my_bin = kBinDense;
       else if (!forced && my_work > bins.bloom && my_work <= bins.sparse && se >= 2)
         my_bin = kBinSparse;

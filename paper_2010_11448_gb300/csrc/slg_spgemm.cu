@@ -17,7 +17,7 @@ constexpr int kRowsPerBlock = 64;
 
 // (full columns: far ends lie anywhere in [0, R), threshold 1)
 __device__ __forceinline__ int bin_of_full(int32_t work, int32_t size, int32_t R) {
-  if (work > kDenseMinWork && is_dense(work, size, R, kDenseRatio)) return kBinDense;
+  if (work > kDenseMinWork && is_dense(work, size, 1, R, kDenseRatio)) return kBinDense;
   if (work <= kWarpMaxWork) return kBinWarp;
   if (work <= kCtaSMaxWork) return kBinCtaS;
   if (work <= kCtaLMaxWork) return kBinCtaL;
