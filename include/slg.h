@@ -293,6 +293,25 @@ int slg_filter(const int32_t *in_i, const int32_t *in_j, const int32_t *in_w,
                void *stream);
 
 /*
+ * slg_filter in two calls, for callers that allocate the outputs by the
+ * kept count (one pass over the weights less than slg_filter twice):
+ *   slg_filter_count  counts; `tiles` is a device array of
+ *                     as many entries as slg_filter_tiles says; it receives
+ *                     where each tile's kept triples start
+ *   slg_filter_write  writes them; in_w, n, s and tiles as in the count.
+ *                     Nothing is written beyond `capacity`.  Enqueued on
+ *                     `stream`; does not synchronise
+ * They return SLG_OK, SLG_ERR_INVALID or SLG_ERR_CUDA.
+ */
+int slg_filter_tiles(int64_t n, int64_t *n_tiles);
+int slg_filter_count(const int32_t *in_w, int64_t n, int32_t s, int64_t *tiles,
+                     int64_t *n_pairs, void *stream);
+int slg_filter_write(const int32_t *in_i, const int32_t *in_j,
+                     const int32_t *in_w, int64_t n, int32_t s,
+                     const int64_t *tiles, int32_t *out_i, int32_t *out_j,
+                     int32_t *out_w, int64_t capacity, void *stream);
+
+/*
  * slg_build_sweep -- L_s for `count` thresholds with one walk: L_{s_min}
  * (the smallest threshold) is built by slg_build, every other list is
  * filtered from it (slg_filter).

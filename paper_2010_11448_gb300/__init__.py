@@ -133,6 +133,10 @@ ABI_FUNCTIONS = {
     "slg_tile_overlap": (ctypes.c_int, [_VP, ctypes.c_int32, ctypes.c_int32, _VP, _VP]),
     "slg_filter": (ctypes.c_int, [_VP, _VP, _VP, ctypes.c_int64, ctypes.c_int32, _VP, _VP,
                                   _VP, ctypes.c_int64, _I64P, _VP]),
+    "slg_filter_tiles": (ctypes.c_int, [ctypes.c_int64, _I64P]),
+    "slg_filter_count": (ctypes.c_int, [_VP, ctypes.c_int64, ctypes.c_int32, _VP, _I64P, _VP]),
+    "slg_filter_write": (ctypes.c_int, [_VP, _VP, _VP, ctypes.c_int64, ctypes.c_int32, _VP, _VP,
+                                        _VP, _VP, ctypes.c_int64, _VP]),
     "slg_build_sweep": (ctypes.c_int, [_HP, _VP, ctypes.c_int32, ctypes.c_uint32, _VP, _VP,
                                        _VP, _VP, _VP, _VP]),
     "slg_squeeze": (ctypes.c_int, [_VP, _VP, ctypes.c_int64, ctypes.c_int32, _VP, _VP, _VP,
@@ -498,12 +502,26 @@ def filter_pairs(i, j, w, s: int, out=None, stream=None, weights=True):
     s' <= s: the triples with w >= s, in order (slg_filter)."""
     n = int(i.shape[0])
     if out is None:
+        # the count's tile offsets serve the write as well
+        import torch
+        lib = load()
         cnt = ctypes.c_int64(0)
-        rc = load().slg_filter(i.data_ptr(), j.data_ptr(), w.data_ptr(), n, int(s), None, None,
-                               None, 0, ctypes.byref(cnt), _stream(stream))
-        if rc not in (0, SLG_ERR_CAPACITY):
+        lib.slg_filter_tiles(n, ctypes.byref(cnt))
+        tiles = torch.empty(cnt.value, dtype=torch.int64, device=i.device)
+        rc = lib.slg_filter_count(w.data_ptr(), n, int(s), tiles.data_ptr(), ctypes.byref(cnt),
+                                  _stream(stream))
+        p = int(cnt.value)
+        oi, oj, ow = _outputs(p, not weights, i.device)
+        if rc == 0 and p > 0:
+            rc = lib.slg_filter_write(i.data_ptr(), j.data_ptr(), w.data_ptr(), n, int(s),
+                                      tiles.data_ptr(), oi.data_ptr(), oj.data_ptr(),
+                                      ow.data_ptr() if ow is not None else None, p,
+                                      _stream(stream))
+            # done with `tiles` and the inputs, as slg_filter is on return
+            (stream or torch.cuda.current_stream()).synchronize()
+        if rc != 0:
             raise SlgError(rc, "slg_filter")
-        out = _outputs(cnt.value, not weights, i.device)
+        return oi[:p], oj[:p], (ow[:p] if ow is not None else None)
     oi, oj, ow = out
     cnt = ctypes.c_int64(0)
     rc = load().slg_filter(i.data_ptr(), j.data_ptr(), w.data_ptr(), n, int(s), oi.data_ptr(),

@@ -1396,8 +1396,42 @@ int slg_filter(const int32_t *in_i, const int32_t *in_j, const int32_t *in_w, in
   SLG_TRY(cudaStreamSynchronize(st));
   *n_pairs = total;
   if (total > capacity) return SLG_ERR_CAPACITY;
-  if (total > 0) SLG_TRY(launch_keep_write(in_i, in_j, in_w, n, s, tile, out_i, out_j, out_w, st));
+  if (total > 0)
+    SLG_TRY(launch_keep_write(in_i, in_j, in_w, n, s, tile, out_i, out_j, out_w, capacity, st));
   SLG_TRY(cudaStreamSynchronize(st));
+  return SLG_OK;
+}
+
+int slg_filter_tiles(int64_t n, int64_t *n_tiles) {
+  if (n < 0 || !n_tiles) return SLG_ERR_INVALID;
+  *n_tiles = keep_tiles(n) + 1;
+  return SLG_OK;
+}
+
+int slg_filter_count(const int32_t *in_w, int64_t n, int32_t s, int64_t *tiles,
+                     int64_t *n_pairs, void *stream) {
+  if (!n_pairs || n < 0 || s < 1 || !tiles || (n > 0 && !in_w)) return SLG_ERR_INVALID;
+  *n_pairs = 0;
+  if (n == 0) return SLG_OK;
+  cudaStream_t st = (cudaStream_t)stream;
+  SLG_TRY(launch_keep_count(in_w, n, s, reinterpret_cast<long long *>(tiles), st));
+  long long total = 0;
+  SLG_TRY(cudaMemcpyAsync(&total, tiles + keep_tiles(n), sizeof(long long),
+                          cudaMemcpyDeviceToHost, st));
+  SLG_TRY(cudaStreamSynchronize(st));
+  *n_pairs = total;
+  return SLG_OK;
+}
+
+int slg_filter_write(const int32_t *in_i, const int32_t *in_j, const int32_t *in_w, int64_t n,
+                     int32_t s, const int64_t *tiles, int32_t *out_i, int32_t *out_j,
+                     int32_t *out_w, int64_t capacity, void *stream) {
+  if (n < 0 || s < 1 || capacity < 0 || !tiles || (n > 0 && (!in_i || !in_j || !in_w)) ||
+      (capacity > 0 && (!out_i || !out_j)))
+    return SLG_ERR_INVALID;
+  if (n == 0 || capacity == 0) return SLG_OK;
+  SLG_TRY(launch_keep_write(in_i, in_j, in_w, n, s, reinterpret_cast<const long long *>(tiles),
+                            out_i, out_j, out_w, capacity, (cudaStream_t)stream));
   return SLG_OK;
 }
 
@@ -1423,7 +1457,14 @@ int slg_build_sweep(const slg_hypergraph *h, const int32_t *s, int32_t count, ui
   const int64_t n0 = n_pairs[k0];
   cudaStream_t st = (cudaStream_t)stream;
   int result = SLG_OK;
-  for (int32_t k = 0; k < count; ++k) {
+  // thresholds in ascending order: each list is filtered from the last one
+  // that was written with its weights (L_s'' of L_s' for s' <= s''), which is
+  // far shorter than the first
+  std::vector<int32_t> order((size_t)count);
+  for (int32_t k = 0; k < count; ++k) order[k] = k;
+  std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t b) { return s[a] < s[b]; });
+  int32_t from = k0;
+  for (int32_t k : order) {
     if (k == k0) continue;
     if (s[k] == s[k0]) {  // the same list
       n_pairs[k] = n0;
@@ -1441,10 +1482,11 @@ int slg_build_sweep(const slg_hypergraph *h, const int32_t *s, int32_t count, ui
       }
       continue;
     }
-    rc = slg_filter(out_i[k0], out_j[k0], out_w[k0], n0, s[k], out_i[k], out_j[k], out_w[k],
-                    capacity[k], &n_pairs[k], stream);
+    rc = slg_filter(out_i[from], out_j[from], out_w[from], n_pairs[from], s[k], out_i[k], out_j[k],
+                    out_w[k], capacity[k], &n_pairs[k], stream);
     if (rc == SLG_ERR_CAPACITY) result = rc;
     else if (rc != SLG_OK) return rc;
+    else if (out_w[k]) from = k;
   }
   SLG_TRY(cudaStreamSynchronize(st));
   t_stats = base_stats;

@@ -635,7 +635,8 @@ cudaError_t launch_keep_count(const int32_t *w, int64_t n, int32_t s, long long 
                               cudaStream_t st);
 cudaError_t launch_keep_write(const int32_t *in_i, const int32_t *in_j, const int32_t *in_w,
                               int64_t n, int32_t s, const long long *tile, int32_t *out_i,
-                              int32_t *out_j, int32_t *out_w, cudaStream_t st);
+                              int32_t *out_j, int32_t *out_w, int64_t capacity,
+                              cudaStream_t st);
 
 // After the edge list (slg_post.cu): pair checks, ID squeezing, adjacency,
 // components.

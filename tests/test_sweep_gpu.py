@@ -143,3 +143,21 @@ def test_sweep_with_relabel_and_tensor():
             got = slg.build_sweep(dh, [2, 8, 32], dual=dual, **kw)
             for s, t in zip([2, 8, 32], got):
                 assert np.array_equal(as_np(t), want(h, s, dual)), (dual, kw, s)
+
+
+@pytest.mark.parametrize("size", [31, 1023, 1025, 16_383, 16_385, 70_000])
+@pytest.mark.parametrize("s", [1, 3, 6, 7])
+def test_filter_tiles(size, s):
+    # warps of 1,024 triples in tiles of 16,384: remainders, all kept, none kept
+    w = (torch.arange(size, dtype=torch.int32, device="cuda") * 5) % 7
+    i = torch.arange(size, dtype=torch.int32, device="cuda")
+    idx = torch.nonzero(w >= s)[:, 0].int()
+    oi, oj, ow = slg.filter_pairs(i, i + 1, w, s)
+    assert torch.equal(oi, idx) and torch.equal(oj, idx + 1)
+    assert torch.equal(ow, w[idx.long()])
+    out = slg.alloc_outputs(size)
+    a, b, c = slg.filter_pairs(i, i + 1, w, s, out=out)
+    assert torch.equal(a, idx) and torch.equal(b, idx + 1) and torch.equal(c, ow)
+    # an offset of one entry: no alignment is assumed
+    a, b, c = slg.filter_pairs(i[1:], i[1:] + 1, w[1:], s)
+    assert torch.equal(a, idx[idx > 0])
