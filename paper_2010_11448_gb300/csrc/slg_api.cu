@@ -1493,20 +1493,6 @@ int slg_build_sweep(const slg_hypergraph *h, const int32_t *s, int32_t count, ui
   return result;
 }
 
-// Device check of a pair list; returns SLG_OK or SLG_ERR_INVALID (synchronises).
-static int check_pairs(const int32_t *a, const int32_t *b, int64_t n, int32_t R, int canonical,
-                       Pool &pool, cudaStream_t st) {
-  if (n == 0) return SLG_OK;
-  int32_t *err = nullptr;
-  SLG_TRY(pool.get(&err, 1));
-  SLG_TRY(cudaMemsetAsync(err, 0, sizeof(int32_t), st));
-  SLG_TRY(launch_check_pairs(a, b, n, R, canonical, err, st));
-  int32_t h = 0;
-  SLG_TRY(cudaMemcpyAsync(&h, err, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-  SLG_TRY(cudaStreamSynchronize(st));
-  return h ? SLG_ERR_INVALID : SLG_OK;
-}
-
 int slg_squeeze(const int32_t *in_i, const int32_t *in_j, int64_t n, int32_t R, int32_t *out_i,
                 int32_t *out_j, int32_t *old_of_new, int32_t *n_ids, void *stream) {
   if (!n_ids || n < 0 || R < 0 || (n > 0 && (!in_i || !in_j || !out_i || !out_j)) ||
@@ -1514,20 +1500,25 @@ int slg_squeeze(const int32_t *in_i, const int32_t *in_j, int64_t n, int32_t R, 
     return SLG_ERR_INVALID;
   cudaStream_t st = (cudaStream_t)stream;
   Pool pool(st);
-  int rc = check_pairs(in_i, in_j, n, R, 0, pool, st);
-  if (rc) return rc;
-  int32_t *mark, *rank, *tile;
-  SLG_TRY(pool.get(&mark, (size_t)R + 1));
-  SLG_TRY(pool.get(&rank, (size_t)R + 1));
-  SLG_TRY(pool.get(&tile, (size_t)xscan_tiles((int64_t)R + 1) + 1));
-  SLG_TRY(cudaMemsetAsync(mark, 0, ((size_t)R + 1) * sizeof(int32_t), st));
-  SLG_TRY(launch_mark(in_i, in_j, n, mark, st));
-  SLG_TRY(launch_xscan(mark, rank, (int64_t)R + 1, tile, st));
-  SLG_TRY(launch_squeeze(in_i, in_j, n, R, mark, rank, out_i, out_j, old_of_new, st));
-  int32_t ids = 0;
-  SLG_TRY(cudaMemcpyAsync(&ids, rank + R, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+  const size_t words = ((size_t)R + 31) / 32;
+  uint32_t *bits;  // the map, then the error flag
+  int32_t *cnt, *rank, *tile;
+  int64_t *word;
+  SLG_TRY(pool.get(&bits, words + 1));
+  SLG_TRY(pool.get(&cnt, words + 1));
+  SLG_TRY(pool.get(&rank, words + 2));  // the flag is copied behind the total
+  SLG_TRY(pool.get(&tile, (size_t)xscan_tiles((int64_t)words + 1) + 1));
+  SLG_TRY(pool.get(&word, words));
+  int32_t *err = reinterpret_cast<int32_t *>(bits + words);
+  SLG_TRY(cudaMemsetAsync(bits, 0, (words + 1) * sizeof(uint32_t), st));
+  SLG_TRY(launch_squeeze(in_i, in_j, n, R, bits, cnt, rank, word, tile, out_i, out_j, old_of_new,
+                         err, st));
+  SLG_TRY(cudaMemcpyAsync(rank + words + 1, err, sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
+  int32_t got[2] = {0, 0};
+  SLG_TRY(cudaMemcpyAsync(got, rank + words, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
   SLG_TRY(cudaStreamSynchronize(st));
-  *n_ids = ids;
+  if (got[1]) return SLG_ERR_INVALID;
+  *n_ids = got[0];
   return SLG_OK;
 }
 
@@ -1538,31 +1529,31 @@ int slg_adjacency(const int32_t *in_i, const int32_t *in_j, const int32_t *in_w,
     return SLG_ERR_INVALID;
   cudaStream_t st = (cudaStream_t)stream;
   Pool pool(st);
-  int rc = check_pairs(in_i, in_j, n, V, 1, pool, st);
-  if (rc) return rc;
-  int32_t *up, *lo;
-  SLG_TRY(pool.get(&up, (size_t)V + 1));
-  SLG_TRY(pool.get(&lo, (size_t)V + 1));
-  SLG_TRY(cudaMemsetAsync(up, 0, ((size_t)V + 1) * sizeof(int32_t), st));
-  SLG_TRY(cudaMemsetAsync(lo, 0, ((size_t)V + 1) * sizeof(int32_t), st));
-  long long *off = reinterpret_cast<long long *>(adj_off);
-  SLG_TRY(launch_adjacency_offsets(in_i, in_j, n, V, up, lo, off, st));
+  int32_t *ends, *U, *L, *tile, *hist = nullptr;
+  const size_t v1 = (size_t)V + 1;
+  SLG_TRY(pool.get(&ends, 2 * v1 + 1));  // segment starts and ends, the error flag
+  SLG_TRY(pool.get(&U, v1));
+  SLG_TRY(pool.get(&L, v1));
+  SLG_TRY(pool.get(&tile, (size_t)xscan_tiles((int64_t)v1) + 1));
+  int32_t *err = ends + 2 * v1;
+  SLG_TRY(cudaMemsetAsync(ends, 0, (2 * v1 + 1) * sizeof(int32_t), st));
+  uint32_t *key[2] = {nullptr, nullptr};
+  int32_t *vi[2] = {nullptr, nullptr}, *vw[2] = {nullptr, nullptr};
   if (n > 0) {
-    long long *first, *lfirst;
-    uint32_t *keys, *keys_tmp;
-    int32_t *pos, *pos_tmp, *hist;
-    SLG_TRY(pool.get(&first, (size_t)V + 1));
-    SLG_TRY(pool.get(&lfirst, (size_t)V + 1));
-    SLG_TRY(pool.get(&keys, (size_t)n));
-    SLG_TRY(pool.get(&keys_tmp, (size_t)n));
-    SLG_TRY(pool.get(&pos, (size_t)n));
-    SLG_TRY(pool.get(&pos_tmp, (size_t)n));
-    SLG_TRY(pool.get(&hist, radix_sort_scratch_ints(n)));
-    SLG_TRY(launch_adjacency_fill(in_i, in_j, in_w, n, V, off, lo, first, lfirst, keys,
-                                  keys_tmp, pos, pos_tmp, hist, adj, adj_w, st));
+    const int passes = adjacency_passes(V);
+    for (int q = 0; q < 2; ++q) {
+      if (passes > 1 || q == 1) SLG_TRY(pool.get(&key[q], (size_t)n));
+      if (passes > q + 1) SLG_TRY(pool.get(&vi[q], (size_t)n));
+      if (passes > q + 1 && adj_w) SLG_TRY(pool.get(&vw[q], (size_t)n));
+    }
+    SLG_TRY(pool.get(&hist, adjacency_scratch_ints(n)));
   }
+  SLG_TRY(launch_adjacency(in_i, in_j, in_w, n, V, ends, ends + v1, U, L, tile, key, vi, vw, hist,
+                           reinterpret_cast<long long *>(adj_off), adj, adj_w, err, st));
+  int32_t bad = 0;
+  SLG_TRY(cudaMemcpyAsync(&bad, err, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
   SLG_TRY(cudaStreamSynchronize(st));
-  return SLG_OK;
+  return bad ? SLG_ERR_INVALID : SLG_OK;
 }
 
 int slg_components(const int32_t *in_i, const int32_t *in_j, int64_t n, int32_t R,
@@ -1572,25 +1563,20 @@ int slg_components(const int32_t *in_i, const int32_t *in_j, int64_t n, int32_t 
     return SLG_ERR_INVALID;
   cudaStream_t st = (cudaStream_t)stream;
   Pool pool(st);
-  int rc = check_pairs(in_i, in_j, n, R, 0, pool, st);
-  if (rc) return rc;
-  int32_t *mark, *err;
+  // the count, the error flag, the roots with others
   unsigned long long *cnt;
-  SLG_TRY(pool.get(&mark, (size_t)R + 1));
-  SLG_TRY(pool.get(&err, 1));
-  SLG_TRY(pool.get(&cnt, 1));
-  SLG_TRY(cudaMemsetAsync(mark, 0, ((size_t)R + 1) * sizeof(int32_t), st));
-  SLG_TRY(cudaMemsetAsync(err, 0, sizeof(int32_t), st));
-  SLG_TRY(cudaMemsetAsync(cnt, 0, sizeof(unsigned long long), st));
-  SLG_TRY(launch_mark(in_i, in_j, n, mark, st));
-  SLG_TRY(launch_components(in_i, in_j, n, R, labels, mark, cnt, err, st));
-  unsigned long long hc = 0;
-  int32_t he = 0;
-  SLG_TRY(cudaMemcpyAsync(&hc, cnt, sizeof(hc), cudaMemcpyDeviceToHost, st));
-  SLG_TRY(cudaMemcpyAsync(&he, err, sizeof(he), cudaMemcpyDeviceToHost, st));
+  SLG_TRY(pool.get(&cnt, 2 + ((size_t)R + 1) / 2));
+  int32_t *err = reinterpret_cast<int32_t *>(cnt + 1);
+  int32_t *child = reinterpret_cast<int32_t *>(cnt + 2);
+  SLG_TRY(cudaMemsetAsync(cnt, 0, (2 + ((size_t)R + 1) / 2) * sizeof(unsigned long long), st));
+  SLG_TRY(launch_components(in_i, in_j, n, R, labels, child, cnt, err, st));
+  unsigned long long got[2] = {0, 0};
+  SLG_TRY(cudaMemcpyAsync(got, cnt, sizeof(got), cudaMemcpyDeviceToHost, st));
   SLG_TRY(cudaStreamSynchronize(st));
-  if (he) return SLG_ERR_TIMEOUT;  // a bounded loop gave up (not expected)
-  *n_components = (int64_t)hc;
+  const int32_t bad = (int32_t)got[1];
+  if (bad == 1) return SLG_ERR_INVALID;
+  if (bad) return SLG_ERR_TIMEOUT;  // a bounded loop gave up (not expected)
+  *n_components = (int64_t)got[0];
   return SLG_OK;
 }
 

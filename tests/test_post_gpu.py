@@ -91,3 +91,38 @@ def test_empty_and_invalid():
     assert lib.slg_adjacency(a.data_ptr(), b.data_ptr(), None, 2, 8, off.data_ptr(),
                              adj.data_ptr(), None, None) == 0
     assert np.array_equal(np_(adj), [3, 2, 1, 0])
+
+
+def random_list(V, n, seed):
+    """A canonical list of about n distinct pairs over V ids."""
+    rng = np.random.default_rng(seed)
+    i = rng.integers(0, V - 1, 2 * n)
+    j = i + 1 + (rng.random(2 * n) ** 3 * (V - 1 - i)).astype(np.int64)
+    key = np.unique(i * V + np.minimum(j, V - 1))
+    key = np.sort(rng.permutation(key)[:n])
+    w = rng.integers(1, 1000, key.shape[0]).astype(np.int32)
+    return (key // V).astype(np.int32), (key % V).astype(np.int32), w
+
+
+# ids of 1, 10, 11, 20 and 21 bits (one, two and three digit passes), lists of
+# one warp, one tile (8,192 pairs) and its edges, id maps above and below the
+# 1.6 million ids of the shared one
+@pytest.mark.parametrize("V,n", [(2, 1), (3, 3), (1_024, 8_192), (1_025, 8_193), (70_000, 20_001),
+                                 (1_048_576, 100_000), (1_048_577, 70_001), (1_700_000, 65_536),
+                                 (9_000_000, 40_000)])
+def test_sizes_against_oracle(V, n):
+    i, j, w = random_list(V, n, V + n)
+    t = [torch.from_numpy(x).cuda() for x in (i, j, w)]
+    si, sj, old = slg.squeeze(t[0], t[1], V)
+    wi, wj, wold = oracle.squeeze(i, j, V)
+    assert np.array_equal(np_(si), wi) and np.array_equal(np_(sj), wj)
+    assert np.array_equal(np_(old), wold)
+    off, adj, adj_w = slg.adjacency(*t, V)
+    woff, wadj, wadjw = oracle.adjacency(i, j, w, V)
+    assert np.array_equal(np_(off), woff) and np.array_equal(np_(adj), wadj)
+    assert np.array_equal(np_(adj_w), wadjw)
+    off, adj, none = slg.adjacency(*t, V, weights=False)
+    assert none is None and np.array_equal(np_(adj), wadj)
+    lab, k = slg.components(t[0], t[1], V)
+    wlab, wk = oracle.components(i, j, V)
+    assert np.array_equal(np_(lab), wlab) and k == wk
