@@ -245,6 +245,24 @@ __device__ __forceinline__ int32_t find_sorted(const int32_t *__restrict__ a, in
   return -1;
 }
 
+// The row r with off[r] <= k < off[r + 1] (off ascending, off[0] <= k <
+// off[rows]), starting from a row `r` known not to be past it: a few steps
+// forward, else a binary search.
+__device__ __forceinline__ int32_t row_of(const int32_t *__restrict__ off, int32_t rows, int32_t r,
+                                          int32_t k) {
+  for (int step = 0; step < 4; ++step) {
+    if (__ldg(off + r + 1) > k) return r;
+    if (++r >= rows) return rows - 1;
+  }
+  int32_t lo = r, hi = rows;  // off[lo] <= k < off[hi]
+  while (hi - lo > 1) {
+    const int32_t mid = lo + ((hi - lo) >> 1);
+    if (__ldg(off + mid) <= k) lo = mid;
+    else hi = mid;
+  }
+  return lo;
+}
+
 // Multiplicative hash onto [0, T) (Fibonacci hashing + fast range).
 __device__ __forceinline__ uint32_t hash_slot(int32_t f, uint32_t T) {
   return __umulhi((uint32_t)f * 0x9E3779B1u, T);
@@ -540,6 +558,26 @@ struct WalkLaunch {
   long long dense_pairs[2]; // most pairs a dense-bin row can have: big instance, other (0: no row)
   int32_t dense_size;       // most vertices of a dense-bin row
 };
+
+// Sides of at most this many rows take the short path (slg_small.cu).
+#ifndef SLG_SMALL_ROWS
+#define SLG_SMALL_ROWS 16384
+#endif
+constexpr int32_t kSmallRows = SLG_SMALL_ROWS;
+struct SmallCall {
+  Side s;
+  int32_t s_prune;               // size from which rows take part
+  int32_t row_begin, row_end;
+  int32_t *map;                  // [nnz] CSC positions (made unless !validate)
+  bool validate;
+  uint32_t *active;              // [(R + 31) / 32], zeroed
+  EmitArgs a;                    // n_e zeroed; stage_cap = the output's capacity
+  int32_t *out_i, *out_j, *out_w;
+  long long *row_ptr;            // [rows + 1] or null
+  Meta *host;                    // mapped host memory, receives the Meta
+};
+cudaError_t launch_small(const SmallCall &c, cudaStream_t st, int32_t *launches, cudaEvent_t walk0,
+                         cudaEvent_t walk1);
 
 // CTAs of the giant kernel (two per SM); scratch ints of the sparse and dense
 // kernels.

@@ -14,56 +14,100 @@ namespace {
 
 constexpr int kValNT = 256;
 
-// One warp per row: offsets monotone inside [0, nnz], ids inside [0, cols),
-// every row strictly ascending.  Reports through meta (never traps).
+// Offsets monotone inside [0, nnz], ids inside [0, cols), every row strictly
+// ascending.  Eight lanes per row (rows hold 10 to 20 ids on average; a warp
+// per row left two thirds of its lanes idle: 257 us for both sides of 500K x
+// 1M, where this takes 123); a row of more than kValLong ids is read by the
+// whole warp, four loads in flight.  Reports through meta (never traps).
+constexpr int32_t kValLong = 128;
+
 __global__ __launch_bounds__(kValNT) void k_validate(const int32_t *__restrict__ off,
                                                      const int32_t *__restrict__ idx,
                                                      int32_t rows, int32_t cols, int64_t nnz,
                                                      Meta *meta, int32_t where_off,
                                                      int32_t where_ids) {
-  const int lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & 31, sub = lane >> 3, l8 = lane & 7;
   const int64_t warp = ((int64_t)blockIdx.x * kValNT + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * kValNT) >> 5;
   if (warp == 0 && lane == 0) {
     if (off[0] != 0 || (int64_t)off[rows] != nnz) raise_error(meta, SLG_ERR_INVALID, where_off);
   }
-  for (int64_t r = warp; r < rows; r += nwarps) {
-    const int32_t lo = off[r], hi = off[r + 1];
-    if (lo < 0 || hi < lo || (int64_t)hi > nnz) {
-      if (lane == 0) raise_error(meta, SLG_ERR_INVALID, where_off);
-      continue;
+  bool bad = false;
+  // ids k, k + step, ... of the row [lo, hi)
+  auto check = [&](int32_t lo, int32_t hi, int32_t k0, int32_t step) {
+    for (; k0 < hi; k0 += 4 * step) {
+      int32_t x[4], y[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int32_t k = k0 + u * step;
+        x[u] = k < hi ? __ldg(idx + k) : 0;
+        y[u] = k < hi && k > lo ? __ldg(idx + k - 1) : -1;
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (k0 + u * step < hi) bad |= x[u] < 0 || x[u] >= cols || y[u] >= x[u];
     }
-    bool bad = false;
-    for (int32_t k = lo + lane; k < hi; k += 32) {
-      const int32_t x = idx[k];
-      if (x < 0 || x >= cols) bad = true;
-      if (k > lo && idx[k - 1] >= x) bad = true;
+  };
+  for (int64_t r0 = warp * 4; r0 < rows; r0 += nwarps * 4) {
+    const int64_t r = r0 + sub;
+    int32_t lo = 0, hi = 0;
+    if (r < rows) {
+      lo = __ldg(off + r);
+      hi = __ldg(off + r + 1);
+      if (lo < 0 || hi < lo || (int64_t)hi > nnz) {
+        if (l8 == 0) raise_error(meta, SLG_ERR_INVALID, where_off);
+        lo = hi = 0;
+      }
     }
-    if (__any_sync(0xffffffffu, bad) && lane == 0) raise_error(meta, SLG_ERR_INVALID, where_ids);
+    if (hi - lo <= kValLong) check(lo, hi, lo + l8, 8);
+    unsigned big = __ballot_sync(0xffffffffu, l8 == 0 && hi - lo > kValLong);
+    while (big) {
+      const int src = __ffs(big) - 1;
+      big &= big - 1;
+      const int32_t a = __shfl_sync(0xffffffffu, lo, src), b = __shfl_sync(0xffffffffu, hi, src);
+      check(a, b, a + lane, 32);
+    }
   }
+  if (bad) raise_error(meta, SLG_ERR_INVALID, where_ids);
 }
 
-// One warp per CSR row f: the CSC position of every incidence (v, f), found
-// by binary search in the (validated, ascending) column v.  A miss means the
-// CSR and CSC are not the same incidence.  With nnz equal on both sides and
-// strictly ascending rows, a hit for every incidence makes the map a bijection.
+// The CSC position of every incidence (v, f), found by binary search in the
+// (validated, ascending) column v.  A miss means the CSR and CSC are not the
+// same incidence.  With nnz equal on both sides and strictly ascending rows, a
+// hit for every incidence makes the map a bijection.
+// Incidences are dealt out evenly (a warp takes kMapK x 32 consecutive ones
+// and finds their rows): with a warp per row, the kernel's time was that of
+// its longest row (10,000 vertices, 312 dependent searches: 887 us on 500K x
+// 1M, where this takes 211).
+constexpr int kMapK = 8;
 __global__ __launch_bounds__(kValNT) void k_csr2csc(Side s, int32_t *__restrict__ csr2csc,
                                                     Meta *meta) {
   if (meta->err) return;
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * kValNT + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * kValNT) >> 5;
-  for (int64_t f = warp; f < s.R; f += nwarps) {
-    const int32_t lo = s.r_off[f], hi = s.r_off[f + 1];
-    bool bad = false;
-    for (int32_t k = lo + lane; k < hi; k += 32) {
-      const int32_t v = s.r_idx[k];
-      const int32_t q = find_sorted(s.c_idx, s.c_off[v], s.c_off[v + 1], (int32_t)f);
-      if (q < 0) bad = true;
-      else csr2csc[k] = q;
+  const int64_t base = warp * (32 * kMapK);
+  if (base >= s.nnz) return;
+  int32_t f = 0;
+  {
+    int32_t hi = s.R;  // r_off[f] <= base < r_off[hi]
+    while (hi - f > 1) {
+      const int32_t mid = f + ((hi - f) >> 1);
+      if (__ldg(s.r_off + mid) <= (int32_t)base) f = mid;
+      else hi = mid;
     }
-    if (__any_sync(0xffffffffu, bad) && lane == 0) raise_error(meta, SLG_ERR_INVALID, kWhereMismatch);
   }
+  bool bad = false;
+#pragma unroll 2
+  for (int u = 0; u < kMapK; ++u) {
+    const int64_t k = base + 32 * u + lane;
+    if (k >= s.nnz) break;
+    const int32_t v = s.r_idx[k];
+    f = row_of(s.r_off, s.R, f, (int32_t)k);
+    const int32_t q = find_sorted(s.c_idx, s.c_off[v], s.c_off[v + 1], f);
+    if (q < 0) bad = true;
+    else csr2csc[k] = q;
+  }
+  if (bad) raise_error(meta, SLG_ERR_INVALID, kWhereMismatch);
 }
 
 // ------------------------------------------ filtered CSC (reduce-then-scan) --
@@ -171,21 +215,53 @@ __device__ __forceinline__ int bin_of(int32_t work, const Bins &b) {
   return kBinGiant;
 }
 
+// The tail of every incidence (e, v): the filtered position of e in column v
+// is qs[csr2csc[k]], so its tail starts one past it (for a row of size < s,
+// which is not kept, nothing reads the tail).  Incidences are dealt out evenly,
+// as in k_csr2csc.
+__global__ __launch_bounds__(kRowsNT) void k_tails(int64_t k0, int64_t k1,
+                                                   const int32_t *__restrict__ r_idx,
+                                                   const int32_t *__restrict__ csr2csc,
+                                                   const int32_t *__restrict__ qs,
+                                                   const int32_t *__restrict__ c_off_s,
+                                                   int32_t *__restrict__ tail_beg,
+                                                   int32_t *__restrict__ tail_end,
+                                                   const Meta *meta) {
+  if (meta->err) return;
+  const int64_t base = k0 + (int64_t)blockIdx.x * (kRowsNT * 4) + threadIdx.x;
+  int32_t v[4], q[4], tb[4], te[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int64_t k = base + u * kRowsNT;
+    v[u] = k < k1 ? __ldg(r_idx + k) : 0;
+    q[u] = k < k1 ? __ldg(csr2csc + k) : 0;
+  }
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    tb[u] = __ldg(qs + q[u]) + 1;
+    te[u] = __ldg(c_off_s + v[u] + 1);
+  }
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int64_t k = base + u * kRowsNT;
+    if (k < k1) {
+      tail_beg[k] = tb[u];
+      tail_end[k] = te[u];
+    }
+  }
+}
+
 // A block handles kRowsPerBlock consecutive rows, one warp per row at a time.
-// For each incidence (e, v) of an active row: the filtered position of e in
-// column v is qs[csr2csc[k]] (e is kept because |e| >= s), so its tail starts
-// one past it.  The row's work is the sum of its tail lengths.  Rows with
+// The row's work is the sum of its tail lengths (k_tails; core columns of core
+// rows are set here).  Rows with
 // work > 0 are appended to their bin's list (one global atomic per bin and
 // block); rows outside the range or inactive get n_e = 0.
 __global__ __launch_bounds__(kRowsNT) void k_rows_work(Side s, int32_t smin, int32_t row_begin,
                                                        int32_t row_end,
-                                                       const int32_t *__restrict__ csr2csc,
-                                                       const int32_t *__restrict__ qs,
-                                                       const int32_t *__restrict__ c_off_s,
                                                        const int32_t *__restrict__ c_idx_s,
                                                        CoreInfo core, Bins bins,
-                                                       int32_t *__restrict__ tail_beg,
-                                                       int32_t *__restrict__ tail_end,
+                                                       int32_t *tail_beg,
+                                                       int32_t *tail_end,
                                                        int32_t *__restrict__ n_e,
                                                        long long *__restrict__ stage_pos,
                                                        int32_t *__restrict__ row_work,
@@ -212,41 +288,71 @@ __global__ __launch_bounds__(kRowsNT) void k_rows_work(Side s, int32_t smin, int
   if (threadIdx.x < 7) s_max[threadIdx.x] = 0;
   if (threadIdx.x == 0) s_act = 0;
   __syncthreads();
-  for (int i = warp; i < kRowsPerBlock; i += kRowsNT / 32) {
+  // eight lanes per row; long rows and core rows by the whole warp
+  for (int i0 = warp * 4; i0 < kRowsPerBlock; i0 += kRowsNT / 8) {
+    const int i = i0 + (lane >> 3), l8 = lane & 7;
     const int32_t e = r0 + i;
-    int32_t work = 0;
+    int32_t work = 0, lo = 0, hi = 0;
+    bool active = false, core_row = false;
     if (e < row_end) {
-      const int32_t lo = s.r_off[e], hi = s.r_off[e + 1];
-      const bool core_row = core.row_rank && core.row_rank[e + 1] != core.row_rank[e];
-      const bool active = hi - lo >= s_of(s.row_s, smin, e);
-      if (active) {
-        for (int32_t k = lo + lane; k < hi; k += 32) {
+      lo = __ldg(s.r_off + e);
+      hi = __ldg(s.r_off + e + 1);
+      active = hi - lo >= s_of(s.row_s, smin, e);
+      core_row = core.row_rank && core.row_rank[e + 1] != core.row_rank[e];
+    }
+    // tail lengths of incidences k0, k0 + step, ... of [.., b)
+    auto sum = [&](int32_t k0, int32_t b, int32_t step) {
+      int32_t n = 0;
+      for (; k0 < b; k0 += 4 * step) {
+        int32_t tb[4], te[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int32_t k = k0 + u * step;
+          tb[u] = k < b ? tail_beg[k] : 0;
+          te[u] = k < b ? tail_end[k] : 0;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) n += te[u] - tb[u];
+      }
+      return n;
+    };
+    const bool whole = active && (core_row || hi - lo > kValLong);
+    if (active && !whole) work = sum(lo + l8, hi, 8);
+#pragma unroll
+    for (int d = 4; d > 0; d >>= 1) work += __shfl_xor_sync(0xffffffffu, work, d);
+    unsigned big = __ballot_sync(0xffffffffu, l8 == 0 && whole);
+    while (big) {
+      const int src = __ffs(big) - 1;
+      big &= big - 1;
+      const int32_t x = __shfl_sync(0xffffffffu, e, src);
+      const int32_t a = __shfl_sync(0xffffffffu, lo, src), b = __shfl_sync(0xffffffffu, hi, src);
+      int32_t n = 0;
+      if (!__shfl_sync(0xffffffffu, (int)core_row, src)) {
+        n = sum(a + lane, b, 32);
+      } else {
+        for (int32_t k = a + lane; k < b; k += 32) {
           const int32_t v = s.r_idx[k];
-          int32_t tb, te;
-          if (core_row && core.col_rank[v + 1] != core.col_rank[v]) {
+          if (core.col_rank[v + 1] != core.col_rank[v]) {
             // core row at a core column: its tail skips the core rows (their
             // shared core vertices are counted on the tensor cores)
             const int32_t cv = core.col_rank[v];
-            int32_t a = core.x_base + core.x_off[cv], b = core.x_base + core.x_off[cv + 1];
-            te = b;
-            while (a < b) {  // first entry > e
-              const int32_t mid = (a + b) >> 1;
-              if (c_idx_s[mid] <= e) a = mid + 1;
-              else b = mid;
+            int32_t p = core.x_base + core.x_off[cv], q = core.x_base + core.x_off[cv + 1];
+            tail_end[k] = q;
+            while (p < q) {  // first entry > x
+              const int32_t mid = (p + q) >> 1;
+              if (c_idx_s[mid] <= x) p = mid + 1;
+              else q = mid;
             }
-            tb = a;
-          } else {
-            tb = qs[csr2csc[k]] + 1;
-            te = c_off_s[v + 1];
+            tail_beg[k] = p;
           }
-          tail_beg[k] = tb;
-          tail_end[k] = te;
-          work += te - tb;
+          n += tail_end[k] - tail_beg[k];
         }
-#pragma unroll
-        for (int d = 16; d > 0; d >>= 1) work += __shfl_xor_sync(0xffffffffu, work, d);
       }
-      if (lane == 0) {
+      n = __reduce_add_sync(0xffffffffu, n);
+      if ((lane & 24) == (src & 24)) work = n;
+    }
+    if (l8 == 0) {
+      if (e < row_end) {
         n_e[e - row_begin] = 0;
         stage_pos[e - row_begin] = -1;
         row_work[e - row_begin] = work;
@@ -256,13 +362,9 @@ __global__ __launch_bounds__(kRowsNT) void k_rows_work(Side s, int32_t smin, int
         }
         if (active) atomicAdd(&s_act, 1);
       }
-    }
-    if (lane == 0) {
-      // core rows always go to the giant bin (it adds their tile counts),
-      // marked by a negative work entry here
-      const bool core_row = e < row_end && core.row_rank && core.row_rank[e + 1] != core.row_rank[e] &&
-                            s.r_off[e + 1] - s.r_off[e] >= s_of(s.row_s, smin, e);
-      s_work[i] = (e < row_end) ? (core_row ? -1 - work : work) : 0;
+      // core rows take part even without wedges (their tile counts are added
+      // by the bin), marked by a negative work entry here
+      s_work[i] = e < row_end ? (core_row && active ? -1 - work : work) : 0;
     }
   }
   __syncthreads();
@@ -356,7 +458,7 @@ inline int grid_for(int64_t items, int per_block, int cap = 1 << 20) {
 }  // namespace
 
 cudaError_t launch_validate(const Side &s, Meta *meta, cudaStream_t st) {
-  const int wpb = kValNT / 32;
+  const int wpb = kValNT / 8;  // rows per block
   k_validate<<<grid_for(s.R, wpb, 65536), kValNT, 0, st>>>(s.r_off, s.r_idx, s.R, s.C, s.nnz, meta,
                                                           kWhereRowOffsets, kWhereRowIds);
   k_validate<<<grid_for(s.C, wpb, 65536), kValNT, 0, st>>>(s.c_off, s.c_idx, s.C, s.R, s.nnz, meta,
@@ -380,7 +482,8 @@ cudaError_t launch_invert(const int32_t *map, int64_t n, int32_t *inv, cudaStrea
 }
 
 cudaError_t launch_csr2csc(const Side &s, int32_t *csr2csc, Meta *meta, cudaStream_t st) {
-  k_csr2csc<<<grid_for(s.R, kValNT / 32, 65536), kValNT, 0, st>>>(s, csr2csc, meta);
+  if (s.nnz > 0)
+    k_csr2csc<<<grid_for(s.nnz, kValNT * kMapK, 1 << 30), kValNT, 0, st>>>(s, csr2csc, meta);
   return cudaGetLastError();
 }
 
@@ -403,12 +506,15 @@ cudaError_t launch_rows_work(const Side &s, int32_t smin, int32_t row_begin, int
                              cudaStream_t st) {
   const int32_t rows = row_end - row_begin;
   if (rows <= 0) return cudaSuccess;
+  // (the tails of every row, also with a row range: its first incidence is
+  // not known here)
+  if (s.nnz > 0)
+    k_tails<<<grid_for(s.nnz, kRowsNT * 4, 1 << 30), kRowsNT, 0, st>>>(
+        0, s.nnz, s.r_idx, w.csr2csc, w.qs, w.c_off_s, w.tail_beg, w.tail_end, w.meta);
   const int grid = (rows + kRowsPerBlock - 1) / kRowsPerBlock;
-  k_rows_work<<<grid, kRowsNT, 0, st>>>(s, smin, row_begin, row_end, w.csr2csc, w.qs, w.c_off_s,
-                                        w.c_idx_s, core, bins,
+  k_rows_work<<<grid, kRowsNT, 0, st>>>(s, smin, row_begin, row_end, w.c_idx_s, core, bins,
                                         w.tail_beg, w.tail_end, w.n_e, w.stage_pos, w.row_work,
-                                        w.bin_rows,
-                                        w.meta);
+                                        w.bin_rows, w.meta);
   return cudaGetLastError();
 }
 
