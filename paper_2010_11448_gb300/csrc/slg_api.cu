@@ -484,7 +484,7 @@ int run_binned(Call &c, int64_t *result) {
     if (rcc) return rcc;
   }
   SLG_TRY(launch_rows_work(c.sd, s_prune, c.row_begin, c.row_end, w, core, t_bins, c.st));
-  c.launches += 4 + (c.rows > 0 ? 1 : 0);
+  c.launches += 4 + (c.rows > 0 ? 2 : 0);
   if (c.op == kOpWedges) {
     if (c.row_work_out)
       SLG_TRY(cudaMemcpyAsync(c.row_work_out, w.row_work, sizeof(int32_t) * (size_t)c.rows,
@@ -731,6 +731,70 @@ int run_spgemm(Call &c, int64_t *result) {
   return SLG_OK;
 }
 
+// A side of at most kSmallRows rows: three kernels, one allocation, one host
+// round trip (slg_small.cu).
+// *room false: its memory (at most 8 bytes for each of R (R - 1) / 2 pairs)
+// could not be had, nothing was done.
+int run_small(Call &c, const Prepared *pp, long long *row_ptr_out, int64_t *result, bool *room) {
+  const int64_t nnz = c.sd.nnz;
+  const bool build = c.op == kOpBuild;
+  const size_t words = ((size_t)c.sd.R + 31) / 32, rows = (size_t)c.rows;
+  auto up = [](size_t n) { return (n + 255) & ~(size_t)255; };
+  const size_t o_act = up(sizeof(Meta)), o_ne = o_act + up(words * 4);
+  const size_t o_sp = o_ne + up(rows * 4), o_map = o_sp + up(rows * 8);
+  const size_t o_j = o_map + (pp ? 0 : up((size_t)nnz * 4));
+  const int64_t most = (int64_t)c.sd.R * (c.sd.R - 1) / 2;
+  const size_t cap = build ? (size_t)std::min<int64_t>(c.capacity, most) : 0;
+  const size_t o_w = o_j + up(cap * 4), bytes = o_w + (c.unweighted ? 0 : up(cap * 4));
+  unsigned char *buf = nullptr;
+  *room = c.pool->get(&buf, bytes) == cudaSuccess;
+  if (!*room) return SLG_OK;
+  SLG_TRY(cudaMemsetAsync(buf, 0, o_sp, c.st));  // totals, active rows, pair counts
+  c.w.meta = reinterpret_cast<Meta *>(buf);
+  SmallCall s = {};
+  s.s = c.sd;
+  s.s_prune = (c.flags & SLG_NO_PRUNE) ? 1 : c.smin;
+  s.row_begin = c.row_begin;
+  s.row_end = c.row_end;
+  s.validate = !pp;
+  s.map = pp ? pp->map[(c.flags & SLG_DUAL) ? 1 : 0] : reinterpret_cast<int32_t *>(buf + o_map);
+  s.active = reinterpret_cast<uint32_t *>(buf + o_act);
+  s.a.mode = build ? kStage : kCount;
+  s.a.unweighted = c.unweighted;
+  s.a.smin = c.smin;
+  s.a.row_begin = c.row_begin;
+  s.a.n_e = reinterpret_cast<int32_t *>(buf + o_ne);
+  s.a.stage_pos = reinterpret_cast<long long *>(buf + o_sp);
+  s.a.stage_j = reinterpret_cast<int32_t *>(buf + o_j);
+  s.a.stage_w = c.unweighted ? nullptr : reinterpret_cast<int32_t *>(buf + o_w);
+  s.a.stage_cap = (long long)cap;
+  s.a.meta = c.w.meta;
+  s.out_i = c.out_i;
+  s.out_j = c.out_j;
+  s.out_w = c.out_w;
+  s.row_ptr = row_ptr_out;
+  s.host = c.meta_view;
+  const bool on = c.evs->on;
+  cudaEvent_t *ev = c.evs->ev;
+  if (on) cudaEventRecord(ev[kEvPlan], c.st);
+  SLG_TRY(launch_small(s, c.st, &c.launches, on ? ev[kEvWalk] : nullptr,
+                       on ? ev[kEvWalk + 1] : nullptr));
+  if (on) {
+    for (int b = 2; b <= kNumBins; ++b) cudaEventRecord(ev[kEvWalk + b], c.st);
+    cudaEventRecord(ev[kEvScan], c.st);
+    cudaEventRecord(ev[kEvGather0], c.st);
+    cudaEventRecord(ev[kEvGather1], c.st);
+  }
+  SLG_TRY(cudaStreamSynchronize(c.st));
+  const Meta &m = *c.meta_host;
+  if (m.err) {
+    t_err_where = m.err_where;
+    return m.err;
+  }
+  *result = (int64_t)m.pairs;
+  return build && (int64_t)m.pairs > c.capacity ? SLG_ERR_CAPACITY : SLG_OK;
+}
+
 // The whole pipeline for one side, one s and one row range.
 int run(const slg_hypergraph *h, int32_t smin, uint32_t flags, int32_t row_begin,
         int32_t row_end, Op op, int32_t *out_i, int32_t *out_j, int32_t *out_w,
@@ -792,66 +856,75 @@ int run(const slg_hypergraph *h, int32_t smin, uint32_t flags, int32_t row_begin
   // a prepared input (validated, maps made): its map of this side is used
   // as it is (read only; relabelling makes its own)
   const Prepared *pp = (t_prep && !relabel && same_input(t_prep->h, *h)) ? t_prep : nullptr;
-  SLG_TRY(pool.get(&w.meta, 1));
-  if (pp) w.csr2csc = pp->map[(flags & SLG_DUAL) ? 1 : 0];
-  else SLG_TRY(pool.get(&w.csr2csc, (size_t)nnz));
-  SLG_TRY(pool.get(&w.qs, (size_t)nnz + 1));
-  SLG_TRY(pool.get(&w.c_idx_s, (size_t)nnz * ((flags & SLG_TENSOR_CORE) ? 2 : 1) + 1));
-  SLG_TRY(pool.get(&w.c_off_s, (size_t)c.sd.C + 1));
-  SLG_TRY(pool.get(&w.tail_beg, (size_t)nnz));
-  SLG_TRY(pool.get(&w.tail_end, (size_t)nnz));
-  SLG_TRY(pool.get(&w.tile, (size_t)ntiles + 1));
-  SLG_TRY(pool.get(&w.bin_rows, (size_t)kNumLists * (c.rows > 0 ? c.rows : 1)));
-  SLG_TRY(pool.get(&w.n_e, (size_t)c.rows + 1));
-  SLG_TRY(pool.get(&w.row_work, (size_t)c.rows + 1));
-  SLG_TRY(pool.get(&w.stage_pos, (size_t)c.rows + 1));
-  SLG_TRY(pool.get(&w.row_ptr, (size_t)c.rows + 1));
-  SLG_TRY(pool.get(&w.tile64, (size_t)ntiles64 + 1));
-  SLG_TRY(cudaMemsetAsync(w.meta, 0, sizeof(Meta), st));
-
-  // Validation and the CSR->CSC map (a consistency check for every path),
-  // unless the input was prepared.
-  if (evs.on) cudaEventRecord(evs.ev[kEvPlan], st);
-  if (!pp) {
-    SLG_TRY(launch_validate(c.sd, w.meta, st));
-    SLG_TRY(launch_csr2csc(c.sd, w.csr2csc, w.meta, st));
-    c.launches += 3;
-  }
-
-  // Degree-ordered relabelling: the rest of the call runs on a renumbered
-  // copy of the side (built only from input that passed validation).
+  bool small = c.sd.R <= kSmallRows && (flags & SLG_ALGO_MASK) == SLG_ALGO_BINNED &&
+                     op != kOpWedges && !relabel && !row_s && !(flags & SLG_TENSOR_CORE);
   int32_t *perm = nullptr;
-  if (relabel) {
-    rc = read_meta(c);
-    if (rc) return rc;
-    int32_t *r_off2, *r_idx2, *c_idx2, *scr;
-    SLG_TRY(pool.get(&perm, (size_t)c.sd.R + 1));
-    SLG_TRY(pool.get(&r_off2, (size_t)c.sd.R + 1));
-    SLG_TRY(pool.get(&r_idx2, (size_t)nnz + 1));
-    SLG_TRY(pool.get(&c_idx2, (size_t)nnz + 1));
-    SLG_TRY(pool.get(&scr, relabel_scratch_ints(c.sd.R, nnz)));
-    if (evs.on) cudaEventRecord(evs.ev[kEvRelabel0], st);
-    SLG_TRY(launch_relabel(c.sd, relabel == SLG_RELABEL_DESC, perm, r_off2, r_idx2, c_idx2, scr,
-                           st, &c.launches));
-    c.sd.r_off = r_off2;
-    c.sd.r_idx = r_idx2;
-    c.sd.c_idx = c_idx2;
-    SLG_TRY(launch_csr2csc(c.sd, w.csr2csc, w.meta, st));
-    if (evs.on) cudaEventRecord(evs.ev[kEvRelabel1], st);
-    c.launches += 1;
-  }
-
   int64_t value = 0;
-  const uint32_t algo = flags & SLG_ALGO_MASK;
-  if (algo == SLG_ALGO_PLAIN) rc = run_plain(c, &value);
-  else if (algo == SLG_ALGO_SPGEMM) rc = run_spgemm(c, &value);
-  else rc = run_binned(c, &value);
-  if (rc == SLG_OK || rc == SLG_ERR_CAPACITY) *result = value;
-  if (rc != SLG_OK) return rc;
-  if (row_ptr_out) {
-    SLG_TRY(cudaMemcpyAsync(row_ptr_out, w.row_ptr, sizeof(long long) * ((size_t)c.rows + 1),
-                            cudaMemcpyDeviceToDevice, st));
-    SLG_TRY(cudaStreamSynchronize(st));
+  if (small) {
+    rc = run_small(c, pp, row_ptr_out, &value, &small);
+    if (small && (rc == SLG_OK || rc == SLG_ERR_CAPACITY)) *result = value;
+    if (rc != SLG_OK) return rc;
+  }
+  if (!small) {
+    SLG_TRY(pool.get(&w.meta, 1));
+    if (pp) w.csr2csc = pp->map[(flags & SLG_DUAL) ? 1 : 0];
+    else SLG_TRY(pool.get(&w.csr2csc, (size_t)nnz));
+    SLG_TRY(pool.get(&w.qs, (size_t)nnz + 1));
+    SLG_TRY(pool.get(&w.c_idx_s, (size_t)nnz * ((flags & SLG_TENSOR_CORE) ? 2 : 1) + 1));
+    SLG_TRY(pool.get(&w.c_off_s, (size_t)c.sd.C + 1));
+    SLG_TRY(pool.get(&w.tail_beg, (size_t)nnz));
+    SLG_TRY(pool.get(&w.tail_end, (size_t)nnz));
+    SLG_TRY(pool.get(&w.tile, (size_t)ntiles + 1));
+    SLG_TRY(pool.get(&w.bin_rows, (size_t)kNumLists * (c.rows > 0 ? c.rows : 1)));
+    SLG_TRY(pool.get(&w.n_e, (size_t)c.rows + 1));
+    SLG_TRY(pool.get(&w.row_work, (size_t)c.rows + 1));
+    SLG_TRY(pool.get(&w.stage_pos, (size_t)c.rows + 1));
+    SLG_TRY(pool.get(&w.row_ptr, (size_t)c.rows + 1));
+    SLG_TRY(pool.get(&w.tile64, (size_t)ntiles64 + 1));
+    SLG_TRY(cudaMemsetAsync(w.meta, 0, sizeof(Meta), st));
+
+    // Validation and the CSR->CSC map (a consistency check for every path),
+    // unless the input was prepared.
+    if (evs.on) cudaEventRecord(evs.ev[kEvPlan], st);
+    if (!pp) {
+      SLG_TRY(launch_validate(c.sd, w.meta, st));
+      SLG_TRY(launch_csr2csc(c.sd, w.csr2csc, w.meta, st));
+      c.launches += 3;
+    }
+
+    // Degree-ordered relabelling: the rest of the call runs on a renumbered
+    // copy of the side (built only from input that passed validation).
+    if (relabel) {
+      rc = read_meta(c);
+      if (rc) return rc;
+      int32_t *r_off2, *r_idx2, *c_idx2, *scr;
+      SLG_TRY(pool.get(&perm, (size_t)c.sd.R + 1));
+      SLG_TRY(pool.get(&r_off2, (size_t)c.sd.R + 1));
+      SLG_TRY(pool.get(&r_idx2, (size_t)nnz + 1));
+      SLG_TRY(pool.get(&c_idx2, (size_t)nnz + 1));
+      SLG_TRY(pool.get(&scr, relabel_scratch_ints(c.sd.R, nnz)));
+      if (evs.on) cudaEventRecord(evs.ev[kEvRelabel0], st);
+      SLG_TRY(launch_relabel(c.sd, relabel == SLG_RELABEL_DESC, perm, r_off2, r_idx2, c_idx2, scr,
+                             st, &c.launches));
+      c.sd.r_off = r_off2;
+      c.sd.r_idx = r_idx2;
+      c.sd.c_idx = c_idx2;
+      SLG_TRY(launch_csr2csc(c.sd, w.csr2csc, w.meta, st));
+      if (evs.on) cudaEventRecord(evs.ev[kEvRelabel1], st);
+      c.launches += 1;
+    }
+
+    const uint32_t algo = flags & SLG_ALGO_MASK;
+    if (algo == SLG_ALGO_PLAIN) rc = run_plain(c, &value);
+    else if (algo == SLG_ALGO_SPGEMM) rc = run_spgemm(c, &value);
+    else rc = run_binned(c, &value);
+    if (rc == SLG_OK || rc == SLG_ERR_CAPACITY) *result = value;
+    if (rc != SLG_OK) return rc;
+    if (row_ptr_out) {
+      SLG_TRY(cudaMemcpyAsync(row_ptr_out, w.row_ptr, sizeof(long long) * ((size_t)c.rows + 1),
+                              cudaMemcpyDeviceToDevice, st));
+      SLG_TRY(cudaStreamSynchronize(st));
+    }
   }
 
   // Relabelled pairs -> caller ids in canonical (i, j) order.
@@ -1026,7 +1099,7 @@ cudaError_t enqueue_plan(slg_plan *p, const Bins &bins, cudaStream_t st, int32_t
   } else {
     PLAN_TRY(cudaMemsetAsync(p->offsets, 0, sizeof(long long) * (p->count + 1), st));
   }
-  if (launches) *launches = 1 + 2 + 1 + 4 + 1 + n + 3 + 2;
+  if (launches) *launches = 1 + 2 + 1 + 4 + 2 + n + 3 + 2;
   return cudaSuccess;
 }
 #undef PLAN_TRY

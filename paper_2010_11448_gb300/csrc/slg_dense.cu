@@ -335,20 +335,7 @@ __global__ __launch_bounds__(C::NT, C::MINB) void k_walk_dense(
             if (!unweighted) tw[t] = n;
           }
         };
-        if (c) {
-          int32_t t = out + before + inc - c;
-          for (int32_t x = m0; x < m1; ++x) {
-            uint32_t m = map[x];
-            if (m) {
-              map[x] = 0;
-              do {
-                const int b = __ffs(m) - 1;
-                m &= m - 1;
-                emit_one(t++, (x << 5) + b);
-              } while (m);
-            }
-          }
-        }
+        for_survivors(map, m0, m1, out + before + inc - c, total > kSurvDense * nm, emit_one);
         out += total;
         __syncthreads();  // the counters are read
       }

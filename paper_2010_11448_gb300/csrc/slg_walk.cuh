@@ -52,6 +52,44 @@ __device__ __forceinline__ void l2_discard(const int32_t *p, long long n) {
     asm volatile("discard.global.L2 [%0], 128;" ::"l"(x) : "memory");
 }
 
+// Survivors per word of the bits from which for_survivors works by words.
+constexpr int32_t kSurvDense = 4;
+
+// fn(t, o) for every set bit o of map[m0, m1) in ascending o, t counting from
+// `start`, where each thread owns consecutive words and `start` is its first
+// place; clears the words.  `dense` (uniform): the bits are many, so a warp
+// takes its threads' words one by one, a lane per bit (consecutive places are
+// then written by consecutive lanes); else each thread takes its own.
+template <class Fn>
+__device__ __forceinline__ void for_survivors(uint32_t *map, int32_t m0, int32_t m1, int32_t start,
+                                              bool dense, Fn &&fn) {
+  if (!dense) {
+    for (int32_t x = m0; x < m1; ++x) {
+      uint32_t m = map[x];
+      if (!m) continue;
+      map[x] = 0;
+      do {
+        const int32_t b = __ffs(m) - 1;
+        m &= m - 1;
+        fn(start++, (x << 5) + b);
+      } while (m);
+    }
+    return;
+  }
+  const int lane = threadIdx.x & 31;
+  for (int src = 0; src < 32; ++src) {
+    const int32_t a = __shfl_sync(0xffffffffu, m0, src), b = __shfl_sync(0xffffffffu, m1, src);
+    int32_t t = __shfl_sync(0xffffffffu, start, src);
+    for (int32_t x = a; x < b; ++x) {
+      const uint32_t m = map[x];
+      if ((m >> lane) & 1u) fn(t + __popc(m & ((1u << lane) - 1u)), (x << 5) + lane);
+      t += __popc(m);
+    }
+  }
+  __syncwarp();  // the warp's words are read
+  for (int32_t x = m0; x < m1; ++x) map[x] = 0;
+}
+
 // fn(a[i]) for i = lo + threadIdx.x, lo + threadIdx.x + NT, ... < hi, with Q
 // loads issued together before their first use (the scratch reads are
 // latency-bound).
