@@ -274,6 +274,23 @@ int slg_wedges(const slg_hypergraph *h, int32_t s, uint32_t flags,
                int64_t *wedges, void *stream);
 
 /*
+ * slg_build_alloc -- slg_build (row_ptr NULL) or slg_build_csr (row_ptr of
+ * R + 1 entries) for callers that allocate the outputs by the pair count:
+ * once |L_s| is known, `alloc` is called on the calling thread and stores
+ * device arrays of n_pairs entries in *out_i, *out_j and *out_w (out_i may
+ * stay NULL with row_ptr, out_w with SLG_UNWEIGHTED; nothing is needed for
+ * n_pairs = 0).  A counting call before the build, and its walk, are saved.
+ * A non-zero return of `alloc` ends the call with SLG_ERR_NOMEM.
+ * Binned algorithm only, without relabelling (else SLG_ERR_UNSUPPORTED).
+ * slg_graph_build_alloc: the same through a prepared hypergraph.
+ */
+typedef int (*slg_alloc_fn)(void *ctx, int64_t n_pairs, int32_t **out_i,
+                            int32_t **out_j, int32_t **out_w);
+int slg_build_alloc(const slg_hypergraph *h, int32_t s, uint32_t flags,
+                    int64_t *row_ptr, slg_alloc_fn alloc, void *ctx,
+                    int64_t *n_pairs, void *stream);
+
+/*
  * slg_filter -- L_s from the canonical edge list of L_s' for any s' <= s:
  * the triples with w >= s, in the same order (Section III: L_s keeps the
  * overlaps of weight >= s, so L_s ⊆ L_s' with equal weights).
@@ -551,6 +568,9 @@ int slg_graph_count(const slg_graph *graph, int32_t s, uint32_t flags, int64_t *
 int slg_graph_build(const slg_graph *graph, int32_t s, uint32_t flags, int32_t *out_i,
                     int32_t *out_j, int32_t *out_w, int64_t capacity, int64_t *n_pairs,
                     void *stream);
+int slg_graph_build_alloc(const slg_graph *g, int32_t s, uint32_t flags,
+                          int64_t *row_ptr, slg_alloc_fn alloc, void *ctx,
+                          int64_t *n_pairs, void *stream);
 int slg_graph_destroy(slg_graph *graph);
 
 /* Returns the device memory that the library keeps for later calls on the

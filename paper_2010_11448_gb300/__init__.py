@@ -103,6 +103,8 @@ class _Query(ctypes.Structure):
 
 
 _I64P = ctypes.POINTER(ctypes.c_int64)
+_VPP = ctypes.POINTER(ctypes.c_void_p)
+_AllocFn = ctypes.CFUNCTYPE(ctypes.c_int, ctypes.c_void_p, ctypes.c_int64, _VPP, _VPP, _VPP)
 _VP = ctypes.c_void_p
 _HP = ctypes.POINTER(_Hypergraph)
 
@@ -112,6 +114,8 @@ ABI_FUNCTIONS = {
     "slg_count_noalloc": (ctypes.c_int, [_HP, ctypes.c_int32, ctypes.c_uint32, _I64P, _VP]),
     "slg_build": (ctypes.c_int, [_HP, ctypes.c_int32, ctypes.c_uint32, _VP, _VP, _VP,
                                  ctypes.c_int64, _I64P, _VP]),
+    "slg_build_alloc": (ctypes.c_int, [_HP, ctypes.c_int32, ctypes.c_uint32, _VP, _AllocFn, _VP,
+                                       _I64P, _VP]),
     "slg_build_rows": (ctypes.c_int, [_HP, ctypes.c_int32, ctypes.c_uint32,
                                       ctypes.c_int32, ctypes.c_int32, _VP, _VP, _VP,
                                       ctypes.c_int64, _I64P, _VP]),
@@ -158,6 +162,8 @@ ABI_FUNCTIONS = {
     "slg_graph_count": (ctypes.c_int, [_VP, ctypes.c_int32, ctypes.c_uint32, _I64P, _VP]),
     "slg_graph_build": (ctypes.c_int, [_VP, ctypes.c_int32, ctypes.c_uint32, _VP, _VP, _VP,
                                        ctypes.c_int64, _I64P, _VP]),
+    "slg_graph_build_alloc": (ctypes.c_int, [_VP, ctypes.c_int32, ctypes.c_uint32, _VP, _AllocFn,
+                                             _VP, _I64P, _VP]),
     "slg_graph_destroy": (ctypes.c_int, [_VP]),
     "slg_strerror": (ctypes.c_char_p, [ctypes.c_int]),
     "slg_abi_version": (ctypes.c_int, []),
@@ -280,17 +286,62 @@ def _outputs(capacity, unweighted, device):
     return oi, oj, ow
 
 
+def _build_alloc(fn, what, arg, s, flags, unweighted, device, stream, row_ptr=None):
+    """One walk, the outputs allocated by the pair count it finds
+    (slg_build_alloc): (i, j, w), i None with `row_ptr`; None when the outputs
+    could not be allocated next to the walk's memory."""
+    import torch
+    got = {}
+
+    def alloc(_, n, oi, oj, ow):
+        try:
+            got["out"] = out = _outputs(n, unweighted, device)
+            if row_ptr is not None:
+                got["out"] = out = (None, *out[1:])
+            for p, t in zip((oi, oj, ow), out):
+                if t is not None:
+                    p[0] = t.data_ptr()
+            return 0
+        except torch.cuda.OutOfMemoryError:
+            got["oom"] = True
+        except BaseException as exc:  # noqa: B902 - raised again below
+            got["exc"] = exc
+        return 1
+
+    n = ctypes.c_int64(0)
+    cb = _AllocFn(alloc)
+    rc = fn(arg, int(s), flags, row_ptr.data_ptr() if row_ptr is not None else None, cb, None,
+            ctypes.byref(n), _stream(stream))
+    if "exc" in got:
+        raise got["exc"]
+    if "oom" in got:
+        return None
+    if rc != 0:
+        raise SlgError(rc, what)
+    if n.value == 0:
+        oi, oj, ow = _outputs(0, unweighted, device)
+    else:
+        oi, oj, ow = got["out"]
+    p = int(n.value)
+    return (oi[:p] if row_ptr is None else None), oj[:p], (ow[:p] if ow is not None else None)
+
+
 def build(h: DeviceHypergraph, s: int, dual=False, unweighted=False,
           algo="binned", capacity=None, out=None, stream=None, tensor=False,
           relabel=None, prune=True):
     """The canonical edge list of L_s as int32 tensors (i, j, w); w is None
-    with unweighted=True.  Without ``capacity``/``out`` the pair count is
-    taken first with ``count`` (an extra walk).  tensor=True counts a dense
+    with unweighted=True.  Without ``capacity``/``out`` the arrays are
+    allocated once the walk has counted the pairs.  tensor=True counts a dense
     core block on the tensor cores; relabel="asc"/"desc" renumbers the rows
     by size for the walk; prune=False switches off the degree-based pruning
     (all give the same result)."""
     flags = _flags(dual, unweighted, algo, tensor, relabel, prune)
     if out is None:
+        if capacity is None and algo == "binned" and relabel is None:
+            got = _build_alloc(load().slg_build_alloc, "slg_build", ctypes.byref(h.struct), s,
+                               flags, unweighted, h.e_off.device, stream)
+            if got is not None:
+                return got
         if capacity is None:
             capacity = count(h, s, dual, unweighted, algo, stream, tensor)
         out = _outputs(capacity, unweighted, h.e_off.device)
@@ -372,6 +423,12 @@ def build_csr(h: DeviceHypergraph, s: int, dual=False, unweighted=False, algo="b
     flags = _flags(dual, unweighted, algo, tensor, None, prune)
     R = h.rows(dual)
     if out is None:
+        if capacity is None and algo == "binned":
+            ptr = torch.empty(R + 1, dtype=torch.int64, device=h.e_off.device)
+            got = _build_alloc(load().slg_build_alloc, "slg_build_csr", ctypes.byref(h.struct),
+                               s, flags, unweighted, h.e_off.device, stream, ptr)
+            if got is not None:
+                return ptr, got[1], got[2]
         if capacity is None:
             capacity = count(h, s, dual, unweighted, algo, stream, tensor)
         _, oj, ow = _outputs(capacity, unweighted, h.e_off.device)
@@ -690,6 +747,11 @@ class Graph:
               out=None, stream=None, tensor=False, prune=True):
         flags = _flags(dual, unweighted, algo, tensor, None, prune)
         if out is None:
+            if capacity is None and algo == "binned":
+                got = _build_alloc(load().slg_graph_build_alloc, "slg_graph_build", self._g, s,
+                                   flags, unweighted, self.h.e_off.device, stream)
+                if got is not None:
+                    return got
             if capacity is None:
                 capacity = self.count(s, dual, unweighted, algo, stream, tensor, prune)
             out = _outputs(capacity, unweighted, self.h.e_off.device)

@@ -274,6 +274,9 @@ struct Call {
   int32_t *row_work_out;  // slg_row_work: per-row wedge work (device)
   bool tile_ran;          // the dense-core tile kernel was launched
   int64_t capacity;
+  slg_alloc_fn alloc;     // gives the outputs once the pairs are counted, or null
+  void *alloc_ctx;
+  bool rows_form;         // compressed row form: out_i may be null
   cudaStream_t st;
   DeviceCtx *ctx;
   Pool *pool;
@@ -470,6 +473,15 @@ int plan_core(Call &c, CoreInfo *core) {
   return SLG_OK;
 }
 
+// The caller's outputs for `pairs` pairs (Call::alloc).
+int call_alloc(Call &c, int64_t pairs) {
+  c.capacity = pairs;
+  if (pairs == 0) return SLG_OK;
+  if (c.alloc(c.alloc_ctx, pairs, &c.out_i, &c.out_j, &c.out_w) != 0) return SLG_ERR_NOMEM;
+  return (c.out_i || c.rows_form) && c.out_j && (c.unweighted || c.out_w) ? SLG_OK
+                                                                           : SLG_ERR_INVALID;
+}
+
 // Default path: filtered CSC, binned single walk, staging, scan, gather.
 int run_binned(Call &c, int64_t *result) {
   Work &w = c.w;
@@ -494,16 +506,26 @@ int run_binned(Call &c, int64_t *result) {
     *result = (int64_t)c.meta_host->wedges;
     return SLG_OK;
   }
-  if (c.op == kOpBuild && c.capacity > 0) {
-    if (c.pool->get(&w.stage_j, (size_t)c.capacity) == cudaSuccess &&
-        (c.unweighted || c.pool->get(&w.stage_w, (size_t)c.capacity) == cudaSuccess))
-      w.stage_cap = c.capacity;
-    else
-      w.stage_cap = 0;  // rows that find no staging room are re-walked directly
-  }
+  auto stage = [&](int64_t cap) {
+    w.stage_cap = 0;  // rows that find no staging room are re-walked directly
+    if (cap > 0 && c.pool->get(&w.stage_j, (size_t)cap) == cudaSuccess &&
+        (c.unweighted || c.pool->get(&w.stage_w, (size_t)cap) == cudaSuccess))
+      w.stage_cap = cap;
+  };
+  if (c.op == kOpBuild && !c.alloc) stage(c.capacity);
   // Planning totals: the giant bin's scratch is sized by its largest row.
   int rc = read_meta(c);
   if (rc) return rc;
+  if (c.alloc) {
+    // The pairs are not known yet.  Each has at least s wedges; on real
+    // lists an eighth of the wedges at s = 2 is plenty (0.06 to 0.08 on
+    // chung_lu_1m), and a list that is longer is walked again.
+    const int64_t W = (int64_t)c.meta_host->wedges;
+    int64_t cap = W / c.smin;
+    if (c.smin > 1) cap = std::min(cap, std::max<int64_t>(W / 8, (int64_t)1 << 22));
+    if (core.T) cap += (int64_t)core.n_core * core.n_core / 2;
+    stage(std::max<int64_t>(cap, 1));
+  }
   // (core rows may have no wedges but still need a giant CTA; their pairs,
   // staged in the same scratch, also come from up to n_core tile items)
   // (a sparse-bin row whose candidates overflow its table is handed to the
@@ -534,6 +556,11 @@ int run_binned(Call &c, int64_t *result) {
   L.w.c_idx_s = w.c_idx_s;
   L.w.tail_beg = w.tail_beg;
   L.w.tail_end = w.tail_end;
+  for (int b : {kBinWarp, kBinCtaS, kBinCtaL})
+    if (!mp.rows_bin[b]) L.skip |= 1u << b;
+  if (!mp.sparse_huge) L.skip |= kSkipSparseBig;
+  if (!mp.sparse_rest) L.skip |= kSkipSparseSmall;
+  if (!mp.rows_bin[kBinGiant] && !mp.rows_bin[kBinSparse]) L.skip |= 1u << kBinGiant;
   cudaEvent_t *ev = c.evs->on ? c.evs->ev + kEvWalk : nullptr;
   if (c.rows > 0) {
     SLG_TRY(launch_walk(L, c.st, &c.launches, ev));
@@ -543,44 +570,58 @@ int run_binned(Call &c, int64_t *result) {
   SLG_TRY(launch_row_scan(c.rows, w, c.st));
   if (c.evs->on) cudaEventRecord(c.evs->ev[kEvScan], c.st);
   c.launches += 3;
+  const Meta &m = *c.meta_host;
+  auto gather = [&]() -> cudaError_t {
+    if (c.evs->on) cudaEventRecord(c.evs->ev[kEvGather0], c.st);
+    if (c.capacity <= 0 || c.rows <= 0) return cudaSuccess;
+    ++c.launches;
+    return launch_gather(c.row_begin, c.rows, w, c.out_i, c.out_j, c.out_w, c.unweighted,
+                         c.capacity, 0, c.st);
+  };
+  // With the outputs in hand the gather follows the scan at once: on the
+  // device it does nothing when the pairs do not fit the outputs or the
+  // staging area.
+  if (c.op == kOpBuild && !c.alloc) SLG_TRY(gather());
+  if (c.op == kOpBuild && !c.alloc && c.evs->on) cudaEventRecord(c.evs->ev[kEvGather1], c.st);
   rc = read_meta(c);
   if (rc) return rc;
-  const Meta &m = *c.meta_host;
   const int64_t pairs = (int64_t)m.pairs;
   *result = pairs;
   if (c.op != kOpBuild) return SLG_OK;
-  if (pairs > c.capacity) return SLG_ERR_CAPACITY;
-  if (c.evs->on) cudaEventRecord(c.evs->ev[kEvGather0], c.st);
-  if (pairs > 0) {
+  if (c.alloc) {
+    rc = call_alloc(c, pairs);
+    if (rc) return rc;
     if (m.stage_overflow == 0) {
-      SLG_TRY(launch_gather(c.row_begin, c.rows, w, c.out_i, c.out_j, c.out_w, c.unweighted,
-                            c.capacity, c.st));
-      c.launches += 1;
-    } else {
-      // Staging too small: walk again, writing straight to the output.
-      SLG_TRY(cudaMemsetAsync(&w.meta->giant_ticket, 0, sizeof(unsigned int), c.st));
-      static_assert(offsetof(Meta, dense_ticket_rest) ==
-                        offsetof(Meta, dense_ticket) + sizeof(unsigned int),
-                    "the two dense ticket counters are cleared together");
-      SLG_TRY(cudaMemsetAsync(&w.meta->dense_ticket, 0, 2 * sizeof(unsigned int), c.st));
-      static_assert(offsetof(Meta, sparse_ticket_rest) ==
-                        offsetof(Meta, sparse_ticket) + sizeof(unsigned int),
-                    "the two sparse ticket counters are cleared together");
-      SLG_TRY(cudaMemsetAsync(&w.meta->sparse_ticket, 0, 2 * sizeof(unsigned int), c.st));
-      // back to the planned giant list: the sparse bin hands the same rows
-      // over again
-      SLG_TRY(cudaMemcpyAsync(&w.meta->rows_bin[kBinGiant], &giant_rows0, sizeof(giant_rows0),
-                              cudaMemcpyHostToDevice, c.st));
-      SLG_TRY(cudaMemcpyAsync(&w.meta->giant_rest, &giant_rest0, sizeof(giant_rest0),
-                              cudaMemcpyHostToDevice, c.st));
-      L.a.mode = kDirect;
-      L.a.row_ptr = w.row_ptr;
-      L.a.out_i = c.out_i;
-      L.a.out_j = c.out_j;
-      L.a.out_w = c.out_w;
-      SLG_TRY(launch_walk(L, c.st, &c.launches));
+      SLG_TRY(gather());
+      if (c.evs->on) cudaEventRecord(c.evs->ev[kEvGather1], c.st);
+      return read_meta(c);
     }
+    if (c.evs->on) cudaEventRecord(c.evs->ev[kEvGather0], c.st);
   }
+  if (pairs > c.capacity) return SLG_ERR_CAPACITY;
+  if (m.stage_overflow == 0) return SLG_OK;
+  // Staging too small: walk again, writing straight to the output.
+  SLG_TRY(cudaMemsetAsync(&w.meta->giant_ticket, 0, sizeof(unsigned int), c.st));
+  static_assert(offsetof(Meta, dense_ticket_rest) ==
+                    offsetof(Meta, dense_ticket) + sizeof(unsigned int),
+                "the two dense ticket counters are cleared together");
+  SLG_TRY(cudaMemsetAsync(&w.meta->dense_ticket, 0, 2 * sizeof(unsigned int), c.st));
+  static_assert(offsetof(Meta, sparse_ticket_rest) ==
+                    offsetof(Meta, sparse_ticket) + sizeof(unsigned int),
+                "the two sparse ticket counters are cleared together");
+  SLG_TRY(cudaMemsetAsync(&w.meta->sparse_ticket, 0, 2 * sizeof(unsigned int), c.st));
+  // back to the planned giant list: the sparse bin hands the same rows
+  // over again
+  SLG_TRY(cudaMemcpyAsync(&w.meta->rows_bin[kBinGiant], &giant_rows0, sizeof(giant_rows0),
+                          cudaMemcpyHostToDevice, c.st));
+  SLG_TRY(cudaMemcpyAsync(&w.meta->giant_rest, &giant_rest0, sizeof(giant_rest0),
+                          cudaMemcpyHostToDevice, c.st));
+  L.a.mode = kDirect;
+  L.a.row_ptr = w.row_ptr;
+  L.a.out_i = c.out_i;
+  L.a.out_j = c.out_j;
+  L.a.out_w = c.out_w;
+  SLG_TRY(launch_walk(L, c.st, &c.launches));
   if (c.evs->on) cudaEventRecord(c.evs->ev[kEvGather1], c.st);
   rc = read_meta(c);
   return rc;
@@ -744,6 +785,7 @@ int run_small(Call &c, const Prepared *pp, long long *row_ptr_out, int64_t *resu
   const size_t o_sp = o_ne + up(rows * 4), o_map = o_sp + up(rows * 8);
   const size_t o_j = o_map + (pp ? 0 : up((size_t)nnz * 4));
   const int64_t most = (int64_t)c.sd.R * (c.sd.R - 1) / 2;
+  // (with Call::alloc the capacity is a first guess)
   const size_t cap = build ? (size_t)std::min<int64_t>(c.capacity, most) : 0;
   const size_t o_w = o_j + up(cap * 4), bytes = o_w + (c.unweighted ? 0 : up(cap * 4));
   unsigned char *buf = nullptr;
@@ -774,6 +816,7 @@ int run_small(Call &c, const Prepared *pp, long long *row_ptr_out, int64_t *resu
   s.out_w = c.out_w;
   s.row_ptr = row_ptr_out;
   s.host = c.meta_view;
+  s.hold = c.alloc != nullptr;
   const bool on = c.evs->on;
   cudaEvent_t *ev = c.evs->ev;
   if (on) cudaEventRecord(ev[kEvPlan], c.st);
@@ -791,8 +834,24 @@ int run_small(Call &c, const Prepared *pp, long long *row_ptr_out, int64_t *resu
     t_err_where = m.err_where;
     return m.err;
   }
-  *result = (int64_t)m.pairs;
-  return build && (int64_t)m.pairs > c.capacity ? SLG_ERR_CAPACITY : SLG_OK;
+  const int64_t pairs = (int64_t)m.pairs;
+  *result = pairs;
+  if (!build || pairs <= (int64_t)cap) {
+    if (!c.alloc) return SLG_OK;
+    const int rc = call_alloc(c, pairs);
+    if (rc != SLG_OK || pairs == 0) return rc;
+    s.out_i = c.out_i;
+    s.out_j = c.out_j;
+    s.out_w = c.out_w;
+    SLG_TRY(launch_small_emit(s, c.st, &c.launches));
+    SLG_TRY(cudaStreamSynchronize(c.st));
+    return SLG_OK;
+  }
+  if (!c.alloc) return SLG_ERR_CAPACITY;
+  // more pairs than guessed: once more, with their number
+  const int rc = call_alloc(c, pairs);
+  c.alloc = nullptr;
+  return rc ? rc : run_small(c, pp, row_ptr_out, result, room);
 }
 
 // The whole pipeline for one side, one s and one row range.
@@ -801,7 +860,8 @@ int run(const slg_hypergraph *h, int32_t smin, uint32_t flags, int32_t row_begin
         int64_t capacity, int64_t *result, cudaStream_t st, const int32_t *row_s = nullptr,
         int32_t *max_row_work = nullptr, long long *row_ptr_out = nullptr,
         int32_t *row_work_out = nullptr, const int32_t *row_fhi = nullptr,
-        int32_t *max_row_size = nullptr) {
+        int32_t *max_row_size = nullptr, slg_alloc_fn alloc = nullptr,
+        void *alloc_ctx = nullptr) {
   int rc = check_args(h, smin, flags);
   if (rc != SLG_OK) return rc;
   if (!result) return SLG_ERR_INVALID;
@@ -818,7 +878,7 @@ int run(const slg_hypergraph *h, int32_t smin, uint32_t flags, int32_t row_begin
   const bool rows_form = op == kOpBuild && row_ptr_out != nullptr;
   if (op == kOpBuild) {
     if (capacity < 0) return SLG_ERR_INVALID;
-    if (capacity > 0 && ((!rows_form && !out_i) || !out_j || (!c.unweighted && !out_w)))
+    if (!alloc && capacity > 0 && ((!rows_form && !out_i) || !out_j || (!c.unweighted && !out_w)))
       return SLG_ERR_INVALID;
   }
   if (rows_form && ((flags & SLG_ALGO_MASK) == SLG_ALGO_SPGEMM ||
@@ -831,7 +891,10 @@ int run(const slg_hypergraph *h, int32_t smin, uint32_t flags, int32_t row_begin
   c.out_i = out_i;
   c.out_j = out_j;
   c.out_w = out_w;
-  c.capacity = capacity;
+  c.capacity = alloc ? (int64_t)1 << 22 : capacity;
+  c.alloc = alloc;
+  c.alloc_ctx = alloc_ctx;
+  c.rows_form = rows_form;
   c.st = st;
   c.row_work_out = row_work_out;
   const int64_t nnz = c.sd.nnz;
@@ -1093,7 +1156,7 @@ cudaError_t enqueue_plan(slg_plan *p, const Bins &bins, cudaStream_t st, int32_t
   PLAN_TRY(launch_row_scan(sd.R, w, st));
   if (p->pairs > 0) {
     PLAN_TRY(launch_gather(0, sd.R, w, p->out_i, p->out_j, p->out_w, L.a.unweighted,
-                           p->pairs, st));
+                           p->pairs, 1, st));
     PLAN_TRY(launch_localize(p->out_i, p->out_j, p->pairs, p->row_base, p->count, w.row_ptr,
                              p->offsets, st));
   } else {
@@ -1276,6 +1339,17 @@ int slg_build(const slg_hypergraph *h, int32_t s, uint32_t flags, int32_t *out_i
   const int32_t R = (flags & SLG_DUAL) ? h->n_vertices : h->n_edges;
   return run(h, s, flags, 0, R, kOpBuild, out_i, out_j, out_w, capacity, n_pairs,
              (cudaStream_t)stream);
+}
+
+int slg_build_alloc(const slg_hypergraph *h, int32_t s, uint32_t flags, int64_t *row_ptr,
+                    slg_alloc_fn alloc, void *ctx, int64_t *n_pairs, void *stream) {
+  if (!h || !alloc) return SLG_ERR_INVALID;
+  if ((flags & SLG_ALGO_MASK) != SLG_ALGO_BINNED || (flags & (SLG_RELABEL_ASC | SLG_RELABEL_DESC)))
+    return SLG_ERR_UNSUPPORTED;
+  const int32_t R = (flags & SLG_DUAL) ? h->n_vertices : h->n_edges;
+  return run(h, s, flags, 0, R, kOpBuild, nullptr, nullptr, nullptr, 0, n_pairs,
+             (cudaStream_t)stream, nullptr, nullptr, reinterpret_cast<long long *>(row_ptr),
+             nullptr, nullptr, nullptr, alloc, ctx);
 }
 
 int slg_build_rows(const slg_hypergraph *h, int32_t s, uint32_t flags, int32_t row_begin,
@@ -2036,6 +2110,15 @@ extern "C" int slg_graph_build(const slg_graph *g, int32_t s, uint32_t flags, in
   if (rc != SLG_OK) return rc;
   PrepScope scope(&g->p);
   return slg_build(&g->p.h, s, flags, out_i, out_j, out_w, capacity, n_pairs, stream);
+}
+
+extern "C" int slg_graph_build_alloc(const slg_graph *g, int32_t s, uint32_t flags,
+                                     int64_t *row_ptr, slg_alloc_fn alloc, void *ctx,
+                                     int64_t *n_pairs, void *stream) {
+  const int rc = graph_check(g);
+  if (rc != SLG_OK) return rc;
+  PrepScope scope(&g->p);
+  return slg_build_alloc(&g->p.h, s, flags, row_ptr, alloc, ctx, n_pairs, stream);
 }
 
 extern "C" int slg_graph_destroy(slg_graph *g) {

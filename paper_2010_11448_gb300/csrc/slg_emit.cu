@@ -85,8 +85,14 @@ __global__ __launch_bounds__(kNT) void k_gather(int32_t row_begin, int32_t rows,
                                                 int32_t *__restrict__ out_j,
                                                 int32_t *__restrict__ out_w, int unweighted,
                                                 long long stage_cap, long long out_cap,
-                                                Meta *meta) {
+                                                int strict, Meta *meta) {
   if (meta->err) return;
+  // too many pairs for the output or the staging area: the host goes on from
+  // there (strict: it does not expect that)
+  if (meta->stage_overflow || (long long)meta->pairs > out_cap) {
+    if (strict && threadIdx.x == 0) raise_error(meta, SLG_ERR_INVALID, kWhereStage);
+    return;
+  }
   __shared__ long long s_ptr[kGatherRows + 1];
   __shared__ long long s_sp[kGatherRows];
   const int32_t r0 = blockIdx.x * kGatherRows;
@@ -204,11 +210,11 @@ cudaError_t launch_row_scan(int32_t rows, const Work &w, cudaStream_t st) {
 
 cudaError_t launch_gather(int32_t row_begin, int32_t rows, const Work &w, int32_t *out_i,
                           int32_t *out_j, int32_t *out_w, int unweighted, long long out_cap,
-                          cudaStream_t st) {
+                          int strict, cudaStream_t st) {
   if (rows <= 0) return cudaSuccess;
   const int grid = (rows + kGatherRows - 1) / kGatherRows;
   k_gather<<<grid, kNT, 0, st>>>(row_begin, rows, w.row_ptr, w.stage_pos, w.stage_j, w.stage_w,
-                                 out_i, out_j, out_w, unweighted, w.stage_cap, out_cap, w.meta);
+                                 out_i, out_j, out_w, unweighted, w.stage_cap, out_cap, strict, w.meta);
   return cudaGetLastError();
 }
 

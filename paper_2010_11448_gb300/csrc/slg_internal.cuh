@@ -557,7 +557,10 @@ struct WalkLaunch {
   long long scratch_ints;   // of giant_scratch
   long long dense_pairs[2]; // most pairs a dense-bin row can have: big instance, other (0: no row)
   int32_t dense_size;       // most vertices of a dense-bin row
+  unsigned skip;            // bit b: bin b is known to be empty (kSkipSparseBig, ...)
 };
+// Further bits of WalkLaunch::skip: the sparse bin's two instances.
+constexpr unsigned kSkipSparseBig = 1u << 8, kSkipSparseSmall = 1u << 9;
 
 // Sides of at most this many rows take the short path (slg_small.cu).
 #ifndef SLG_SMALL_ROWS
@@ -575,7 +578,9 @@ struct SmallCall {
   int32_t *out_i, *out_j, *out_w;
   long long *row_ptr;            // [rows + 1] or null
   Meta *host;                    // mapped host memory, receives the Meta
+  bool hold;                     // the outputs come later (launch_small_emit)
 };
+cudaError_t launch_small_emit(const SmallCall &c, cudaStream_t st, int32_t *launches);
 cudaError_t launch_small(const SmallCall &c, cudaStream_t st, int32_t *launches, cudaEvent_t walk0,
                          cudaEvent_t walk1);
 
@@ -605,10 +610,11 @@ cudaError_t launch_meta_copy(const Meta *src, Meta *dst, cudaStream_t st);
 // w16[i] = w[i] (i < n); *bad = 1 if a weight is above 65,535.
 cudaError_t launch_pack_w16(const int32_t *w, int64_t n, uint16_t *w16, int32_t *bad,
                             cudaStream_t st);
-// out_cap: entries of the output arrays (a row beyond them raises an error).
+// out_cap: entries of the output arrays (with more pairs, or rows that found
+// no staging room, nothing is written; strict: that is an error).
 cudaError_t launch_gather(int32_t row_begin, int32_t rows, const Work &w, int32_t *out_i,
                           int32_t *out_j, int32_t *out_w, int unweighted, long long out_cap,
-                          cudaStream_t st);
+                          int strict, cudaStream_t st);
 
 // Batched form (slg_plan.cu): union of many hypergraphs.
 struct BatchGraph {            // one member, device pointers

@@ -409,6 +409,18 @@ int small_ctas(int lb, int32_t R, size_t *smem) {
   return o.sms * std::max(per, 1);
 }
 
+// Places and totals, and (emit) the pairs.
+cudaError_t small_emit(const SmallCall &c, bool emit, cudaStream_t st, int32_t *launches) {
+  const int32_t rows = c.row_end - c.row_begin;
+  const int grid = std::max((rows + kEmRows - 1) / kEmRows, 1);
+  k_small_emit<<<grid, kEmNT, 0, st>>>(c.row_begin, rows, c.a.n_e, c.active, c.a.stage_pos,
+                                       emit ? c.a.stage_j : nullptr, c.a.stage_w, c.out_i, c.out_j,
+                                       c.out_w, c.a.unweighted, c.row_ptr, c.a.stage_cap, c.a.meta,
+                                       reinterpret_cast<volatile uint32_t *>(c.host));
+  ++*launches;
+  return cudaGetLastError();
+}
+
 }  // namespace
 
 cudaError_t launch_small(const SmallCall &c, cudaStream_t st, int32_t *launches, cudaEvent_t walk0,
@@ -431,14 +443,12 @@ cudaError_t launch_small(const SmallCall &c, cudaStream_t st, int32_t *launches,
     ++*launches;
   }
   if (walk1) cudaEventRecord(walk1, st);
-  const int grid = std::max((rows + kEmRows - 1) / kEmRows, 1);
-  const bool emit = c.a.mode != kCount;
-  k_small_emit<<<grid, kEmNT, 0, st>>>(c.row_begin, rows, c.a.n_e, c.active, c.a.stage_pos,
-                                       emit ? c.a.stage_j : nullptr, c.a.stage_w, c.out_i, c.out_j,
-                                       c.out_w, c.a.unweighted, c.row_ptr, c.a.stage_cap, c.a.meta,
-                                       reinterpret_cast<volatile uint32_t *>(c.host));
-  ++*launches;
-  return cudaGetLastError();
+  return small_emit(c, !c.hold && c.a.mode != kCount, st, launches);
+}
+
+// The emission of a held call, once its outputs are there.
+cudaError_t launch_small_emit(const SmallCall &c, cudaStream_t st, int32_t *launches) {
+  return small_emit(c, true, st, launches);
 }
 
 }  // namespace slg

@@ -564,9 +564,14 @@ long long sparse_ints(int32_t max_work) {
 cudaError_t launch_walk_sparse(const WalkLaunch &L, cudaStream_t st, int32_t *launches) {
   if (!L.giant_scratch) return cudaSuccess;  // no row in the bin
   SpOcc &o = sp_occ();
-  sp_launch<SpBig>(L, o.big, 0, st);
-  sp_launch<SpSmall>(L, o.small, 1, st);
-  *launches += 2;
+  if (!(L.skip & kSkipSparseBig)) {
+    sp_launch<SpBig>(L, o.big, 0, st);
+    ++*launches;
+  }
+  if (!(L.skip & kSkipSparseSmall)) {
+    sp_launch<SpSmall>(L, o.small, 1, st);
+    ++*launches;
+  }
   return cudaGetLastError();
 }
 

@@ -707,17 +707,24 @@ cudaError_t launch_walk(const WalkLaunch &L, cudaStream_t st, int32_t *launches,
   const int64_t stride = L.rows;
   int n = 0;
   if (ev) cudaEventRecord(ev[0], st);
-  k_walk_warp<<<o.sms * (o.warp_blocks > 0 ? o.warp_blocks : 1), kWarpNT, 0, st>>>(
-      L.w, lists + 0 * stride, L.a);
-  ++n;
+  auto empty = [&](int bin) { return (L.skip >> bin) & 1u; };
+  if (!empty(kBinWarp)) {
+    k_walk_warp<<<o.sms * (o.warp_blocks > 0 ? o.warp_blocks : 1), kWarpNT, 0, st>>>(
+        L.w, lists + 0 * stride, L.a);
+    ++n;
+  }
   if (ev) cudaEventRecord(ev[1], st);
-  K_CTA_S<<<o.sms * (o.s_blocks > 0 ? o.s_blocks : 1), 256, CfgS::smem(), st>>>(
-      L.w, lists + 1 * stride, L.row_work, L.a);
-  ++n;
+  if (!empty(kBinCtaS)) {
+    K_CTA_S<<<o.sms * (o.s_blocks > 0 ? o.s_blocks : 1), 256, CfgS::smem(), st>>>(
+        L.w, lists + 1 * stride, L.row_work, L.a);
+    ++n;
+  }
   if (ev) cudaEventRecord(ev[2], st);
-  K_CTA_L<<<o.sms * (o.l_blocks > 0 ? o.l_blocks : 1), 256, CfgL::smem(), st>>>(
-      L.w, lists + 2 * stride, L.row_work, L.a);
-  ++n;
+  if (!empty(kBinCtaL)) {
+    K_CTA_L<<<o.sms * (o.l_blocks > 0 ? o.l_blocks : 1), 256, CfgL::smem(), st>>>(
+        L.w, lists + 2 * stride, L.row_work, L.a);
+    ++n;
+  }
   if (ev) cudaEventRecord(ev[3], st);
   // the sparse bin before the giant bin: a sparse row whose candidates
   // overflow its table is appended to the giant bin's list
@@ -730,7 +737,7 @@ cudaError_t launch_walk(const WalkLaunch &L, cudaStream_t st, int32_t *launches,
     const cudaError_t e = launch_walk_dense(L, st, &n);
     if (e != cudaSuccess) return e;
   }
-  if (L.giant_scratch && L.giant_stride > 0) {
+  if (L.giant_scratch && L.giant_stride > 0 && !empty(kBinGiant)) {
     k_walk_giant<<<o.sms * o.g_blocks, kGiantNT, giant_smem(), st>>>(
         L.w, lists + 3 * stride, L.a, L.giant_scratch, L.giant_stride, L.R, (int32_t)stride);
     ++n;

@@ -1,0 +1,85 @@
+"""Builds that allocate their outputs by the pair count (one walk): equal to a
+build into arrays of that size, also when the walk's staging area turns out
+too small (short path: walked again; general path: walked again straight to
+the output, through every bin)."""
+import ctypes
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+import hypergen as hg  # noqa: E402
+import paper_2010_11448_gb300 as slg  # noqa: E402
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2010_11448_gb300 import build_lib
+    build_lib.build()
+    slg.load()
+
+
+def same(h, s, dual=False):
+    dh = slg.to_device(h)
+    ref = slg.build(dh, s, dual, capacity=max(slg.count(dh, s, dual), 1))
+    rows = dh.rows(dual)
+    ptr = torch.zeros(rows + 1, dtype=torch.int64, device="cuda")
+    ptr[1:] = torch.bincount(ref[0].long(), minlength=rows).cumsum(0)
+    with slg.Graph(dh) as g:
+        for got in (slg.build(dh, s, dual), g.build(s, dual)):
+            assert all(torch.equal(a, b) for a, b in zip(got, ref))
+        for got in (slg.build(dh, s, dual, unweighted=True), g.build(s, dual, unweighted=True)):
+            assert got[2] is None and all(torch.equal(a, b) for a, b in zip(got[:2], ref))
+    p, j, w = slg.build_csr(dh, s, dual)
+    assert torch.equal(p, ptr) and torch.equal(j, ref[1]) and torch.equal(w, ref[2])
+    return int(ref[0].numel())
+
+
+def groups(count, size, k, extra):
+    """`count` groups of `size` equal hyperedges of k vertices, dealt out over
+    the ids, and `extra` empty ones: every wedge belongs to a pair of weight k."""
+    m = count * size + extra
+    rng = np.random.default_rng(count)
+    ids = rng.permutation(m)[: count * size].reshape(count, size)
+    r = np.repeat(ids.ravel(), k)
+    c = np.repeat(np.arange(count) * k, size)[:, None] + np.arange(k)
+    return hg.from_pairs(r, c.ravel(), m, count * k)
+
+
+def test_outputs_by_count():
+    for m, n in ((900, 2_000), (30_000, 60_000)):
+        h = hg.chung_lu(m, n, seed=m, size_cap=3000)
+        for dual in (False, True):
+            for s in (1, 2, 6, 10_000):
+                same(h, s, dual)
+
+
+# short path; warp, CTA-S, dense and sparse bins
+@pytest.mark.parametrize("count,size,k,extra", [
+    (20, 800, 2, 0), (20_000, 24, 2, 0), (400, 200, 2, 0), (10, 3_000, 2, 0),
+    (10, 3_000, 2, 500_000), (6, 3_000, 20, 500_000)])
+def test_lists_longer_than_the_staging_area(count, size, k, extra):
+    h = groups(count, size, k, extra)
+    pairs = count * size * (size - 1) // 2
+    assert same(h, 2) == pairs
+
+
+def test_refused():
+    lib = slg.load()
+    dh = slg.to_device(hg.uniform(50, 80, 1, 5, seed=2))
+    n = ctypes.c_int64(0)
+    cb = slg._AllocFn(lambda *a: 1)
+    args = (ctypes.byref(dh.struct), 1)
+    tail = (None, cb, None, ctypes.byref(n), None)
+    assert lib.slg_build_alloc(*args, slg.SLG_ALGO_PLAIN, *tail) == 6
+    assert lib.slg_build_alloc(*args, slg.SLG_RELABEL_ASC, *tail) == 6
+    assert lib.slg_build_alloc(*args, 0, *tail) == 3  # no memory
+    nothing = slg._AllocFn(lambda *a: 0)  # no arrays given
+    assert lib.slg_build_alloc(*args, 0, None, nothing, None, ctypes.byref(n), None) == 1
+    with pytest.raises(slg.SlgError) as ei:
+        slg.build(dh, 0)
+    assert ei.value.status == 1
