@@ -528,12 +528,12 @@ int run_binned(Call &c, int64_t *result) {
   }
   // (core rows may have no wedges but still need a giant CTA; their pairs,
   // staged in the same scratch, also come from up to n_core tile items)
-  // (a sparse-bin row whose candidates overflow its table is handed to the
-  // giant bin, so the giant scratch also covers the sparse rows)
+  // (a row of the sparse or rows bin that overflows its table is handed to
+  // the giant bin, so the giant scratch also covers these rows)
   const Meta &mp = *c.meta_host;
   const int32_t max_giant =
-      (mp.rows_bin[kBinGiant] || mp.rows_bin[kBinSparse])
-          ? std::max(std::max(mp.max_giant_work, mp.max_sparse_work), (int32_t)1) +
+      (mp.rows_bin[kBinGiant] || mp.rows_bin[kBinSparse] || mp.rows_bin[kBinRows])
+          ? std::max(std::max(mp.max_giant_work, mp.max_sparse_work), kCtaSMaxWork) +
                 (core.T ? core.n_core : 0)
           : 0;
   // the giant bin's list as planned (the walk may append overflow rows)
@@ -556,11 +556,12 @@ int run_binned(Call &c, int64_t *result) {
   L.w.c_idx_s = w.c_idx_s;
   L.w.tail_beg = w.tail_beg;
   L.w.tail_end = w.tail_end;
-  for (int b : {kBinWarp, kBinCtaS, kBinCtaL})
+  for (int b : {kBinWarp, kBinCtaS, kBinCtaL, kBinRows})
     if (!mp.rows_bin[b]) L.skip |= 1u << b;
   if (!mp.sparse_huge) L.skip |= kSkipSparseBig;
   if (!mp.sparse_rest) L.skip |= kSkipSparseSmall;
-  if (!mp.rows_bin[kBinGiant] && !mp.rows_bin[kBinSparse]) L.skip |= 1u << kBinGiant;
+  if (!mp.rows_bin[kBinGiant] && !mp.rows_bin[kBinSparse] && !mp.rows_bin[kBinRows])
+    L.skip |= 1u << kBinGiant;
   cudaEvent_t *ev = c.evs->on ? c.evs->ev + kEvWalk : nullptr;
   if (c.rows > 0) {
     SLG_TRY(launch_walk(L, c.st, &c.launches, ev));
@@ -1016,7 +1017,12 @@ int run(const slg_hypergraph *h, int32_t smin, uint32_t flags, int32_t row_begin
     stats.incid_bin[b] = (int64_t)m.incid_bin[b];
     stats.pairs_bin[b] = (int64_t)m.pairs_bin[b];
   }
-  // the dense bin's rows are reported as giant ones
+  // the rows bin's rows are reported as the small CTA bin's, the dense
+  // bin's as giant ones
+  stats.rows_bin[kBinCtaS] += (int64_t)m.rows_bin[kBinRows];
+  stats.wedges_bin[kBinCtaS] += (int64_t)m.wedges_bin[kBinRows];
+  stats.incid_bin[kBinCtaS] += (int64_t)m.incid_bin[kBinRows];
+  stats.pairs_bin[kBinCtaS] += (int64_t)m.pairs_bin[kBinRows];
   stats.rows_bin[kBinGiant] += (int64_t)m.rows_bin[kBinDense];
   stats.wedges_bin[kBinGiant] += (int64_t)m.wedges_bin[kBinDense];
   stats.incid_bin[kBinGiant] += (int64_t)m.incid_bin[kBinDense];

@@ -23,11 +23,13 @@ constexpr int32_t kEmpty = -1;
 // kDenseMinWork wedges whose far ends are dense in their id span (is_dense)
 // go to the dense bin; of the others, rows with s >= 2 from Bins::bloom up to
 // Bins::sparse wedges go to the sparse bin and the rest above the CTA bins to
-// the giant bin.  The statistics count the dense bin's rows as giant ones
-// (kNumBins bins are reported, kNumLists lists are kept).
+// the giant bin.  Rows with s >= 2 of at most Bins::ctas
+// wedges take the rows bin (a warp each), s = 1 ones the warp and CTA bins.
+// The statistics count the dense bin's rows as giant ones and the rows bin's
+// as the small CTA bin's (kNumBins bins are reported, kNumLists lists kept).
 enum Bin : int {
   kBinWarp = 0, kBinCtaS = 1, kBinCtaL = 2, kBinGiant = 3, kBinSparse = 4, kNumBins = 5,
-  kBinDense = 5, kNumLists = 6
+  kBinDense = 5, kBinRows = 6, kNumLists = 7
 };
 
 // Upper bounds on a row's wedge count for each non-giant bin.  The hash tables
@@ -601,6 +603,7 @@ constexpr int32_t kComponentsMaxR = 1 << 24;
 constexpr int kWalkEv[kNumBins] = {0, 1, 2, 4, 3};
 cudaError_t launch_walk(const WalkLaunch &L, cudaStream_t st, int32_t *launches,
                         cudaEvent_t *ev = nullptr);
+cudaError_t launch_walk_rows(const WalkLaunch &L, cudaStream_t st);
 cudaError_t launch_walk_sparse(const WalkLaunch &L, cudaStream_t st, int32_t *launches);
 cudaError_t launch_walk_dense(const WalkLaunch &L, cudaStream_t st, int32_t *launches);
 cudaError_t launch_row_scan(int32_t rows, const Work &w, cudaStream_t st);

@@ -387,6 +387,8 @@ __global__ __launch_bounds__(kRowsNT) void k_rows_work(Side s, int32_t smin, int
         my_bin = kBinDense;
       else if (!forced && my_work > bins.bloom && my_work <= bins.sparse && se >= 2)
         my_bin = kBinSparse;
+      else if (!forced && my_work <= bins.ctas && se >= 2)
+        my_bin = kBinRows;
       if (my_bin == kBinGiant) atomicMax(&s_max[1], my_work);
       if (my_bin == kBinSparse) atomicMax(&s_max[2], my_work);
       if (my_bin == kBinDense) {
@@ -404,7 +406,7 @@ __global__ __launch_bounds__(kRowsNT) void k_rows_work(Side s, int32_t smin, int
   __syncthreads();
   if (threadIdx.x < kNumLists) {
     const int b = threadIdx.x;
-    if (b < kBinGiant) {
+    if (b < kBinGiant || b == kBinRows) {
       s_base[b] = s_cnt[b] ? (int32_t)atomicAdd(&meta->rows_bin[b], (unsigned long long)s_cnt[b]) : 0;
     } else {
       // the huge rows of the giant, sparse and dense bins fill their list from
@@ -443,7 +445,7 @@ __global__ __launch_bounds__(kRowsNT) void k_rows_work(Side s, int32_t smin, int
     const int64_t len = row_end - row_begin;
     int64_t pos = s_base[my_bin] + my_slot;
     if (huge) pos = s_hbase[my_bin - kBinGiant] + my_slot;
-    else if (my_bin >= kBinGiant) pos = len - 1 - pos;
+    else if (my_bin >= kBinGiant && my_bin != kBinRows) pos = len - 1 - pos;
     bin_rows[(int64_t)my_bin * len + pos] = r0 + threadIdx.x;
   }
 }

@@ -12,7 +12,9 @@
 //                               pairs in shared memory;
 //   dense bin  (slg_dense.cu):  rows with enough wedges for their id span are
 //                               counted in windows of packed counters;
-//   sparse bin (slg_sparse.cu): other rows with s >= 2, up to 16,384 wedges;
+//   sparse bin (slg_sparse.cu): other rows with s >= 2, up to 65,536 wedges;
+//   rows bin   (slg_sparse.cu): rows with s >= 2 and work <= 1024, a warp each
+//                               (the warp and CTA bins keep the s = 1 rows);
 //   giant bin  (the rest):      a CTA splits the row's far ends into f-range
 //                               buckets through a per-CTA global scratch and
 //                               counts each bucket, in ascending f, in the
@@ -714,6 +716,11 @@ cudaError_t launch_walk(const WalkLaunch &L, cudaStream_t st, int32_t *launches,
     ++n;
   }
   if (ev) cudaEventRecord(ev[1], st);
+  if (!empty(kBinRows)) {
+    const cudaError_t e = launch_walk_rows(L, st);
+    if (e != cudaSuccess) return e;
+    ++n;
+  }
   if (!empty(kBinCtaS)) {
     K_CTA_S<<<o.sms * (o.s_blocks > 0 ? o.s_blocks : 1), 256, CfgS::smem(), st>>>(
         L.w, lists + 1 * stride, L.row_work, L.a);

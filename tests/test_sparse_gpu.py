@@ -211,3 +211,34 @@ def test_tails_set_aside_large_rows(aside_large, s):
     assert slg.last_stats()["rows_bin"][4] > 0
     assert np.array_equal(got[np.isin(got[:, 0], rows)], want)
     assert slg.count(dh, s) == got.shape[0]
+
+
+# the rows bin: one batch of 32 tails and one more, wedges up to its limit of
+# 1,024, more far ends of two wedges than its table of 256 holds (handed over)
+@pytest.mark.parametrize("k,deg", [(2, 500), (2, 512), (31, 33), (32, 32), (33, 31), (40, 25),
+                                   (3, 120)])
+def test_short_rows(k, deg):
+    rng = np.random.default_rng(k * deg)
+    m, n, hubs = 60_000, 200_000, 40
+    r, c = [], []
+    for hub in range(hubs):  # row `hub`: k vertices of `deg` other hyperedges each
+        v = 1_000 + hub * k + np.arange(k)
+        r.append(np.full(k, hub))
+        c.append(v)
+        far = rng.choice(np.arange(hubs, m), deg, replace=False)
+        for x in range(k):  # the same far ends for the first two vertices
+            f = far if x < 2 else rng.choice(np.arange(hubs, m), deg, replace=False)
+            r.append(f)
+            c.append(np.full(deg, v[x]))
+    size = rng.integers(4, 8, m)
+    r.append(np.repeat(np.arange(m), size))
+    c.append(rng.integers(10_000, n, int(size.sum())))
+    h = hg.from_pairs(np.concatenate(r), np.concatenate(c), m, n)
+    dh = slg.to_device(h)
+    for s in (2, 3, 4, 6):
+        want = oracle.canonical(*oracle.line_graph_of(h, s, threads=8))
+        assert np.array_equal(as_np(slg.build(dh, s)), want), s
+        i, j, w = slg.build(dh, s, unweighted=True)
+        assert w is None and np.array_equal(
+            np.stack([i.cpu().numpy(), j.cpu().numpy()], 1), want[:, :2])
+        assert slg.count(dh, s) == want.shape[0]
