@@ -326,27 +326,40 @@ cudaError_t ensure_scratch(Call &c, size_t *summ_off) {
   return ensure_giant(*c.ctx, counters + pw * (rp >> 10), c.st);
 }
 
-// Scratch of the sparse, giant and dense bins (their kernels run one after the
-// other and share it): 4 ints per wedge of the largest giant row and giant CTA;
-// the dense bin's per-CTA need for its largest row.  Sets L's dense_pairs,
-// dense_size and giant_stride and returns the ints.
+// Scratch of the sparse, dense and giant bins: the first two side by side
+// (their kernels run concurrently), the giant bin's (4 ints per wedge of the
+// largest giant row and giant CTA) in the same place, since its kernel runs
+// after them.  Sets L's sizes and returns the ints; place_scratch sets its
+// pointers.
+long long up32(long long n) { return (n + 31) & ~31ll; }
+
 size_t scratch_ints(WalkLaunch *L, int32_t max_giant, int32_t max_sparse, long long pairs_big,
                     long long pairs_small, int32_t dense_size) {
   L->giant_stride = 4ll * max_giant;
   L->dense_pairs[0] = pairs_big;
   L->dense_pairs[1] = pairs_small;
   L->dense_size = dense_size;
-  const size_t sp = max_sparse > 0 ? (size_t)sparse_ints(max_sparse) : 0;
-  return std::max(std::max((size_t)giant_ctas() * (size_t)L->giant_stride, sp),
-                  (size_t)dense_ints(pairs_big, pairs_small, dense_size));
+  L->sparse_ints = max_sparse > 0 ? sparse_ints(max_sparse) : 0;
+  const long long side = up32(dense_ints(0, pairs_big, dense_size)) +
+                         up32(dense_ints(1, pairs_small, dense_size)) + L->sparse_ints;
+  return (size_t)std::max((long long)giant_ctas() * L->giant_stride, side);
+}
+
+void place_scratch(WalkLaunch *L, int32_t *base) {
+  L->giant_scratch = base;
+  L->dense_scratch[0] = base;
+  L->dense_scratch[1] = base + up32(dense_ints(0, L->dense_pairs[0], L->dense_size));
+  int32_t *sp = L->dense_scratch[1] + up32(dense_ints(1, L->dense_pairs[1], L->dense_size));
+  L->sparse_scratch = L->sparse_ints > 0 ? sp : nullptr;
 }
 
 cudaError_t giant_scratch(Call &c, int32_t max_giant, int32_t max_sparse, long long pairs_big,
                           long long pairs_small, int32_t dense_size, WalkLaunch *L) {
-  L->giant_scratch = nullptr;
   const size_t n = scratch_ints(L, max_giant, max_sparse, pairs_big, pairs_small, dense_size);
-  L->scratch_ints = (long long)n;
-  return n ? c.pool->get(&L->giant_scratch, n) : cudaSuccess;
+  int32_t *base = nullptr;
+  const cudaError_t e = n ? c.pool->get(&base, n) : cudaSuccess;
+  if (base) place_scratch(L, base);
+  return e;
 }
 
 thread_local int32_t t_err_where = 0;  // kWhere* of the last device-raised error
@@ -1098,7 +1111,7 @@ struct slg_plan {
   int32_t *row_base = nullptr;     // [count + 1] first row of each member (side)
   slg::Work w = {};
   int32_t *giant = nullptr;
-  slg::WalkLaunch scratch = {};    // giant_stride, dense_pairs, dense_size, scratch_ints
+  slg::WalkLaunch scratch = {};    // giant_stride, dense_pairs, dense_size, sparse_ints
   int32_t *out_i = nullptr, *out_j = nullptr, *out_w = nullptr;
   long long *offsets = nullptr;    // [count + 1]
   int64_t pairs = 0;
@@ -1151,12 +1164,12 @@ cudaError_t enqueue_plan(slg_plan *p, const Bins &bins, cudaStream_t st, int32_t
   L.row_work = w.row_work;
   L.rows = sd.R;
   L.R = sd.R;
-  L.giant_scratch = p->giant;
   L.giant_stride = p->scratch.giant_stride;
   L.dense_pairs[0] = p->scratch.dense_pairs[0];
   L.dense_pairs[1] = p->scratch.dense_pairs[1];
   L.dense_size = p->scratch.dense_size;
-  L.scratch_ints = p->scratch.scratch_ints;
+  L.sparse_ints = p->scratch.sparse_ints;
+  if (p->giant) place_scratch(&L, p->giant);
   int32_t n = 0;
   if (sd.R > 0) PLAN_TRY(launch_walk(L, st, &n));
   PLAN_TRY(launch_row_scan(sd.R, w, st));
@@ -1911,7 +1924,6 @@ extern "C" int slg_plan_create(const slg_hypergraph *hs, const int32_t *s, int32
   if (max_work > 0) {
     const size_t n = scratch_ints(&p->scratch, max_work, max_work, std::min<long long>(max_work, R),
                                   std::min<long long>(max_work, R), max_size);
-    p->scratch.scratch_ints = (long long)n;
     SLG_TRY(p->mem.get(&p->giant, n));
   }
   // 4. autotuner: bin thresholds, timed on this batch

@@ -427,34 +427,29 @@ long long dense_stride(long long max_pairs, int32_t max_size, long long *pair_ca
 
 }  // namespace
 
-// The two instances run one after the other and share the scratch.
-long long dense_ints(long long pairs_big, long long pairs_small, int32_t size_big) {
+// Scratch ints of an instance (small: 0 the big one, 1 the other).
+long long dense_ints(int small, long long pairs, int32_t size_big) {
+  if (pairs <= 0) return 0;
   DnOcc &o = dn_occ();
   long long pc = 0;
   int32_t ec = 0;
-  const long long b = pairs_big > 0 ? o.big * dense_stride<DnBig>(pairs_big, size_big, &pc, &ec) : 0;
-  const long long s = pairs_small > 0
-                          ? o.small * dense_stride<DnSmall>(pairs_small, kDenseBigSize, &pc, &ec)
-                          : 0;
-  return std::max(b, s);
+  return small ? o.small * dense_stride<DnSmall>(pairs, kDenseBigSize, &pc, &ec)
+               : o.big * dense_stride<DnBig>(pairs, size_big, &pc, &ec);
 }
 
-cudaError_t launch_walk_dense(const WalkLaunch &L, cudaStream_t st, int32_t *launches) {
+cudaError_t launch_walk_dense(const WalkLaunch &L, int small, cudaStream_t st) {
   DnOcc &o = dn_occ();
   const int32_t *rows = L.bin_rows + (int64_t)kBinDense * L.rows;
   long long pc = 0;
   int32_t ec = 0;
-  if (L.dense_pairs[0] > 0) {
+  if (!small) {
     const long long stride = dense_stride<DnBig>(L.dense_pairs[0], L.dense_size, &pc, &ec);
     k_walk_dense<DnBig><<<o.big, DnBig::NT, dense_smem<DnBig>(), st>>>(
-        L.w, rows, L.a, L.giant_scratch, stride, pc, ec, L.R, L.rows, 0);
-    ++*launches;
-  }
-  if (L.dense_pairs[1] > 0) {
+        L.w, rows, L.a, L.dense_scratch[0], stride, pc, ec, L.R, L.rows, 0);
+  } else {
     const long long stride = dense_stride<DnSmall>(L.dense_pairs[1], kDenseBigSize, &pc, &ec);
     k_walk_dense<DnSmall><<<o.small, DnSmall::NT, dense_smem<DnSmall>(), st>>>(
-        L.w, rows, L.a, L.giant_scratch, stride, pc, ec, L.R, L.rows, 1);
-    ++*launches;
+        L.w, rows, L.a, L.dense_scratch[1], stride, pc, ec, L.R, L.rows, 1);
   }
   return cudaGetLastError();
 }

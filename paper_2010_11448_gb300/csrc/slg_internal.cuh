@@ -553,10 +553,12 @@ struct WalkLaunch {
   const int32_t *bin_rows;  // [kNumLists][rows] row lists
   const int32_t *row_work;  // [rows] wedges per row
   int32_t rows;             // rows in the range (list stride)
-  int32_t *giant_scratch;   // [giant_ctas][4 * max giant work] wedge ends + pairs
+  int32_t *giant_scratch;   // [giant_ctas][4 * max giant work] wedge ends + pairs; before the
+                            // giant kernel, the other bins' scratch one behind the other
   long long giant_stride;   // ints per giant CTA
   int32_t R;                // rows of the side (far ends lie in [0, R))
-  long long scratch_ints;   // of giant_scratch
+  int32_t *dense_scratch[2], *sparse_scratch;  // in giant_scratch
+  long long sparse_ints;    // of sparse_scratch
   long long dense_pairs[2]; // most pairs a dense-bin row can have: big instance, other (0: no row)
   int32_t dense_size;       // most vertices of a dense-bin row
   unsigned skip;            // bit b: bin b is known to be empty (kSkipSparseBig, ...)
@@ -590,7 +592,7 @@ cudaError_t launch_small(const SmallCall &c, cudaStream_t st, int32_t *launches,
 // kernels.
 int giant_ctas();
 long long sparse_ints(int32_t max_work);
-long long dense_ints(long long pairs_big, long long pairs_small, int32_t size_big);
+long long dense_ints(int small, long long pairs, int32_t size_big);
 // The largest side (rows) a build supports: row ids and the giant bin's
 // super-chunk bounds stay below 2^31.
 constexpr int32_t kMaxRows = (int32_t)((1u << 31) - (1u << 23));
@@ -605,7 +607,7 @@ cudaError_t launch_walk(const WalkLaunch &L, cudaStream_t st, int32_t *launches,
                         cudaEvent_t *ev = nullptr);
 cudaError_t launch_walk_rows(const WalkLaunch &L, cudaStream_t st);
 cudaError_t launch_walk_sparse(const WalkLaunch &L, cudaStream_t st, int32_t *launches);
-cudaError_t launch_walk_dense(const WalkLaunch &L, cudaStream_t st, int32_t *launches);
+cudaError_t launch_walk_dense(const WalkLaunch &L, int small, cudaStream_t st);
 cudaError_t launch_row_scan(int32_t rows, const Work &w, cudaStream_t st);
 // The device Meta into host memory the device can address (mapped pinned
 // memory), by a kernel: no copy engine involved.

@@ -188,7 +188,7 @@ __device__ __forceinline__ int32_t lower_pos(const int32_t *__restrict__ a, int3
 
 // part 0: the rows above kSparseBigWork wedges (the front of the list), 1: the
 // others (its back), each on its own ticket.  buf: the CTA's share of the
-// giant bin's scratch (free while this kernel runs), for the pairs of rows of
+// bin's scratch, for the pairs of rows of
 // several ranges: buf_stride ints, at least the largest row's work.
 template <class C>
 __global__ __launch_bounds__(C::NT, C::MINB) void k_walk_sparse(
@@ -759,7 +759,7 @@ void sp_launch(const WalkLaunch &L, int ctas, int part, cudaStream_t st) {
   k_walk_sparse<C><<<ctas, C::NT, sparse_smem<C>(), st>>>(
       L.w, L.bin_rows + (int64_t)kBinSparse * stride, L.a,
       const_cast<int32_t *>(L.bin_rows) + (int64_t)kBinGiant * stride, (int32_t)stride,
-      L.giant_scratch, (L.scratch_ints / (long long)ctas) & ~31ll, L.R, part);
+      L.sparse_scratch, (L.sparse_ints / (long long)ctas) & ~31ll, L.R, part);
 }
 
 }  // namespace
@@ -780,7 +780,7 @@ cudaError_t launch_walk_rows(const WalkLaunch &L, cudaStream_t st) {
 }
 
 cudaError_t launch_walk_sparse(const WalkLaunch &L, cudaStream_t st, int32_t *launches) {
-  if (!L.giant_scratch) return cudaSuccess;  // no row in the bin
+  if (!L.sparse_scratch) return cudaSuccess;  // no row in the bin
   SpOcc &o = sp_occ();
   if (!(L.skip & kSkipSparseBig)) {
     sp_launch<SpBig>(L, o.big, 0, st);

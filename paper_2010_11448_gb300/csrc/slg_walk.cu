@@ -702,48 +702,149 @@ int giant_ctas_for_device() {
 
 int giant_ctas() { return giant_ctas_for_device(); }
 
+namespace {
+
+// Two streams beside the caller's for the bins' kernels, and the events that
+// order them: this host thread's, made on first use on a device (one set per
+// thread; given back when the thread ends or turns to another device).
+struct SideStreams {
+  int dev = -1;
+  bool ok = false;
+  cudaStream_t s[2] = {nullptr, nullptr};
+  cudaEvent_t fork = nullptr, done[2] = {nullptr, nullptr};
+
+  void drop() {
+    for (cudaStream_t &x : s)
+      if (x) cudaStreamDestroy(x), x = nullptr;
+    for (cudaEvent_t *x : {&fork, &done[0], &done[1]})
+      if (*x) cudaEventDestroy(*x), *x = nullptr;
+    ok = false;
+  }
+  ~SideStreams() { drop(); }
+
+  // Whether they can be forked from st.  A stream that was forked into a
+  // capture stays in it until the capture ends, so in the meantime they serve
+  // that capture only.
+  bool ready(cudaStream_t st) {
+    int d = 0;
+    if (cudaGetDevice(&d) != cudaSuccess) return false;
+    if (d != dev) {
+      drop();
+      dev = d;
+      ok = true;
+      cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+      cudaThreadExchangeStreamCaptureMode(&mode);
+      for (cudaStream_t &x : s)
+        ok &= cudaStreamCreateWithFlags(&x, cudaStreamNonBlocking) == cudaSuccess;
+      for (cudaEvent_t *x : {&fork, &done[0], &done[1]})
+        ok &= cudaEventCreateWithFlags(x, cudaEventDisableTiming) == cudaSuccess;
+      cudaThreadExchangeStreamCaptureMode(&mode);
+      if (!ok) {
+        drop();
+        cudaGetLastError();
+      }
+    }
+    for (int i = 0; ok && i < 2; ++i) {
+      cudaStreamCaptureStatus a = cudaStreamCaptureStatusNone, b = a;
+      unsigned long long ia = 0, ib = 0;
+      if (cudaStreamGetCaptureInfo(s[i], &a, &ia) != cudaSuccess) return cudaGetLastError(), false;
+      if (a == cudaStreamCaptureStatusNone) continue;
+      if (cudaStreamGetCaptureInfo(st, &b, &ib) != cudaSuccess) return cudaGetLastError(), false;
+      if (a != cudaStreamCaptureStatusActive || b != a || ia != ib) return false;
+    }
+    return ok;
+  }
+};
+
+}  // namespace
+
+// The bins' kernels are independent of each other (each keeps its rows, its
+// tickets and its part of the scratch; the totals are atomic), except the
+// giant kernel, which also takes the rows that others handed over.  Each is
+// sized to fill the device, but the long rows of DnBig (a CTA per SM) leave
+// most of it idle at the end, and on a mid-size graph from the start: so where
+// that bin has rows, the sparse bin and DnSmall run beside it on one stream
+// and the other bins on a second.  One after the other -> so: counting pass of
+// 120K x 240K 1,057 -> 800 us, host builds of 200K x 400K 4,157 -> 3,464,
+// 16-member batch 2,505 -> 2,150..2,198, L_3 of 500K x 1M in row form 6,092 ->
+// 5,777, L_1 of 100K x 200K 2,499 -> 2,287; chung_lu_1m's four lists 105.7 ms
+// both ways.  DnSmall beside the sparse bin costs more than it fills (L_2
+// sweep of 150K x 300K 10,190 -> 10,711 us), as does a fork without DnBig (L_3
+// of a dual of 30K x 60K 1,346 -> 1,362).  With per-bin timing (ev) they run
+// one after the other.
 cudaError_t launch_walk(const WalkLaunch &L, cudaStream_t st, int32_t *launches,
                         cudaEvent_t *ev) {
   Occ &o = occ_for_device();
   const int32_t *lists = L.bin_rows;
   const int64_t stride = L.rows;
   int n = 0;
-  if (ev) cudaEventRecord(ev[0], st);
+  cudaError_t err = cudaSuccess;
+  auto keep = [&](cudaError_t e) {
+    if (err == cudaSuccess) err = e;
+  };
   auto empty = [&](int bin) { return (L.skip >> bin) & 1u; };
+  static thread_local SideStreams side;
+  const bool has_sparse = L.sparse_scratch && (L.skip & (kSkipSparseBig | kSkipSparseSmall)) !=
+                                                  (kSkipSparseBig | kSkipSparseSmall);
+  const bool dense_big = L.dense_pairs[0] > 0, dense_small = L.dense_pairs[1] > 0;
+  const bool chain = has_sparse || dense_small;
+  const bool ctas = !empty(kBinWarp) || !empty(kBinCtaS) || !empty(kBinCtaL) || !empty(kBinRows);
+  const bool fork = !ev && dense_big && (chain || ctas) && side.ready(st);
+  const bool use[2] = {fork && chain, fork && ctas};
+  cudaStream_t s1 = use[0] ? side.s[0] : st, s2 = use[1] ? side.s[1] : st;
+  if (fork) keep(cudaEventRecord(side.fork, st));
+  for (int i = 0; i < 2; ++i)
+    if (use[i]) keep(cudaStreamWaitEvent(side.s[i], side.fork, 0));
+  if (err != cudaSuccess) return err;  // nothing was launched
+  if (ev) cudaEventRecord(ev[0], st);
+  // rows with the longest run first
+  if (!ev && dense_big) {
+    keep(launch_walk_dense(L, 0, st));
+    ++n;
+  }
+  if (!ev && has_sparse) keep(launch_walk_sparse(L, s1, &n));
   if (!empty(kBinWarp)) {
-    k_walk_warp<<<o.sms * (o.warp_blocks > 0 ? o.warp_blocks : 1), kWarpNT, 0, st>>>(
+    k_walk_warp<<<o.sms * (o.warp_blocks > 0 ? o.warp_blocks : 1), kWarpNT, 0, s2>>>(
         L.w, lists + 0 * stride, L.a);
     ++n;
   }
   if (ev) cudaEventRecord(ev[1], st);
   if (!empty(kBinRows)) {
-    const cudaError_t e = launch_walk_rows(L, st);
-    if (e != cudaSuccess) return e;
+    keep(launch_walk_rows(L, s2));
     ++n;
   }
   if (!empty(kBinCtaS)) {
-    K_CTA_S<<<o.sms * (o.s_blocks > 0 ? o.s_blocks : 1), 256, CfgS::smem(), st>>>(
+    K_CTA_S<<<o.sms * (o.s_blocks > 0 ? o.s_blocks : 1), 256, CfgS::smem(), s2>>>(
         L.w, lists + 1 * stride, L.row_work, L.a);
     ++n;
   }
   if (ev) cudaEventRecord(ev[2], st);
   if (!empty(kBinCtaL)) {
-    K_CTA_L<<<o.sms * (o.l_blocks > 0 ? o.l_blocks : 1), 256, CfgL::smem(), st>>>(
+    K_CTA_L<<<o.sms * (o.l_blocks > 0 ? o.l_blocks : 1), 256, CfgL::smem(), s2>>>(
         L.w, lists + 2 * stride, L.row_work, L.a);
     ++n;
   }
   if (ev) cudaEventRecord(ev[3], st);
-  // the sparse bin before the giant bin: a sparse row whose candidates
-  // overflow its table is appended to the giant bin's list
-  {
-    const cudaError_t e = launch_walk_sparse(L, st, &n);
-    if (e != cudaSuccess) return e;
-  }
+  if (ev && has_sparse) keep(launch_walk_sparse(L, st, &n));
   if (ev) cudaEventRecord(ev[4], st);
-  if (L.giant_scratch) {
-    const cudaError_t e = launch_walk_dense(L, st, &n);
-    if (e != cudaSuccess) return e;
+  if (ev && dense_big) {
+    keep(launch_walk_dense(L, 0, st));
+    ++n;
   }
+  if (dense_small) {
+    keep(launch_walk_dense(L, 1, s1));
+    ++n;
+  }
+  keep(cudaGetLastError());
+  for (int i = 0; i < 2; ++i) {
+    if (!use[i]) continue;
+    // joined also after an error: nothing may run on when the call returns
+    cudaError_t e = cudaEventRecord(side.done[i], side.s[i]);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(st, side.done[i], 0);
+    if (e != cudaSuccess) cudaStreamSynchronize(side.s[i]);
+    keep(e);
+  }
+  if (err != cudaSuccess) return err;
   if (L.giant_scratch && L.giant_stride > 0 && !empty(kBinGiant)) {
     k_walk_giant<<<o.sms * o.g_blocks, kGiantNT, giant_smem(), st>>>(
         L.w, lists + 3 * stride, L.a, L.giant_scratch, L.giant_stride, L.R, (int32_t)stride);
