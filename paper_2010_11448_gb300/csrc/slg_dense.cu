@@ -37,6 +37,17 @@
 // dual 10.98 -> 9.53 ms, step of chung_lu_1m 118.4 -> 115.1 ms with four
 // of 256 threads (five with 8,192 words: 9.83, 117.6; eight of 128 threads
 // with 4,608 words: 8.86, 118.8).
+//
+// The longest tails are split over the warps in blocks of 32 entries, a
+// cursor per warp.  They had been cut into runs of 256 entries per window, of
+// which a window meets only some, so that its warps waited for one another
+// (barriers were half of a warp's time): L_2 sweep of a 150K x 300K dual
+// 10,134 -> 9,351 us (11,383 with the tails left whole), L_3 of a 30K x 60K
+// dual 1,346 -> 1,322 (1,702).  From 128, 256, 512 entries per window: sweep
+// 9,651, 9,661, 9,866 us, step of chung_lu_1m 106.3, 105.7, 105.7 ms.  4-bit
+// counters tried first for rows of 16 to 64 vertices, the row counted anew on
+// an overflow, gave 3 % on the sweep, nothing elsewhere, and lose where rows
+// are alike: not kept.
 #include <algorithm>
 #include <mutex>
 
@@ -55,82 +66,109 @@ namespace {
 #ifndef SLG_DN_LONG
 #define SLG_DN_LONG 16
 #endif
-#ifndef SLG_DN_SEG
-#define SLG_DN_SEG 256
+#ifndef SLG_DN_SPLIT
+#define SLG_DN_SPLIT 256
+#endif
+#ifndef SLG_DN_BIG_SPLIT
+#define SLG_DN_BIG_SPLIT 1024
 #endif
 #ifndef SLG_DN_US
-#define SLG_DN_US 4
+#define SLG_DN_US 2
 #endif
 #ifndef SLG_DN_UL
 #define SLG_DN_UL 2
 #endif
-constexpr int kDnSeg = SLG_DN_SEG;            // a tail's entries per window and list entry, about
-constexpr int kDnUS = SLG_DN_US;              // short entries in flight per 8 lanes
-constexpr int kDnUL = SLG_DN_UL;              // long entries in flight per warp
 
 // The two instances of the kernel: NT threads, WORDS counter words per
 // window, MAP words of survivor bits (counters of at least 32 WORDS / (32
-// MAP) bits), MINB CTAs per SM, ENT list entries in shared memory, EXTRA of
-// them beyond one per tail.
+// MAP) bits), MINB CTAs per SM, ENT list entries in shared memory, NSPLIT
+// split tails at most, from SPLIT entries per window.
 struct DnSmall {
   static constexpr int NT = SLG_DN_NT, MINB = SLG_DN_MINB, WORDS = SLG_DN_WORDS, MAP = WORDS / 4;
-  static constexpr int EXTRA = 128, ENT = kDenseBigSize + EXTRA + 1;
+  static constexpr int NSPLIT = 16, SPLIT = SLG_DN_SPLIT, UL = SLG_DN_UL, US = SLG_DN_US;
+  static constexpr int ENT = kDenseBigSize + 1;
 };
 struct DnBig {
   static constexpr int NT = 1024, MINB = 1, WORDS = SLG_DN_BIG_WORDS, MAP = WORDS / 16;
-  static constexpr int EXTRA = 512, ENT = 1024;
+  static constexpr int NSPLIT = 16, SPLIT = SLG_DN_BIG_SPLIT, UL = 2, US = 4;
+  static constexpr int ENT = 512;
 };
 
-// [counters][survivor bits][entries C::ENT x 8][totals 2 x 32 x 4]
-// [n_long, n_short, row, pad][base 8]
+// [counters][survivor bits][entries C::ENT x 8][split cursors NSPLIT x NW x 8]
+// [totals 2 x 32 x 4][n_long, n_short, row, n_split][base 8]
 template <class C>
 constexpr size_t dense_smem() {
   static_assert(C::WORDS % 64 == 0, "16-byte alignment of the parts");
-  return (size_t)C::WORDS * 4 + (size_t)C::MAP * 4 + (size_t)C::ENT * 8 + 2 * 32 * 4 + 16 + 16;
+  return (size_t)C::WORDS * 4 + (size_t)C::MAP * 4 + (size_t)C::ENT * 8 +
+         (size_t)C::NSPLIT * (C::NT / 32) * 8 + 2 * 32 * 4 + 16 + 16;
 }
 
-// Adds n to counter o (2^LB bits wide, packed in 32-bit words) and marks o in
-// the survivor bits when this takes it to s or above.
+// Adds n to counter o (2^LB bits wide, packed in 32-bit words); when this
+// takes it to s or above, marks o in the survivor bits and returns 1.
 template <int LB>
-__device__ __forceinline__ bool dn_add(uint32_t *cnt, uint32_t *map, int32_t o, uint32_t n,
-                                       uint32_t smin, bool mark) {
+__device__ __forceinline__ int32_t dn_add(uint32_t *cnt, uint32_t *map, int32_t o, uint32_t n,
+                                          uint32_t smin, bool mark) {
   constexpr int LW = 5 - LB;                     // log2 counters per word
   constexpr uint32_t kField = LB == 5 ? ~0u : (1u << ((1 << LB) & 31)) - 1u;
   const int sh = (o & ((1 << LW) - 1)) << LB;
   const uint32_t old = (atomicAdd(cnt + (o >> LW), n << sh) >> sh) & kField;
-  const bool hit = old < smin && old + n >= smin;
-  if (hit && mark) atomicOr(map + (o >> 5), 1u << (o & 31));
-  return hit;
+  if (!(old < smin && old + n >= smin)) return 0;
+  if (mark) atomicOr(map + (o >> 5), 1u << (o & 31));
+  return 1;
 }
 
 // One window's sweep over the row's list entries; the counters of ids
 // [F0, F1).  Returns the thread's number of survivors; *any: something was
 // counted.  Bound by the latency of the cursor and far-end loads, so several
 // entries' loads are in flight per warp.
-template <int LB, int NW>
+template <int LB, class C>
 __device__ __forceinline__ int32_t dn_sweep(const int32_t *__restrict__ c_idx, int2 *ent,
-                                            int32_t nl, int2 *ent_s, int32_t ns, int32_t F0,
-                                            int32_t F1, uint32_t *cnt, uint32_t *map,
-                                            uint32_t smin, bool mark, bool *any) {
+                                            int32_t nl, int2 *ent_s, int32_t ns, int2 *split,
+                                            int32_t nh, int32_t F0, int32_t F1, uint32_t *cnt,
+                                            uint32_t *map, uint32_t smin, bool mark, bool *any) {
+  constexpr int NW = C::NT / 32, UL = C::UL, US = C::US;
   const int32_t lane = (int32_t)(threadIdx.x & 31), wq = (int32_t)(threadIdx.x >> 5);
   int32_t c = 0;
+  // split tails: every warp takes each NW-th block of 32 entries, two blocks
+  // per step; the block in which the window ends is read again by the next
+  const uint32_t span = (uint32_t)(F1 - F0);
+  for (int32_t x = 0; x < nh; ++x) {
+    const int2 en = split[x * NW + wq];
+    // unsigned: a cursor may lie 64 NW beyond the last incidence
+    const uint32_t end = (uint32_t)en.y;
+    uint32_t cur = (uint32_t)en.x;
+    for (;;) {  // warp-uniform
+      const uint32_t i = cur + lane;
+      const int32_t a = i < end ? __ldg(c_idx + i) : 0x7fffffff;
+      const int32_t b = i + 32 * NW < end ? __ldg(c_idx + i + 32 * NW) : 0x7fffffff;
+      const bool v0 = (uint32_t)(a - F0) < span, v1 = (uint32_t)(b - F0) < span;
+      if (v0) c += dn_add<LB>(cnt, map, a - F0, 1u, smin, mark);
+      if (v1) c += dn_add<LB>(cnt, map, b - F0, 1u, smin, mark);
+      *any |= v0 | v1;
+      if (!__all_sync(0xffffffffu, a < F1)) break;
+      cur += 32 * NW;
+      if (!__all_sync(0xffffffffu, b < F1)) break;
+      cur += 32 * NW;
+    }
+    if (cur != (uint32_t)en.x && lane == 0) split[x * NW + wq].x = (int32_t)cur;
+  }
   // long tails, a warp each, 64 entries per step
-  for (int32_t x0 = wq; x0 < nl; x0 += kDnUL * NW) {
-    int2 en[kDnUL];
-    int32_t f[kDnUL][2];
+  for (int32_t x0 = wq; x0 < nl; x0 += UL * NW) {
+    int2 en[UL];
+    int32_t f[UL][2];
 #pragma unroll
-    for (int u = 0; u < kDnUL; ++u) {
+    for (int u = 0; u < UL; ++u) {
       const int32_t x = x0 + u * NW;
       en[u] = x < nl ? ent[x] : make_int2(0, 0);
     }
 #pragma unroll
-    for (int u = 0; u < kDnUL; ++u) {
+    for (int u = 0; u < UL; ++u) {
       const int32_t i = en[u].x + lane;
       f[u][0] = i < en[u].y ? __ldg(c_idx + i) : 0x7fffffff;
       f[u][1] = i + 32 < en[u].y ? __ldg(c_idx + i + 32) : 0x7fffffff;
     }
 #pragma unroll
-    for (int u = 0; u < kDnUL; ++u) {
+    for (int u = 0; u < UL; ++u) {
       int32_t cur = en[u].x, a = f[u][0], b = f[u][1];
       for (;;) {  // warp-uniform
         const bool v0 = a < F1, v1 = b < F1;
@@ -152,21 +190,21 @@ __device__ __forceinline__ int32_t dn_sweep(const int32_t *__restrict__ c_idx, i
   }
   // short tails, 8 lanes each
   const int sub = lane >> 3, l8 = lane & 7;
-  for (int32_t x0 = wq * 4; x0 < ns; x0 += kDnUS * NW * 4) {
-    int2 en[kDnUS];
-    int32_t f[kDnUS];
+  for (int32_t x0 = wq * 4; x0 < ns; x0 += US * NW * 4) {
+    int2 en[US];
+    int32_t f[US];
 #pragma unroll
-    for (int u = 0; u < kDnUS; ++u) {
+    for (int u = 0; u < US; ++u) {
       const int32_t x = x0 + u * NW * 4 + sub;
       en[u] = x < ns ? ent_s[x] : make_int2(0, 0);
     }
 #pragma unroll
-    for (int u = 0; u < kDnUS; ++u) {
+    for (int u = 0; u < US; ++u) {
       const int32_t i = en[u].x + l8;
       f[u] = i < en[u].y ? __ldg(c_idx + i) : 0x7fffffff;
     }
 #pragma unroll
-    for (int u = 0; u < kDnUS; ++u) {
+    for (int u = 0; u < US; ++u) {
       int32_t cur = en[u].x, a = f[u];
       for (;;) {
         const bool v = a < F1;
@@ -200,8 +238,9 @@ __global__ __launch_bounds__(C::NT, C::MINB) void k_walk_dense(
   uint4 *cnt4 = reinterpret_cast<uint4 *>(smem);
   uint32_t *map = cnt + C::WORDS;
   int2 *s_ent = reinterpret_cast<int2 *>(map + C::MAP);
-  int32_t *s_tot = reinterpret_cast<int32_t *>(s_ent + C::ENT);
-  int32_t *s_n = s_tot + 64;  // [0] long entries, [1] short entries, [2] row
+  int2 *split = s_ent + C::ENT;
+  int32_t *s_tot = reinterpret_cast<int32_t *>(split + C::NSPLIT * NW);
+  int32_t *s_n = s_tot + 64;  // [0] long entries, [1] short entries, [2] row, [3] split tails
   long long *s_base = reinterpret_cast<long long *>(s_n + 4);
   // per-CTA global scratch: staged pairs (j, w), then the list entries of
   // rows with more tails than shared memory holds
@@ -223,6 +262,7 @@ __global__ __launch_bounds__(C::NT, C::MINB) void k_walk_dense(
       const unsigned t = atomicAdd(ticket, 1u);
       s_n[0] = 0;
       s_n[1] = 0;
+      s_n[3] = 0;
       s_n[2] = t >= nrows ? -1 : rows[part ? list_len - 1 - t : t];
     }
     __syncthreads();
@@ -233,57 +273,58 @@ __global__ __launch_bounds__(C::NT, C::MINB) void k_walk_dense(
     const int32_t f_lo = a.full_rows ? 0 : e + 1;
     const int32_t f_hi = a.row_fhi ? a.row_fhi[e] : R;
     const int32_t k0 = w.r_off[e], k1 = w.r_off[e + 1];
-    const int lb = dense_lg_bits(k1 - k0);
-    const int lw = 5 - lb;
-    const int32_t win = C::WORDS << lw;  // ids per window
-    const int32_t nwin = (f_hi - f_lo + win - 1) / win;
     const CoreInfo &ci = a.core;
     const bool core_row = ci.T && ci.row_rank[e + 1] != ci.row_rank[e];
     const int32_t ri = core_row ? ci.row_rank[e] : 0;
     const int32_t *Trow = core_row ? ci.T + (long long)ri * ci.Mp : nullptr;
     const long long dbase = a.mode == kDirect ? a.row_ptr[e - a.row_begin] : -1;
+    int32_t out = 0;  // pairs of the row so far
+    int32_t mine = 0;  // count mode: the thread's survivors
+    bool fail = false;
+    const int lb = dense_lg_bits(k1 - k0);
+    const int lw = 5 - lb;
+    const int32_t win = C::WORDS << lw;  // ids per window
+    const int32_t nwin = (f_hi - f_lo + win - 1) / win;
     // 1. the row's non-empty tails as list entries (cursor, end): the ones
     // with many entries per window from the front (a warp sweeps one), the
-    // others from the back (8 lanes sweep one).  A tail with more than seg
-    // entries is cut into several, so that no warp sweeps far more of a
-    // window than the others: at most (k1 - k0) + C::EXTRA entries.
-    const bool in_smem = k1 - k0 <= C::ENT - C::EXTRA;
+    // others from the back (8 lanes sweep one).  The longest, of which there
+    // can be fewer than NSPLIT, are split over all warps, with a cursor each,
+    // so that no warp sweeps far more of a window than the others.
+    const bool in_smem = k1 - k0 <= C::ENT;
     int2 *ent = in_smem ? s_ent : g_ent;
     const int32_t ecap = in_smem ? C::ENT : ent_cap;
-    if (!in_smem && k1 - k0 + C::EXTRA > ent_cap) {  // sized by the planning: cannot happen
+    if (!in_smem && k1 - k0 > ent_cap) {  // sized by the planning: cannot happen
       if (tid == 0) raise_error(meta, SLG_ERR_INVALID, kWhereGiant);
       break;
     }
     const int32_t work = a.row_work[e - a.row_begin];
-    const int32_t seg = max(kDnSeg * min(nwin, 1 << 20), work / (C::EXTRA - 1) + 1);
+    const int32_t split_min = max(C::SPLIT * min(nwin, 1 << 20), work / C::NSPLIT + 1);
     const int32_t long_min = SLG_DN_LONG * min(nwin, 1 << 24);
     for (int32_t k = k0 + tid; k < k1; k += NT) {
-      int32_t b = __ldg(w.tail_beg + k);
-      const int32_t end = __ldg(w.tail_end + k);
-      while (b < end) {
-        const int32_t n = min(seg, end - b);
-        int32_t pos;
-        if (n >= long_min) pos = atomicAdd(s_n + 0, 1);
-        else pos = ecap - 1 - atomicAdd(s_n + 1, 1);
-        ent[pos] = make_int2(b, b + n);
-        b += n;
+      const int32_t b = __ldg(w.tail_beg + k), end = __ldg(w.tail_end + k), n = end - b;
+      if (n <= 0) continue;
+      const int32_t h = n >= split_min ? atomicAdd(s_n + 3, 1) : C::NSPLIT;
+      if (h < C::NSPLIT) {
+        for (int32_t q = 0; q < NW; ++q)
+          split[h * NW + q] = make_int2((int32_t)((uint32_t)b + 32u * q), end);
+      } else {
+        const int32_t pos =
+            n >= long_min ? atomicAdd(s_n + 0, 1) : ecap - 1 - atomicAdd(s_n + 1, 1);
+        ent[pos] = make_int2(b, end);
       }
     }
     __syncthreads();
-    const int32_t nl = s_n[0], ns = s_n[1];
+    const int32_t nl = s_n[0], ns = s_n[1], nh = min(s_n[3], C::NSPLIT);
     int2 *ent_s = ent + (ecap - ns);
-    int32_t out = 0;  // pairs of the row so far
-    int32_t mine = 0;  // count mode: the thread's survivors
     int par = 0;
-    bool fail = false;
     for (int32_t F0 = f_lo; F0 < f_hi; F0 += win) {
       const int32_t F1 = f_hi - F0 > win ? F0 + win : f_hi;
       bool any = false;
       // 2. sweep
-      if (lb == 2) mine += dn_sweep<2, NW>(w.c_idx_s, ent, nl, ent_s, ns, F0, F1, cnt, map, smin, emit, &any);
-      else if (lb == 3) mine += dn_sweep<3, NW>(w.c_idx_s, ent, nl, ent_s, ns, F0, F1, cnt, map, smin, emit, &any);
-      else if (lb == 4) mine += dn_sweep<4, NW>(w.c_idx_s, ent, nl, ent_s, ns, F0, F1, cnt, map, smin, emit, &any);
-      else mine += dn_sweep<5, NW>(w.c_idx_s, ent, nl, ent_s, ns, F0, F1, cnt, map, smin, emit, &any);
+      if (lb == 2) mine += dn_sweep<2, C>(w.c_idx_s, ent, nl, ent_s, ns, split, nh, F0, F1, cnt, map, smin, emit, &any);
+      else if (lb == 3) mine += dn_sweep<3, C>(w.c_idx_s, ent, nl, ent_s, ns, split, nh, F0, F1, cnt, map, smin, emit, &any);
+      else if (lb == 4) mine += dn_sweep<4, C>(w.c_idx_s, ent, nl, ent_s, ns, split, nh, F0, F1, cnt, map, smin, emit, &any);
+      else mine += dn_sweep<5, C>(w.c_idx_s, ent, nl, ent_s, ns, split, nh, F0, F1, cnt, map, smin, emit, &any);
       if (core_row) {
         // tile counts of the core rows in the window, after row e itself
         const int32_t p0 = max(core_lower(ci.core_list, ci.n_core, F0), ri + 1);
@@ -421,7 +462,7 @@ template <class C>
 long long dense_stride(long long max_pairs, int32_t max_size, long long *pair_cap,
                        int32_t *ent_cap) {
   *pair_cap = (max_pairs + 31) & ~31ll;
-  *ent_cap = max_size > C::ENT - C::EXTRA ? (max_size + C::EXTRA + 15) & ~15 : 0;
+  *ent_cap = max_size > C::ENT ? (max_size + 15) & ~15 : 0;
   return 2 * *pair_cap + 2ll * *ent_cap;
 }
 

@@ -77,3 +77,28 @@ def test_long_tails_are_cut():
             i, j, w = slg.build_rows(slg.to_device(h), s, int(e), int(e) + 1,
                                      capacity=max(n_e, 1))
             assert np.array_equal(as_np((i, j, w)), want[want[:, 0] == e]), (s, e)
+
+
+# the longest tails are split over the warps in blocks of 32 entries: one block
+# less, exactly and more than a round of all warps, alone, with others beside
+# them and with the whole length in one window or spread over all
+@pytest.mark.parametrize("tails", [(2_049,), (4_000, 4_000), (1_023, 1_025, 2_080, 40),
+                                   (1_500,) * 15, (1_500,) * 17, (3_000, 255, 256, 257, 31, 33)])
+@pytest.mark.parametrize("spread", [True, False])
+def test_split_tails(tails, spread):
+    m, n = 100_000, 50_000
+    rng = np.random.default_rng(len(tails))
+    r, c = [np.zeros(len(tails), np.int64)], [np.arange(len(tails))]
+    for v, deg in enumerate(tails):
+        far = rng.choice(np.arange(1, m) if spread else np.arange(90_000, 95_000), deg, False)
+        r.append(far)
+        c.append(np.full(deg, v))
+    size = rng.integers(1, 4, m - 1)
+    r.append(np.repeat(np.arange(1, m), size))
+    c.append(rng.integers(100, n, int(size.sum())))
+    h = hg.from_pairs(np.concatenate(r), np.concatenate(c), m, n)
+    dh = slg.to_device(h)
+    for s in (1, 2, 3):
+        want = oracle.canonical(*oracle.line_graph_of(h, s, threads=8))
+        assert np.array_equal(as_np(slg.build(dh, s)), want), s
+        assert slg.count(dh, s) == want.shape[0]
