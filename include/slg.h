@@ -499,14 +499,17 @@ typedef struct slg_stats {
   int64_t wedges;          /* W_s visited */
   int64_t pairs;           /* |L_s| */
   int64_t rows_active;     /* rows with size >= s */
-  int64_t rows_bin[5];     /* rows per bin */
+  int64_t rows_bin[5];     /* rows per bin: warp, CTA-S (and rows bin),
+                              CTA-L, giant (and dense bin), sparse */
   int64_t wedges_bin[5];   /* wedges per bin */
   int64_t incid_bin[5];    /* CSR incidences of the rows of each bin */
   int64_t pairs_bin[5];    /* pairs emitted by each bin */
-  int32_t kernel_launches; /* kernels launched by the call */
+  int32_t kernel_launches; /* kernels launched by the call (those that
+                              had work: empty bins are not launched) */
   int32_t profiled;        /* 1 if the ms_* fields below were measured */
   float ms_plan;           /* validation, maps, filtered CSC, bins */
-  float ms_walk[5];        /* the walk kernel of each bin */
+  float ms_walk[5];        /* the walk kernels of each bin, run one after
+                              the other while profiling (else they overlap) */
   float ms_scan;           /* row offsets */
   float ms_gather;         /* output assembly */
   int64_t core_rows;       /* dense core used by SLG_TENSOR_CORE: rows, */
@@ -514,16 +517,13 @@ typedef struct slg_stats {
   int64_t core_nnz;        /* found or the flag was not given) */
   int64_t giant_cycles[4]; /* giant bin, SM clock cycles summed over CTAs:
                               walk, partition into buckets, bucket counting
-                              (of partitioned rows), and the whole of its
-                              dense rows */
+                              (of partitioned rows); [3]: the dense bin */
   int64_t max_row_work;    /* largest wedge count of one row */
   float ms_relabel;        /* SLG_RELABEL_*: building the renumbered side */
   float ms_order;          /* SLG_RELABEL_*: caller ids and (i, j) order */
   int64_t sparse_cycles[5]; /* sparse bin, SM clock cycles summed over CTAs:
-                               row set-up, first walk, second pass (over the
-                               copy of the far ends the first walk made),
-                               collect and order the survivors, emit and
-                               clear */
+                               row set-up, first pass, second pass, collect
+                               and order the survivors, emit and clear */
   float ms_tile;           /* the tensor-core tile kernel of the dense core
                               (SLG_TENSOR_CORE builds, slg_tile_overlap) */
 } slg_stats;
