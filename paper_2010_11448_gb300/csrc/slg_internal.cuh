@@ -364,11 +364,9 @@ __device__ __forceinline__ int32_t s_of(const int32_t *row_s, int32_t smin, int3
 
 // Wedge-work thresholds of the bins (runtime; each at most the capacity the
 // bin's kernel is compiled for: kWarpMaxWork, kCtaSMaxWork, kCtaLMaxWork).
-// `sparse`: sparse rows above the CTA bins up to this work take the sparse
-// bin (larger ones hold more repeated far ends per window than its table,
-// and the giant bin's partition serves them better); 0 turns the bin off.
-// `bloom`: rows with s >= 2 above this work (and at most `sparse`) take the
-// sparse bin also when they are dense or fit a CTA bin.
+// `sparse`: rows with s >= 2 that are not dense take the sparse bin up to this
+// work (larger ones the giant bin); 0 turns the bin off.  `bloom`: the least
+// work of its rows (those of at most `ctas` wedges take the rows bin).
 #ifndef SLG_BLOOM_MIN_WORK
 #define SLG_BLOOM_MIN_WORK 1024
 #endif

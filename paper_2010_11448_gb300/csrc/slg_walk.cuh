@@ -1,4 +1,5 @@
-// Device helpers shared by the walk kernels (slg_walk.cu, slg_dense.cu).
+// Device helpers shared by the walk kernels (slg_walk.cu, slg_dense.cu,
+// slg_sparse.cu, slg_small.cu).
 #pragma once
 
 #include "slg_internal.cuh"
