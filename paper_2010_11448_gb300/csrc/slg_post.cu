@@ -543,7 +543,8 @@ cudaError_t launch_squeeze(const int32_t *a, const int32_t *b, int64_t n, int32_
       k_mark<false><<<sms * 2, kMarkNT, 0, st>>>(a, b, n, R, bits, err);
     }
   }
-  k_word_counts<<<grid_for((int64_t)words + 1), kNT, 0, st>>>(bits, words, cnt);
+  // (a word per thread: up to 2^26 + 1 of them, above grid_for's default cap)
+  k_word_counts<<<grid_for((int64_t)words + 1, (int64_t)1 << 30), kNT, 0, st>>>(bits, words, cnt);
   cudaError_t e = launch_xscan(cnt, rank, (int64_t)words + 1, tile, st);
   if (e != cudaSuccess) return e;
   int2 *w2 = static_cast<int2 *>(word);

@@ -126,3 +126,20 @@ def test_sizes_against_oracle(V, n):
     lab, k = slg.components(t[0], t[1], V)
     wlab, wk = oracle.components(i, j, V)
     assert np.array_equal(np_(lab), wlab) and k == wk
+
+
+# id maps of more words than 65,536 blocks of 256 threads take (16,777,216: ids
+# from 536,870,912 on), up to the largest id space
+@pytest.mark.parametrize("R", [536_870_881, 536_870_913, 600_000_000, 2**31 - 1])
+def test_squeeze_of_large_id_spaces(R):
+    rng = np.random.default_rng(R)
+    ids = np.unique(np.concatenate([rng.integers(0, R, 300), [0, 31, 32, R - 1, R - 2, R - 33],
+                                    np.arange(536_870_850, 536_870_881)]))
+    a, b = rng.integers(0, ids.size, (2, 5_000))
+    a, b = ids[np.minimum(a, b)[a != b]], ids[np.maximum(a, b)[a != b]]
+    order = np.lexsort((b, a))
+    i, j = a[order].astype(np.int32), b[order].astype(np.int32)
+    si, sj, old = slg.squeeze(torch.from_numpy(i).cuda(), torch.from_numpy(j).cuda(), R)
+    wi, wj, wold = oracle.squeeze(i, j, R)
+    assert np.array_equal(np_(si), wi) and np.array_equal(np_(sj), wj)
+    assert np.array_equal(np_(old), wold)
