@@ -498,7 +498,8 @@ cudaError_t launch_filter(const Side &s, int32_t smin, const Work &w, cudaStream
   if (ntiles > 0) {
     k_filter_scatter<<<ntiles, kScanNT, 0, st>>>(s, smin, w.tile, w.qs, w.c_idx_s, w.meta);
   }
-  k_filter_offsets<<<grid_for((int64_t)s.C + 1, 256), 256, 0, st>>>(s, w.qs, w.tile, ntiles,
+  // (a column per thread: sides of up to 2^31 - 1 columns)
+  k_filter_offsets<<<grid_for((int64_t)s.C + 1, 256, 1 << 30), 256, 0, st>>>(s, w.qs, w.tile, ntiles,
                                                                     w.c_off_s, w.meta);
   return cudaGetLastError();
 }
