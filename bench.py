@@ -207,7 +207,7 @@ def walk_bytes(st, b):
 GRAPH_CREATE_LAUNCHES = 5
 
 WALK_KERNELS = ["k_walk_warp", "k_walk_rows + k_walk_cta<256,2048>", "k_walk_cta<256,8192>",
-                "k_walk_dense + k_walk_giant", "k_walk_sparse"]
+                "k_walk_dense + k_walk_giant", "k_walk_sparse + k_walk_flat"]
 NBINS = len(WALK_KERNELS)
 
 

@@ -541,11 +541,12 @@ int run_binned(Call &c, int64_t *result) {
   }
   // (core rows may have no wedges but still need a giant CTA; their pairs,
   // staged in the same scratch, also come from up to n_core tile items)
-  // (a row of the sparse or rows bin that overflows its table is handed to
+  // (a row of the sparse, flat or rows bin that overflows its table is handed to
   // the giant bin, so the giant scratch also covers these rows)
   const Meta &mp = *c.meta_host;
   const int32_t max_giant =
-      (mp.rows_bin[kBinGiant] || mp.rows_bin[kBinSparse] || mp.rows_bin[kBinRows])
+      (mp.rows_bin[kBinGiant] || mp.rows_bin[kBinSparse] || mp.rows_bin[kBinRows] ||
+       mp.rows_bin[kBinFlat])
           ? std::max(std::max(mp.max_giant_work, mp.max_sparse_work), kCtaSMaxWork) +
                 (core.T ? core.n_core : 0)
           : 0;
@@ -571,9 +572,18 @@ int run_binned(Call &c, int64_t *result) {
   L.w.tail_end = w.tail_end;
   for (int b : {kBinWarp, kBinCtaS, kBinCtaL, kBinRows})
     if (!mp.rows_bin[b]) L.skip |= 1u << b;
-  if (!mp.sparse_huge) L.skip |= kSkipSparseBig;
-  if (!mp.sparse_rest) L.skip |= kSkipSparseSmall;
-  if (!mp.rows_bin[kBinGiant] && !mp.rows_bin[kBinSparse] && !mp.rows_bin[kBinRows])
+  const bool flat = flat_kernels((long long)mp.wedges_bin[kBinFlat],
+                                 (long long)mp.wedges_bin[kBinSparse]);
+  if (!flat && mp.flat_huge + mp.flat_rest > 0) {
+    SLG_TRY(launch_join_flat(w.bin_rows, c.rows, mp, w.meta, c.st));
+    c.launches += 1;
+  }
+  if (!mp.sparse_huge && (flat || !mp.flat_huge)) L.skip |= kSkipSparseBig;
+  if (!mp.sparse_rest && (flat || !mp.flat_rest)) L.skip |= kSkipSparseSmall;
+  if (!flat || !mp.flat_huge) L.skip |= kSkipFlatBig;
+  if (!flat || !mp.flat_rest) L.skip |= kSkipFlatSmall;
+  if (!mp.rows_bin[kBinGiant] && !mp.rows_bin[kBinSparse] && !mp.rows_bin[kBinRows] &&
+      !mp.rows_bin[kBinFlat])
     L.skip |= 1u << kBinGiant;
   cudaEvent_t *ev = c.evs->on ? c.evs->ev + kEvWalk : nullptr;
   if (c.rows > 0) {
@@ -624,6 +634,10 @@ int run_binned(Call &c, int64_t *result) {
                     offsetof(Meta, sparse_ticket) + sizeof(unsigned int),
                 "the two sparse ticket counters are cleared together");
   SLG_TRY(cudaMemsetAsync(&w.meta->sparse_ticket, 0, 2 * sizeof(unsigned int), c.st));
+  static_assert(offsetof(Meta, flat_ticket_rest) ==
+                    offsetof(Meta, flat_ticket) + sizeof(unsigned int),
+                "the two flat ticket counters are cleared together");
+  SLG_TRY(cudaMemsetAsync(&w.meta->flat_ticket, 0, 2 * sizeof(unsigned int), c.st));
   // back to the planned giant list: the sparse bin hands the same rows
   // over again
   SLG_TRY(cudaMemcpyAsync(&w.meta->rows_bin[kBinGiant], &giant_rows0, sizeof(giant_rows0),
@@ -875,7 +889,7 @@ int run(const slg_hypergraph *h, int32_t smin, uint32_t flags, int32_t row_begin
         int32_t *max_row_work = nullptr, long long *row_ptr_out = nullptr,
         int32_t *row_work_out = nullptr, const int32_t *row_fhi = nullptr,
         int32_t *max_row_size = nullptr, slg_alloc_fn alloc = nullptr,
-        void *alloc_ctx = nullptr) {
+        void *alloc_ctx = nullptr, bool *flat = nullptr) {
   int rc = check_args(h, smin, flags);
   if (rc != SLG_OK) return rc;
   if (!result) return SLG_ERR_INVALID;
@@ -1030,8 +1044,12 @@ int run(const slg_hypergraph *h, int32_t smin, uint32_t flags, int32_t row_begin
     stats.incid_bin[b] = (int64_t)m.incid_bin[b];
     stats.pairs_bin[b] = (int64_t)m.pairs_bin[b];
   }
-  // the rows bin's rows are reported as the small CTA bin's, the dense
-  // bin's as giant ones
+  // the rows bin's rows are reported as the small CTA bin's, the flat bin's
+  // as sparse ones, the dense bin's as giant ones
+  stats.rows_bin[kBinSparse] += (int64_t)m.rows_bin[kBinFlat];
+  stats.wedges_bin[kBinSparse] += (int64_t)m.wedges_bin[kBinFlat];
+  stats.incid_bin[kBinSparse] += (int64_t)m.incid_bin[kBinFlat];
+  stats.pairs_bin[kBinSparse] += (int64_t)m.pairs_bin[kBinFlat];
   stats.rows_bin[kBinCtaS] += (int64_t)m.rows_bin[kBinRows];
   stats.wedges_bin[kBinCtaS] += (int64_t)m.wedges_bin[kBinRows];
   stats.incid_bin[kBinCtaS] += (int64_t)m.incid_bin[kBinRows];
@@ -1042,6 +1060,7 @@ int run(const slg_hypergraph *h, int32_t smin, uint32_t flags, int32_t row_begin
   stats.pairs_bin[kBinGiant] += (int64_t)m.pairs_bin[kBinDense];
   if (max_row_work) *max_row_work = m.max_row_work;
   if (max_row_size) *max_row_size = m.max_row_size;
+  if (flat) *flat = flat_kernels(m.wedges_bin[kBinFlat], m.wedges_bin[kBinSparse]);
   stats.kernel_launches = c.launches;
   stats.core_rows = c.core_rows;
   stats.core_cols = c.core_cols;
@@ -1112,6 +1131,7 @@ struct slg_plan {
   slg::Work w = {};
   int32_t *giant = nullptr;
   slg::WalkLaunch scratch = {};    // giant_stride, dense_pairs, dense_size, sparse_ints
+  bool flat = false;               // Bins::flat
   int32_t *out_i = nullptr, *out_j = nullptr, *out_w = nullptr;
   long long *offsets = nullptr;    // [count + 1]
   int64_t pairs = 0;
@@ -1140,7 +1160,9 @@ cudaError_t enqueue_plan(slg_plan *p, const Bins &bins, cudaStream_t st, int32_t
   PLAN_TRY(launch_validate(sd, w.meta, st));
   PLAN_TRY(launch_csr2csc(sd, w.csr2csc, w.meta, st));
   PLAN_TRY(launch_filter(sd, 1, w, st));
-  PLAN_TRY(launch_rows_work(sd, 1, 0, sd.R, w, CoreInfo{}, bins, st));
+  Bins b = bins;
+  b.flat = p->flat;
+  PLAN_TRY(launch_rows_work(sd, 1, 0, sd.R, w, CoreInfo{}, b, st));
   WalkLaunch L = {};
   L.w.r_off = sd.r_off;
   L.w.r_idx = sd.r_idx;
@@ -1169,6 +1191,7 @@ cudaError_t enqueue_plan(slg_plan *p, const Bins &bins, cudaStream_t st, int32_t
   L.dense_pairs[1] = p->scratch.dense_pairs[1];
   L.dense_size = p->scratch.dense_size;
   L.sparse_ints = p->scratch.sparse_ints;
+  if (!p->flat) L.skip |= kSkipFlatBig | kSkipFlatSmall;
   if (p->giant) place_scratch(&L, p->giant);
   int32_t n = 0;
   if (sd.R > 0) PLAN_TRY(launch_walk(L, st, &n));
@@ -1893,8 +1916,10 @@ extern "C" int slg_plan_create(const slg_hypergraph *hs, const int32_t *s, int32
   // 2. sizes: one counting pass over the union (per-row thresholds)
   int64_t pairs = 0;
   int32_t max_work = 0, max_size = 0;
+  bool flat = false;  // the flat bin has kernels of its own
   int rc = run(&p->u, 1, flags, 0, p->sd.R, kOpCount, nullptr, nullptr, nullptr, 0, &pairs, st,
-               p->sd.row_s, &max_work, nullptr, nullptr, p->sd.row_fhi, &max_size);
+               p->sd.row_s, &max_work, nullptr, nullptr, p->sd.row_fhi, &max_size, nullptr, nullptr,
+               &flat);
   if (rc != SLG_OK) return rc;
   p->pairs = pairs;
   // 3. persistent buffers
@@ -1924,6 +1949,7 @@ extern "C" int slg_plan_create(const slg_hypergraph *hs, const int32_t *s, int32
   if (max_work > 0) {
     const size_t n = scratch_ints(&p->scratch, max_work, max_work, std::min<long long>(max_work, R),
                                   std::min<long long>(max_work, R), max_size);
+    p->flat = flat;
     SLG_TRY(p->mem.get(&p->giant, n));
   }
   // 4. autotuner: bin thresholds, timed on this batch

@@ -22,14 +22,16 @@ constexpr int32_t kEmpty = -1;
 // Row bins by wedge work (the degree-binned scheduler).  Rows above
 // kDenseMinWork wedges whose far ends are dense in their id span (is_dense)
 // go to the dense bin; of the others, rows with s >= 2 from Bins::bloom up to
-// Bins::sparse wedges go to the sparse bin and the rest above the CTA bins to
+// Bins::sparse wedges go to the sparse bin (the flat bin, if their tails are
+// short: short_tails) and the rest above the CTA bins to
 // the giant bin.  Rows with s >= 2 of at most Bins::ctas
 // wedges take the rows bin (a warp each), s = 1 ones the warp and CTA bins.
-// The statistics count the dense bin's rows as giant ones and the rows bin's
-// as the small CTA bin's (kNumBins bins are reported, kNumLists lists kept).
+// The statistics count the dense bin's rows as giant ones, the rows bin's as
+// the small CTA bin's and the flat bin's as sparse ones (kNumBins bins are
+// reported, kNumLists lists kept).
 enum Bin : int {
   kBinWarp = 0, kBinCtaS = 1, kBinCtaL = 2, kBinGiant = 3, kBinSparse = 4, kNumBins = 5,
-  kBinDense = 5, kBinRows = 6, kNumLists = 7
+  kBinDense = 5, kBinFlat = 6, kBinRows = 7, kNumLists = 8
 };
 
 // Upper bounds on a row's wedge count for each non-giant bin.  The hash tables
@@ -47,7 +49,7 @@ constexpr int32_t kCtaLMaxWork = 4096;
 #define SLG_GIANT_HUGE_WORK 32768
 #endif
 constexpr int32_t kGiantHugeWork = SLG_GIANT_HUGE_WORK;
-// Sparse rows above this work take the instance of the sparse kernel with
+// Sparse and flat rows above this work take the instance of their kernel with
 // the larger table.
 #ifndef SLG_SP_BIG_WORK
 #define SLG_SP_BIG_WORK 8192
@@ -58,6 +60,20 @@ constexpr int32_t kSparseBigWork = SLG_SP_BIG_WORK;
 #define SLG_SPARSE_MAX_WORK 65536
 #endif
 constexpr int32_t kSparseMaxWork = SLG_SPARSE_MAX_WORK;
+// Rows of many vertices whose tails are mostly short: of these, the flat bin
+// takes rows of up to kFlatMaxWork wedges.
+constexpr int32_t kFlatMaxWork = 16384;
+__host__ __device__ __forceinline__ bool short_tails(int32_t work, int32_t size) {
+  return size > 48 && work < 32ll * size;
+}
+// Whether the flat bin's kernels run, by its wedges and the sparse bin's; else
+// its rows are given to the sparse bin (launch_join_flat).  A kernel lasts as long
+// as its longest row, so a few such rows are better taken along with the others
+// (counting pass of 120K x 240K, host builds of 200K x 400K: 800 and 3,470 us so,
+// 870 and 3,570 with kernels of their own; chung_lu_1m the same both ways).
+__host__ __device__ __forceinline__ bool flat_kernels(long long flat, long long sparse) {
+  return flat > 0 && (2 * flat >= sparse || flat >= 1ll << 26);
+}
 #ifndef SLG_DENSE_MIN_WORK
 #define SLG_DENSE_MIN_WORK 256
 #endif
@@ -133,8 +149,6 @@ struct Meta {
   unsigned long long wedges;           // W_s
   unsigned long long active;           // rows with size >= s in range
   unsigned long long pairs;            // |L_s| over the row range
-  unsigned long long stage_cursor;     // staging allocator
-  unsigned long long stage_overflow;   // rows that did not fit the staging
   unsigned int giant_ticket;           // dynamic giant-row scheduling
   unsigned int giant_huge;             // giant rows above kGiantHugeWork (front of the list)
   unsigned int giant_rest;             // the other giant rows (back of the list)
@@ -142,6 +156,10 @@ struct Meta {
   unsigned int sparse_ticket_rest;
   unsigned int sparse_huge;
   unsigned int sparse_rest;
+  unsigned int flat_ticket;            // the same four for the flat bin
+  unsigned int flat_ticket_rest;
+  unsigned int flat_huge;
+  unsigned int flat_rest;
   unsigned int dense_ticket;           // the same four for the dense bin (huge: kDenseBigSize)
   unsigned int dense_ticket_rest;
   unsigned int dense_huge;
@@ -149,13 +167,18 @@ struct Meta {
   int32_t max_dense_work[2];           // largest work of a dense-bin row: big instance, other
   int32_t max_dense_size;              // most vertices of a dense-bin row
   int32_t max_row_size;                // most vertices of a row with work
-  int32_t max_sparse_work;             // largest work of a sparse-bin row
+  int32_t max_sparse_work;             // largest work of a sparse- or flat-bin row
   int32_t kept;                        // entries of the filtered CSC
   int32_t max_giant_work;              // largest work of a giant-bin row
   unsigned long long nnz_core;         // incidences of the dense core
   int32_t max_row_work;                // largest work of any row
   unsigned long long giant_cycles[4];  // giant bin: SM cycles in walk, partition, buckets; dense bin
   unsigned long long sparse_cycles[5]; // sparse bin: row set-up, walk, collect, emit, staging
+  // Every row that emits adds to pairs_bin and to stage_cursor, so they lie more
+  // than an L2 line apart (in one line, k_walk_rows of an L_2 of 200K x 400K took
+  // 0.41 instead of 0.32 ms).
+  unsigned long long stage_cursor;     // staging allocator
+  unsigned long long stage_overflow;   // rows that did not fit the staging
 };
 
 // Where a device-side check fired (for error reports).
@@ -377,6 +400,7 @@ struct Bins {
   int32_t sparse = kSparseMaxWork;
   int32_t bloom = SLG_BLOOM_MIN_WORK;
   int32_t dense = kDenseRatio;
+  bool flat = true;  // the flat bin is on
 };
 
 // Dense core for the tensor-core tile path (all null / 0 when unused).
@@ -482,13 +506,14 @@ struct WalkLaunch {
   long long giant_stride;   // ints per giant CTA
   int32_t R;                // rows of the side (far ends lie in [0, R))
   int32_t *dense_scratch[2], *sparse_scratch;  // in giant_scratch
-  long long sparse_ints;    // of sparse_scratch
+  long long sparse_ints;    // of sparse_scratch (the flat kernels' as well: they follow)
   long long dense_pairs[2]; // most pairs a dense-bin row can have: big instance, other (0: no row)
   int32_t dense_size;       // most vertices of a dense-bin row
   unsigned skip;            // bit b: bin b is known to be empty (kSkipSparseBig, ...)
 };
-// Further bits of WalkLaunch::skip: the sparse bin's two instances.
+// Further bits of WalkLaunch::skip: the two instances of the sparse and flat bins.
 constexpr unsigned kSkipSparseBig = 1u << 8, kSkipSparseSmall = 1u << 9;
+constexpr unsigned kSkipFlatBig = 1u << 10, kSkipFlatSmall = 1u << 11;
 
 // Sides of at most this many rows take the short path (slg_small.cu).
 #ifndef SLG_SMALL_ROWS
@@ -512,8 +537,8 @@ cudaError_t launch_small_emit(const SmallCall &c, cudaStream_t st, int32_t *laun
 cudaError_t launch_small(const SmallCall &c, cudaStream_t st, int32_t *launches, cudaEvent_t walk0,
                          cudaEvent_t walk1);
 
-// CTAs of the giant kernel (two per SM); scratch ints of the sparse and dense
-// kernels.
+// CTAs of the giant kernel (two per SM); scratch ints of the sparse (and flat) and
+// dense kernels.
 int giant_ctas();
 long long sparse_ints(int32_t max_work);
 long long dense_ints(int small, long long pairs, int32_t size_big);
@@ -531,6 +556,8 @@ cudaError_t launch_walk(const WalkLaunch &L, cudaStream_t st, int32_t *launches,
                         cudaEvent_t *ev = nullptr);
 cudaError_t launch_walk_rows(const WalkLaunch &L, cudaStream_t st);
 cudaError_t launch_walk_sparse(const WalkLaunch &L, cudaStream_t st, int32_t *launches);
+cudaError_t launch_join_flat(int32_t *bin_rows, int32_t rows, const Meta &m, Meta *meta,
+                             cudaStream_t st);
 cudaError_t launch_walk_dense(const WalkLaunch &L, int small, cudaStream_t st);
 cudaError_t launch_row_scan(int32_t rows, const Work &w, cudaStream_t st);
 // The device Meta into host memory the device can address (mapped pinned

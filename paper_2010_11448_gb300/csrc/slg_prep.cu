@@ -269,13 +269,13 @@ __global__ __launch_bounds__(kRowsNT) void k_rows_work(Side s, int32_t smin, int
                                                        Meta *meta) {
   if (meta->err) return;
   __shared__ int32_t s_work[kRowsPerBlock];
-  // block maxima of the row work (all rows, giant-bin, sparse-bin, the dense
+  // block maxima of the row work (all rows, giant-bin, sparse- or flat-bin, the dense
   // bin's two instances' rows) and size (dense-bin rows, all rows): one global atomicMax each per
   // block instead of one per row
   __shared__ int32_t s_max[7];
   __shared__ int32_t s_act;  // active rows (size >= s) of the block
   __shared__ int32_t s_cnt[kNumLists], s_base[kNumLists];
-  __shared__ int32_t s_hcnt[3], s_hbase[3];  // giant / sparse / dense rows handed out first
+  __shared__ int32_t s_hcnt[4], s_hbase[4];  // giant / sparse / dense / flat rows handed out first
   __shared__ unsigned long long s_w[kNumLists], s_k[kNumLists];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int32_t r0 = row_begin + blockIdx.x * kRowsPerBlock;
@@ -284,7 +284,7 @@ __global__ __launch_bounds__(kRowsNT) void k_rows_work(Side s, int32_t smin, int
     s_w[threadIdx.x] = 0;
     s_k[threadIdx.x] = 0;
   }
-  if (threadIdx.x < 3) s_hcnt[threadIdx.x] = 0;
+  if (threadIdx.x < 4) s_hcnt[threadIdx.x] = 0;
   if (threadIdx.x < 7) s_max[threadIdx.x] = 0;
   if (threadIdx.x == 0) s_act = 0;
   __syncthreads();
@@ -382,22 +382,25 @@ __global__ __launch_bounds__(kRowsNT) void k_rows_work(Side s, int32_t smin, int
       const int32_t se = s_of(s.row_s, smin, e);
       const int32_t span = (s.row_fhi ? s.row_fhi[e] : s.R) - 1 - e;  // far ends: (e, e + span]
       // a row whose far ends are dense in its span takes the dense bin; else
-      // one with s >= 2 from bins.bloom up to bins.sparse wedges the sparse bin
+      // one with s >= 2 from bins.bloom up to bins.sparse wedges the sparse or
+      // the flat bin
       if ((forced || my_work > kDenseMinWork) && is_dense(my_work, size, se, span, bins.dense))
         my_bin = kBinDense;
-      else if (!forced && my_work > bins.bloom && my_work <= bins.sparse && se >= 2)
-        my_bin = kBinSparse;
+      else if (!forced && my_work > bins.bloom && my_work <= bins.sparse && se >= 2) {
+        if (!bins.flat || !short_tails(my_work, size)) my_bin = kBinSparse;
+        else if (my_work <= kFlatMaxWork) my_bin = kBinFlat;
+      }
       else if (!forced && my_work <= bins.ctas && se >= 2)
         my_bin = kBinRows;
       if (my_bin == kBinGiant) atomicMax(&s_max[1], my_work);
-      if (my_bin == kBinSparse) atomicMax(&s_max[2], my_work);
+      if (my_bin == kBinSparse || my_bin == kBinFlat) atomicMax(&s_max[2], my_work);
       if (my_bin == kBinDense) {
         atomicMax(&s_max[size > kDenseBigSize ? 3 : 6], my_work);
         atomicMax(&s_max[4], size);
       }
       huge = (my_bin == kBinDense && size > kDenseBigSize) ||
              (my_bin == kBinGiant && my_work > kGiantHugeWork) ||
-             (my_bin == kBinSparse && my_work > kSparseBigWork);
+             ((my_bin == kBinSparse || my_bin == kBinFlat) && my_work > kSparseBigWork);
       my_slot = huge ? atomicAdd(&s_hcnt[my_bin - kBinGiant], 1) : atomicAdd(&s_cnt[my_bin], 1);
       atomicAdd(&s_w[my_bin], (unsigned long long)my_work);
       atomicAdd(&s_k[my_bin], (unsigned long long)size);
@@ -409,16 +412,18 @@ __global__ __launch_bounds__(kRowsNT) void k_rows_work(Side s, int32_t smin, int
     if (b < kBinGiant || b == kBinRows) {
       s_base[b] = s_cnt[b] ? (int32_t)atomicAdd(&meta->rows_bin[b], (unsigned long long)s_cnt[b]) : 0;
     } else {
-      // the huge rows of the giant, sparse and dense bins fill their list from
+      // the huge rows of the giant, sparse, dense and flat bins fill their list from
       // the front, the others from the back (the kernels hand out the huge
       // ones first); rows_bin counts both
       const int q = b - kBinGiant;
       unsigned *rest = q == 0   ? &meta->giant_rest
                        : q == 1 ? &meta->sparse_rest
-                                : &meta->dense_rest;
+                       : q == 2 ? &meta->dense_rest
+                                : &meta->flat_rest;
       unsigned *hge = q == 0   ? &meta->giant_huge
                       : q == 1 ? &meta->sparse_huge
-                               : &meta->dense_huge;
+                      : q == 2 ? &meta->dense_huge
+                               : &meta->flat_huge;
       if (s_cnt[b] + s_hcnt[q])
         atomicAdd(&meta->rows_bin[b], (unsigned long long)(s_cnt[b] + s_hcnt[q]));
       s_base[b] = s_cnt[b] ? (int32_t)atomicAdd(rest, (unsigned)s_cnt[b]) : 0;

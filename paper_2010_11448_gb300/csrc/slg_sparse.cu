@@ -34,7 +34,8 @@
 // handed to the giant bin, which runs after this one).
 //
 // Rows of at most kCtaSMaxWork wedges are counted in the same way by one warp
-// each (k_walk_rows), with nothing but warp-wide steps.
+// each (k_walk_rows), with nothing but warp-wide steps; rows of many short tails
+// by a kernel that flattens them (k_walk_flat).
 //
 // Bound by instruction issue (70 % of issue slots) and the latency of the
 // dependent steps of a row, with five rows in flight per SM.
@@ -515,6 +516,229 @@ __global__ __launch_bounds__(C::NT, C::MINB) void k_walk_sparse(
     for (int i = 0; i < 5; ++i) atomicAdd(&meta->sparse_cycles[i], (unsigned long long)s_cyc[i]);
 }
 
+// ------------------------------------------------------------ short tails --
+//
+// The flat bin: rows with s >= 2 of 1,025 to 16,384 wedges whose tails are short
+// (more than 48 vertices, under 32 far ends per tail on average: web-shaped and
+// uniform inputs with a mean of 5 to 25 hyperedges per vertex).  A warp per tail,
+// as in the sparse bin, leaves most of its lanes idle there (58 to 190 instead of
+// 10 to 15 CTA cycles per wedge), and no tail is long enough to be worth setting
+// aside.  The row's wedges are flattened: wedge i's tail is found by a search over
+// the tails' prefix sums, each warp loads kSpSeg consecutive wedges per step and
+// copies their far ends to the CTA's scratch, so that the second pass reads them
+// in order.  Filters, table and survivors are the sparse bin's; a row that
+// overflows the table or has more survivors than are ordered here goes to the
+// giant bin.  (Its own kernel: with this path beside the other in k_walk_sparse the
+// step of chung_lu_1m, which has few such rows, took 107.4 instead of 105.4 ms.)
+//
+// 100K rows of 250 of 1.9M vertices, L_2, whole counting pass: 6.8 -> 2.6 ms; 200K
+// rows of 400 of 9M 19.7 -> 9.3; 4M x 10M lognormal hyperedges with the tile path,
+// L_2, L_8, L_32, per build 23.3, 23.9, 22.5 -> 19.1, 18.0, 16.7.  Mean tails of
+// up to 8, 16, 32: 5.0, 2.7, 2.7 ms and (100K rows of 100 of 300K) 2.9, 2.6, 1.7.
+
+// The two instances of the kernel, for rows of up to kSparseBigWork wedges and more.
+// (The smaller table alone: 92K rows of the 400K x 1,500 handed over, 87.7 -> 102.7
+// ms a pass; the larger alone 9.5 instead of 9.1 on 200K x 400.)
+struct FlSmall {
+  static constexpr int NT = 256, LGT = 11, MINB = 5;
+};
+struct FlBig {  // (256 threads, four CTAs: 26.2 instead of 22.3 ms on 400K rows of 1,500)
+  static constexpr int NT = 512, LGT = 12, MINB = 3;
+};
+
+// [s_base 8][s_ovf 4][s_row 4][s_any 4][s_nsurv 4][pad 8][s_cyc 6 x 8][once][twice][table x 8]
+// [tail places NT][prefix sums NT][ws NT/32+1][queues]
+template <class C>
+constexpr size_t flat_smem() {
+  return 80 + (size_t)kSpWords * 8 + (size_t)(1 << C::LGT) * 8 +
+         (size_t)(2 * C::NT + C::NT / 32 + 1 + C::NT / 32 * kSpQ) * 4;
+}
+
+// part 0: the rows above kSparseBigWork wedges (the front of the list), 1: the
+// others (its back).  buf: the CTA's share of the bin's scratch, at least the
+// largest row's work.
+template <class C>
+__global__ __launch_bounds__(C::NT, C::MINB) void k_walk_flat(
+    Walk w, const int32_t *__restrict__ rows, EmitArgs a, int32_t *__restrict__ giant_rows,
+    int32_t list_len, int32_t *__restrict__ buf, long long buf_stride, int part) {
+  constexpr int NT = C::NT, NW = NT / 32, T_MAX = 1 << C::LGT;
+  Meta *meta = a.meta;
+  if (meta->err) return;
+  extern __shared__ __align__(16) unsigned char smem[];
+  long long *s_base = reinterpret_cast<long long *>(smem);
+  int32_t *s_ovf = reinterpret_cast<int32_t *>(smem + 8);
+  int32_t *s_row = reinterpret_cast<int32_t *>(smem + 12);
+  int32_t *s_any = reinterpret_cast<int32_t *>(smem + 16);
+  int32_t *s_nsurv = reinterpret_cast<int32_t *>(smem + 20);
+  long long *s_cyc = reinterpret_cast<long long *>(smem + 32);  // as in the sparse bin
+  uint32_t *once = reinterpret_cast<uint32_t *>(smem + 80);
+  uint32_t *twice = once + kSpWords;
+  unsigned long long *tab = reinterpret_cast<unsigned long long *>(twice + kSpWords);
+  int32_t *s_beg = reinterpret_cast<int32_t *>(tab + T_MAX);
+  int32_t *s_pref = s_beg + NT;
+  int32_t *ws = s_pref + NT;
+  const int32_t tid = (int32_t)threadIdx.x, lane = tid & 31, wq = tid >> 5;
+  SpQueue q = {ws + NW + 1 + wq * kSpQ, 0};
+  int32_t *list = reinterpret_cast<int32_t *>(once);  // survivors' slots, then their keys
+  unsigned long long *keys = reinterpret_cast<unsigned long long *>(twice);
+  auto zero = [&](uint32_t *p, int n) {  // words, rounded up to four
+    uint4 *p4 = reinterpret_cast<uint4 *>(p);
+    for (int i = tid; i < (n + 3) >> 2; i += NT) p4[i] = make_uint4(0, 0, 0, 0);
+  };
+  zero(once, 2 * kSpWords);
+  clear_slots<NT>(tab, T_MAX);
+  const unsigned nrows = part ? meta->flat_rest : meta->flat_huge;
+  unsigned *ticket = part ? &meta->flat_ticket_rest : &meta->flat_ticket;
+  const bool unweighted = a.unweighted != 0;
+  const bool emit = a.mode != kCount;
+  int32_t *copy = buf + (long long)blockIdx.x * buf_stride;
+  if (tid == 0) {
+    for (int i = 0; i < 5; ++i) s_cyc[i] = 0;
+    s_cyc[5] = clock64();
+  }
+  auto lap = [&](int i) {
+    if (tid == 0) {
+      const long long t1 = clock64();
+      s_cyc[i] += t1 - s_cyc[5];
+      s_cyc[5] = t1;
+    }
+  };
+  for (;;) {
+    __syncthreads();  // the previous row is done
+    if (tid == 0) {
+      const unsigned t = atomicAdd(ticket, 1u);
+      *s_row = t >= nrows ? -1 : rows[part ? list_len - 1 - t : t];
+      *s_ovf = 0;
+      *s_any = 0;
+      *s_nsurv = 0;
+    }
+    __syncthreads();
+    const int32_t e = *s_row;
+    if (e < 0) break;
+    const int32_t smin = s_of(a.row_s, a.smin, e);
+    const int32_t work = a.row_work[e - a.row_begin];
+    const int32_t k0 = w.r_off[e], k1 = w.r_off[e + 1];
+    // (by the planning: cannot happen)
+    bool hand_over = work > kFlatMaxWork || work > buf_stride;
+    const int lgb = min(max(ceil_log2(work) + 5, 12), kSpLogB);  // as in the sparse bin
+    const int lgt = min(max(ceil_log2(work / 2 + 1), 8), C::LGT);
+    lap(0);
+    // 1. both filters, and the copy
+    bool hit = false;
+    int32_t done = 0;
+    for (int32_t base = k0; base < k1 && !hand_over; base += NT) {
+      if (base > k0) __syncthreads();  // the previous batch is read
+      const int32_t k = base + tid;
+      int32_t b = 0, len = 0, total;
+      if (k < k1) {
+        b = __ldg(w.tail_beg + k);
+        len = __ldg(w.tail_end + k) - b;
+      }
+      const int32_t inc = block_inclusive_scan<NT>(len, ws, &total);
+      s_beg[tid] = b - (inc - len);  // + i: wedge i's place
+      s_pref[tid] = inc;             // wedges up to this tail
+      __syncthreads();
+      for (int32_t c0 = wq * kSpSeg; c0 < total; c0 += NW * kSpSeg) {
+        int32_t j = 0, hi = NT - 1;  // the first tail with s_pref > c0
+        while (j < hi) {
+          const int32_t mid = (j + hi) >> 1;
+          if (s_pref[mid] > c0) hi = mid;
+          else j = mid + 1;
+        }
+        int32_t f[kSpG];
+        uint32_t old[kSpG], h[kSpG];
+#pragma unroll
+        for (int g = 0; g < kSpG; ++g) {
+          const int32_t i = c0 + 32 * g + lane;
+          f[g] = -1;
+          if (i < total) {
+            while (s_pref[j] <= i) ++j;
+            f[g] = s_beg[j] + i;
+          }
+        }
+#pragma unroll
+        for (int g = 0; g < kSpG; ++g) f[g] = f[g] >= 0 ? __ldg(w.c_idx_s + f[g]) : -1;
+#pragma unroll
+        for (int g = 0; g < kSpG; ++g) {
+          h[g] = sp_bit(f[g], lgb);
+          old[g] = 0;
+          if (f[g] >= 0) {
+            copy[done + c0 + 32 * g + lane] = f[g];
+            old[g] = atomicOr(once + (h[g] >> 5), 1u << (h[g] & 31));
+          }
+        }
+#pragma unroll
+        for (int g = 0; g < kSpG; ++g)
+          if ((old[g] >> (h[g] & 31)) & 1u) {
+            atomicOr(twice + (h[g] >> 5), 1u << (h[g] & 31));
+            hit = true;
+          }
+      }
+      done += total;
+    }
+    if (hit) *s_any = 1;
+    __syncthreads();  // filters and copy complete
+    lap(1);
+    const int32_t T = 1 << lgt;
+    int32_t dirty_once = 1 << (lgb - 5), dirty_twice = dirty_once;
+    if (*s_any) {  // uniform: else no far end has two wedges
+      // 2. counts
+      for (int32_t c0 = wq * kSpSeg; c0 < work; c0 += NW * kSpSeg) {
+        int32_t f[kSpG];
+        uint32_t word[kSpG], h[kSpG];
+#pragma unroll
+        for (int g = 0; g < kSpG; ++g)
+          f[g] = c0 + 32 * g + lane < work ? copy[c0 + 32 * g + lane] : -1;
+#pragma unroll
+        for (int g = 0; g < kSpG; ++g) {
+          h[g] = sp_bit(f[g], lgb);
+          word[g] = f[g] >= 0 ? twice[h[g] >> 5] : 0u;
+        }
+#pragma unroll
+        for (int g = 0; g < kSpG; ++g) q.push((word[g] >> (h[g] & 31)) & 1u, f[g]);
+        q.drain(c0 + NW * kSpSeg >= work, [&](int32_t x) {
+          sp_insert(tab, x, smin, unweighted, lgt, s_ovf, list, kSpList, s_nsurv);
+        });
+      }
+      __syncthreads();  // counts and survivors final
+      lap(2);
+      // 3. survivors in ascending f, ranked in `twice` while the table is cleared
+      const int32_t n = *s_nsurv;
+      dirty_once = max(dirty_once, min(n, kSpList));  // the list
+      if (*s_ovf || (emit && n > kSpSortMax)) {
+        hand_over = true;
+        clear_slots<NT>(tab, T);
+      } else if (emit && n > 0) {
+        if (tid == 0) *s_base = reserve(a, e, n, kBinFlat);
+        dirty_twice = max(dirty_twice, 2 * ((n + 31) & ~31));
+        for (int32_t i = tid; i < n; i += NT)
+          keys[i] = tab[list[i]] + 1ull;  // the count word holds count - 1
+        __syncthreads();  // keys and base in place, the table is read
+        const long long base = *s_base;
+        clear_slots<NT>(tab, T);
+        rank_keys<NT>(keys, n, [&](int32_t i, unsigned long long x) {
+          if (base >= 0) put(a, base, i, e, (int32_t)(x >> 32), (int32_t)(uint32_t)x);
+        });
+      } else {
+        if (tid == 0) reserve(a, e, n, kBinFlat);
+        clear_slots<NT>(tab, T);
+      }
+    }
+    lap(3);
+    __syncthreads();  // keys and list are read
+    zero(once, dirty_once);
+    zero(twice, dirty_twice);
+    if (hand_over && tid == 0) {  // to the giant bin (launched after this kernel)
+      const unsigned pos = atomicAdd(&meta->giant_rest, 1u);
+      giant_rows[list_len - 1 - pos] = e;
+      atomicAdd(&meta->rows_bin[kBinGiant], 1ull);
+    }
+    lap(4);
+  }
+  if (tid == 0)
+    for (int i = 0; i < 5; ++i) atomicAdd(&meta->sparse_cycles[i], (unsigned long long)s_cyc[i]);
+}
+
 // ------------------------------------------------------------- short rows --
 //
 // Rows of at most kCtaSMaxWork wedges with s >= 2, a warp each: 4 KB of shared
@@ -714,11 +938,27 @@ __global__ __launch_bounds__(kRwNT, SLG_RW_MINB) void k_walk_rows(
   }
 }
 
+// The flat bin's rows behind the sparse bin's, at both ends of its list.
+__global__ __launch_bounds__(256) void k_join_flat(const int32_t *__restrict__ flat,
+                                                   int32_t *__restrict__ sparse,
+                                                   int32_t list_len, unsigned flat_huge,
+                                                   unsigned flat_rest, unsigned huge,
+                                                   unsigned rest, Meta *meta) {
+  const unsigned t = blockIdx.x * 256 + threadIdx.x;
+  if (t < flat_huge) sparse[huge + t] = flat[t];
+  if (t < flat_rest) sparse[list_len - 1 - (rest + t)] = flat[list_len - 1 - t];
+  if (t == 0) {
+    meta->sparse_huge = huge + flat_huge;
+    meta->sparse_rest = rest + flat_rest;
+  }
+}
+
 constexpr size_t rows_smem() { return kRwNW * (sizeof(RwShared) + 8); }
 
 struct SpOcc {
   int small = 0, big = 0;  // CTAs
   int rows = 0;            // CTAs of k_walk_rows
+  int flat_small = 0, flat_big = 0;
   int dev = -1;
 };
 
@@ -728,6 +968,15 @@ int sp_ctas(int sms) {
   cudaFuncSetAttribute(k_walk_sparse<C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        (int)sparse_smem<C>());
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_walk_sparse<C>, C::NT, sparse_smem<C>());
+  return sms * std::max(nb, 1);
+}
+
+template <class C>
+int fl_ctas(int sms) {
+  int nb = 0;
+  cudaFuncSetAttribute(k_walk_flat<C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                       (int)flat_smem<C>());
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_walk_flat<C>, C::NT, flat_smem<C>());
   return sms * std::max(nb, 1);
 }
 
@@ -748,9 +997,20 @@ SpOcc &sp_occ() {
                          (int)rows_smem());
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_walk_rows, kRwNT, rows_smem());
     o.rows = sms * std::max(nb, 1);
+    o.flat_small = fl_ctas<FlSmall>(sms);
+    o.flat_big = fl_ctas<FlBig>(sms);
     o.dev = dev;
   }
   return o;
+}
+
+template <class C>
+void fl_launch(const WalkLaunch &L, int ctas, int part, cudaStream_t st) {
+  const int64_t stride = L.rows;
+  k_walk_flat<C><<<ctas, C::NT, flat_smem<C>(), st>>>(
+      L.w, L.bin_rows + (int64_t)kBinFlat * stride, L.a,
+      const_cast<int32_t *>(L.bin_rows) + (int64_t)kBinGiant * stride, (int32_t)stride,
+      L.sparse_scratch, (L.sparse_ints / (long long)ctas) & ~31ll, part);
 }
 
 template <class C>
@@ -767,8 +1027,21 @@ void sp_launch(const WalkLaunch &L, int ctas, int part, cudaStream_t st) {
 // Scratch ints for rows of up to `max_work` wedges.
 long long sparse_ints(int32_t max_work) {
   SpOcc &o = sp_occ();
-  return std::max((long long)o.small * (std::min(max_work, kSparseBigWork) + 128ll),
-                  (long long)o.big * (max_work + 128ll));
+  return std::max({(long long)std::max(o.small, o.flat_small) *
+                       (std::min(max_work, kSparseBigWork) + 128ll),
+                   (long long)o.flat_big * (std::min(max_work, kFlatMaxWork) + 128ll),
+                   (long long)o.big * (max_work + 128ll)});
+}
+
+// Gives the flat bin's rows to the sparse bin (m: the planning's totals).
+cudaError_t launch_join_flat(int32_t *bin_rows, int32_t rows, const Meta &m, Meta *meta,
+                             cudaStream_t st) {
+  const unsigned n = std::max(m.flat_huge, m.flat_rest);
+  if (n == 0) return cudaSuccess;
+  k_join_flat<<<(n + 255) / 256, 256, 0, st>>>(
+      bin_rows + (int64_t)kBinFlat * rows, bin_rows + (int64_t)kBinSparse * rows, rows, m.flat_huge,
+      m.flat_rest, m.sparse_huge, m.sparse_rest, meta);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_walk_rows(const WalkLaunch &L, cudaStream_t st) {
@@ -788,6 +1061,14 @@ cudaError_t launch_walk_sparse(const WalkLaunch &L, cudaStream_t st, int32_t *la
   }
   if (!(L.skip & kSkipSparseSmall)) {
     sp_launch<SpSmall>(L, o.small, 1, st);
+    ++*launches;
+  }
+  if (!(L.skip & kSkipFlatBig)) {
+    fl_launch<FlBig>(L, o.flat_big, 0, st);
+    ++*launches;
+  }
+  if (!(L.skip & kSkipFlatSmall)) {
+    fl_launch<FlSmall>(L, o.flat_small, 1, st);
     ++*launches;
   }
   return cudaGetLastError();

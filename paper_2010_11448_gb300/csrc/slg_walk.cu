@@ -13,6 +13,8 @@
 //   dense bin  (slg_dense.cu):  rows with enough wedges for their id span are
 //                               counted in windows of packed counters;
 //   sparse bin (slg_sparse.cu): other rows with s >= 2, up to 65,536 wedges;
+//   flat bin   (slg_sparse.cu): of these, rows of many short tails, up to
+//                               16,384 wedges;
 //   rows bin   (slg_sparse.cu): rows with s >= 2 and work <= 1024, a warp each
 //                               (the warp and CTA bins keep the s = 1 rows);
 //   giant bin  (the rest):      a CTA splits the row's far ends into f-range
@@ -784,11 +786,13 @@ cudaError_t launch_walk(const WalkLaunch &L, cudaStream_t st, int32_t *launches,
   };
   auto empty = [&](int bin) { return (L.skip >> bin) & 1u; };
   static thread_local SideStreams side;
-  const bool has_sparse = L.sparse_scratch && (L.skip & (kSkipSparseBig | kSkipSparseSmall)) !=
-                                                  (kSkipSparseBig | kSkipSparseSmall);
+  constexpr unsigned kSkipSparse =
+      kSkipSparseBig | kSkipSparseSmall | kSkipFlatBig | kSkipFlatSmall;
+  const bool has_sparse = L.sparse_scratch && (L.skip & kSkipSparse) != kSkipSparse;
   const bool dense_big = L.dense_pairs[0] > 0, dense_small = L.dense_pairs[1] > 0;
   const bool chain = has_sparse || dense_small;
-  const bool ctas = !empty(kBinWarp) || !empty(kBinCtaS) || !empty(kBinCtaL) || !empty(kBinRows);
+  const bool ctas = !empty(kBinWarp) || !empty(kBinCtaS) || !empty(kBinCtaL) ||
+                    !empty(kBinRows);
   const bool fork = !ev && dense_big && (chain || ctas) && side.ready(st);
   const bool use[2] = {fork && chain, fork && ctas};
   cudaStream_t s1 = use[0] ? side.s[0] : st, s2 = use[1] ? side.s[1] : st;

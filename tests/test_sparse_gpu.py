@@ -242,3 +242,67 @@ def test_short_rows(k, deg):
         assert w is None and np.array_equal(
             np.stack([i.cpu().numpy(), j.cpu().numpy()], 1), want[:, :2])
         assert slg.count(dh, s) == want.shape[0]
+
+
+# the flat bin: rows of more than 48 vertices with less than 32 far ends per tail
+# on average, 1,025 to 16,384 wedges, above 8,192 in the instance with the larger
+# table.  Both sides of each of these limits, one batch of tails (256) and more,
+# more survivors than it orders (992: handed over), tails of no far end
+@pytest.mark.parametrize("k,lens,repeat", [
+    (48, (31, 32), 3), (49, (31,), 3), (49, (32,), 3), (49, (0, 62), 3), (256, (1, 7, 8, 9), 3),
+    (257, (0, 1, 8, 9, 31, 32, 33), 3), (300, (4,), 3), (512, (16,), 3), (513, (16, 17), 3),
+    (512, (16,), 8), (1_024, (16,), 3), (1_025, (16,), 4), (1_000, (0, 1, 30), 2),
+    (600, (25,), 15)])
+@pytest.mark.parametrize("mixed", [False, True])
+def test_short_tails(k, lens, repeat, mixed):
+    m, n = 2_000_000, 120_000
+    rng = np.random.default_rng(k + repeat)
+    total = sum(lens[v % len(lens)] for v in range(k))
+    r, c = [np.zeros(k, np.int64)], [np.arange(k)]
+    pool = rng.choice(np.arange(10, m), max(total // repeat, 100), replace=False)
+    for v in range(k):  # far ends from a pool: most occur in several tails
+        d = lens[v % len(lens)]
+        r.append(rng.choice(pool, d, replace=False))
+        c.append(np.full(d, v))
+    r.append(np.repeat(pool, 3))
+    c.append(rng.integers(10_000, n, 3 * pool.size))
+    if mixed:  # more wedges in a row of long tails: the sparse bin takes both rows
+        for v in range(9):
+            f = rng.choice(pool, pool.size // 2, replace=False) if v < 2 else \
+                rng.choice(np.arange(10, m), 5_000, replace=False)
+            r += [f, np.ones(1, np.int64)]
+            c += [np.full(f.size, 5_000 + v), np.full(1, 5_000 + v)]
+    h = hg.from_pairs(np.concatenate(r), np.concatenate(c), m, n)
+    dh = slg.to_device(h)
+    for s in (2, 3, 4, 6):
+        want = oracle.canonical(*oracle.line_graph_of(h, s, threads=8))
+        got = as_np(slg.build(dh, s))
+        assert np.array_equal(got, want), s
+        i, j, w = slg.build(dh, s, unweighted=True)
+        assert w is None and np.array_equal(
+            np.stack([i.cpu().numpy(), j.cpu().numpy()], 1), want[:, :2])
+        assert slg.count(dh, s) == want.shape[0]
+        if s == 3:
+            plan = slg.Plan([dh], [s])
+            plan.execute()
+            assert np.array_equal(as_np(plan.results()[0]), want)
+
+
+def test_short_tails_do_not_take_a_warp_each():
+    """100,000 rows of 250 vertices with a mean of 13 rows per vertex: nothing
+    but short tails.  A warp per tail and a rank among all tails took 58 CTA cycles
+    per wedge, flattened tails 11."""
+    m, n = 100_000, 1_900_000
+    gen = torch.Generator(device="cuda").manual_seed(1)
+    rows = torch.arange(m, device="cuda").repeat_interleave(250)
+    cols = torch.randint(0, n, rows.shape, generator=gen, device="cuda")
+    key = torch.unique(rows * n + cols)
+    rows, cols = key // n, key % n
+    by = torch.argsort(cols, stable=True)
+    off = lambda x, k: torch.nn.functional.pad(torch.bincount(x, minlength=k).cumsum(0),
+                                               (1, 0)).int()
+    dh = slg.DeviceHypergraph(m, n, off(rows, m), cols.int(), off(cols, n), rows[by].int())
+    slg.count(dh, 2)
+    st = slg.last_stats()
+    assert st["rows_bin"][4] > 30_000
+    assert sum(st["sparse_cycles"]) < 25 * st["wedges_bin"][4]
