@@ -125,7 +125,14 @@ constexpr int kDenseRatio = 16;
 
 // Dense rows: the dense bin's cost per row is its wedges plus so much per
 // window (sweep latency, survivors, clear), the other bins' is their cost per
-// wedge; so the line is drawn at a number of wedges per window.
+// wedge; so the line is drawn at a number of wedges per window.  A window also
+// visits every tail, which the other bins read once: in the large-window
+// instance, whose rows can have more tails than wedges per window, a visit after
+// the first counts as 2.5 wedges (a quarter at s = 1, where hash tables would
+// count the row).  400K rows of 1,500 of 67M vertices, counting pass at s = 2
+// 112.7, 95.3, 90.6 ms with 0.25, 1, 2.5 (125.3 without), at s = 1 117.6, 119.6,
+// 121.3; rows of up to 100,000 vertices over 4M ids (web-shaped input with the
+// tile path) 4.6 -> 1.75 ms; step of chung_lu_1m the same all ways.
 __host__ __device__ __forceinline__ bool is_dense(int32_t work, int32_t size, int32_t s,
                                                   int32_t span, int32_t ratio) {
   const int lw = 5 - dense_lg_bits(size);
@@ -135,7 +142,8 @@ __host__ __device__ __forceinline__ bool is_dense(int32_t work, int32_t size, in
                       : s == 1                                     ? SLG_DENSE_T1
                       : size <= (long long)kDenseFew * (s - 2) ? SLG_DENSE_T4
                                                                    : SLG_DENSE_T2;
-  return (long long)work * ratio >= (long long)per * 16 * nwin;
+  const long long visits = big ? (nwin - 1ll) * size * (s == 1 ? 4 : 40) : 0;
+  return (long long)work * ratio >= (long long)per * 16 * nwin + visits;
 }
 
 // Counters the device writes and the host reads once per call.

@@ -102,3 +102,27 @@ def test_split_tails(tails, spread):
         want = oracle.canonical(*oracle.line_graph_of(h, s, threads=8))
         assert np.array_equal(as_np(slg.build(dh, s)), want), s
         assert slg.count(dh, s) == want.shape[0]
+
+
+def test_more_tails_than_wedges_per_window():
+    """Row 0 has 20,000 vertices and 21 windows of 96K ids.  With tails of 3 far
+    ends a window has a seventh of a wedge per visited tail, and the row is counted
+    elsewhere although it has 2,000 wedges per window; with tails of 60 it is dense."""
+    m, k = 2_000_000, 20_000
+    for tail, dense in ((3, False), (60, True)):
+        rng = np.random.default_rng(tail)
+        r = np.concatenate([np.zeros(k, np.int64), rng.integers(1, m, k * tail)])
+        c = np.concatenate([np.arange(k), np.repeat(np.arange(k), tail)])
+        extra = rng.integers(k, k + 50_000, 2 * k * tail)  # far ends of three vertices
+        h = hg.from_pairs(np.concatenate([r, np.repeat(r[k:], 2)]), np.concatenate([c, extra]),
+                          m, k + 50_000)
+        dh = slg.to_device(h)
+        n, nv, off, idx = oracle.side(h, False)
+        for s in (2, 3):
+            want = oracle.canonical(*oracle.line_graph(n, nv, off, idx, s,
+                                                       rows=np.zeros(1, np.int32), threads=8))
+            pairs = int(slg.row_offsets(dh, s)[1])
+            i, j, w = slg.build_rows(dh, s, 0, 1, capacity=max(pairs, 1))
+            st = slg.last_stats()
+            assert (st["giant_cycles"][3] > 0) == dense, (tail, s)
+            assert np.array_equal(as_np((i, j, w)), want), (tail, s)
