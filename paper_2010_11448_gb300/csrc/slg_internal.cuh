@@ -25,7 +25,8 @@ constexpr int32_t kEmpty = -1;
 // Bins::sparse wedges go to the sparse bin (the flat bin, if their tails are
 // short: short_tails) and the rest above the CTA bins to
 // the giant bin.  Rows with s >= 2 of at most Bins::ctas
-// wedges take the rows bin (a warp each), s = 1 ones the warp and CTA bins.
+// wedges take the rows bin (a warp each; of more than kRowsMaxSize vertices the
+// small CTA bin), s = 1 ones the warp and CTA bins.
 // The statistics count the dense bin's rows as giant ones, the rows bin's as
 // the small CTA bin's and the flat bin's as sparse ones (kNumBins bins are
 // reported, kNumLists lists kept).
@@ -74,6 +75,14 @@ __host__ __device__ __forceinline__ bool short_tails(int32_t work, int32_t size)
 __host__ __device__ __forceinline__ bool flat_kernels(long long flat, long long sparse) {
   return flat > 0 && (2 * flat >= sparse || flat >= 1ll << 26);
 }
+// Rows of more vertices leave the rows bin to the small CTA bin: the kernel lasts
+// as long as its longest row, and a warp there walks 32 tails at a time, a CTA 256
+// (rows of few wedges: late ids, or vertices that few other rows hold).  4 rows of
+// 100,000 vertices and 500 wedges 2.65 -> 0.85 ms, 50 of 20,000 0.84 -> 0.51; with
+// many such rows the warps do better (10,000 of 1,000 vertices 0.20 instead of
+// 0.67), and a few large rows are no reason to run the CTA bin's kernel (lines at
+// 256 to 1,024: counting pass of 120K x 240K 805 -> 853 us, batch of 16 5 % more).
+constexpr int32_t kRowsMaxSize = 16384;
 #ifndef SLG_DENSE_MIN_WORK
 #define SLG_DENSE_MIN_WORK 256
 #endif

@@ -391,7 +391,7 @@ __global__ __launch_bounds__(kRowsNT) void k_rows_work(Side s, int32_t smin, int
         else if (my_work <= kFlatMaxWork) my_bin = kBinFlat;
       }
       else if (!forced && my_work <= bins.ctas && se >= 2)
-        my_bin = kBinRows;
+        my_bin = size <= kRowsMaxSize ? kBinRows : kBinCtaS;
       if (my_bin == kBinGiant) atomicMax(&s_max[1], my_work);
       if (my_bin == kBinSparse || my_bin == kBinFlat) atomicMax(&s_max[2], my_work);
       if (my_bin == kBinDense) {

@@ -306,3 +306,47 @@ def test_short_tails_do_not_take_a_warp_each():
     st = slg.last_stats()
     assert st["rows_bin"][4] > 30_000
     assert sum(st["sparse_cycles"]) < 25 * st["wedges_bin"][4]
+
+
+def hubs(k, count, m=40_000, shared=500, seed=7):
+    """`count` rows with late ids of `k` vertices each, of which `shared` draws are
+    in one later row: many tails, almost all of them empty."""
+    rng = np.random.default_rng(seed)
+    base = np.repeat(np.arange(m - 2 * count), 3)
+    hub = np.arange(count)
+    r = [base, np.repeat(m - 2 * count + hub, k), np.repeat(m - count + hub, shared)]
+    c = [rng.integers(0, 50_000, base.size),
+         50_000 + (hub[:, None] * k + np.arange(k)).ravel(),
+         50_000 + (hub[:, None] * k + rng.integers(0, k, (count, shared))).ravel()]
+    return hg.from_pairs(np.concatenate(r), np.concatenate(c), m, 50_000 + count * k)
+
+
+# on both sides of the 16,384 vertices up to which a warp takes a row
+@pytest.mark.parametrize("k", [16_383, 16_384, 16_385, 40_000])
+def test_rows_of_many_vertices_and_few_wedges(k):
+    h = hubs(k, 10)
+    dh = slg.to_device(h)
+    for s in (2, 3, 50):
+        want = oracle.canonical(*oracle.line_graph_of(h, s, threads=8))
+        assert np.array_equal(as_np(slg.build(dh, s)), want), s
+        assert slg.count(dh, s) == want.shape[0]
+        i, j, w = slg.build(dh, s, unweighted=True)
+        assert w is None and np.array_equal(
+            np.stack([i.cpu().numpy(), j.cpu().numpy()], 1), want[:, :2])
+
+
+def test_rows_of_many_vertices_are_not_left_to_a_warp():
+    """At s = 1 a CTA walks such a row; a warp took three times as long."""
+    dh = slg.to_device(hubs(100_000, 4))
+    slg.set_profiling(True)
+    try:
+        ms = {}
+        for s in (1, 2):
+            got = []
+            for _ in range(5):
+                slg.count(dh, s)
+                got.append(slg.last_stats()["ms_walk"][1])
+            ms[s] = sorted(got)[2]
+    finally:
+        slg.set_profiling(False)
+    assert ms[2] < 1.7 * ms[1], ms
