@@ -486,11 +486,16 @@ int plan_core(Call &c, CoreInfo *core) {
   return SLG_OK;
 }
 
-// The caller's outputs for `pairs` pairs (Call::alloc).
+// The caller's outputs for `pairs` pairs (Call::alloc).  The callback may call the
+// library itself, on this thread, whose calls all leave their totals in the one
+// Meta that this call still reads.
 int call_alloc(Call &c, int64_t pairs) {
   c.capacity = pairs;
   if (pairs == 0) return SLG_OK;
-  if (c.alloc(c.alloc_ctx, pairs, &c.out_i, &c.out_j, &c.out_w) != 0) return SLG_ERR_NOMEM;
+  const Meta totals = *c.meta_host;
+  const int refused = c.alloc(c.alloc_ctx, pairs, &c.out_i, &c.out_j, &c.out_w);
+  *c.meta_host = totals;
+  if (refused) return SLG_ERR_NOMEM;
   return (c.out_i || c.rows_form) && c.out_j && (c.unweighted || c.out_w) ? SLG_OK
                                                                            : SLG_ERR_INVALID;
 }

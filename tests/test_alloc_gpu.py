@@ -83,3 +83,32 @@ def test_refused():
     with pytest.raises(slg.SlgError) as ei:
         slg.build(dh, 0)
     assert ei.value.status == 1
+
+
+# the short path and the general one, lists that fit the staging area and longer ones
+@pytest.mark.parametrize("count,size,extra", [(20, 30, 0), (20, 800, 0), (20, 30, 20_000),
+                                              (20_000, 24, 0)])
+def test_the_callback_may_call_the_library(count, size, extra):
+    h = groups(count, size, 2, extra)
+    dh = slg.to_device(h)
+    other = [slg.to_device(hg.uniform(m, 2 * m, 1, 20, seed=4)) for m in (300, 30_000)]
+    want = [slg.count(x, 1) for x in other]
+    ref = slg.build(dh, 2, capacity=slg.count(dh, 2))
+    stats = slg.last_stats()
+    out, seen = [], []
+
+    def alloc(_, n, oi, oj, ow):
+        seen.extend(slg.count(x, 1) for x in other)
+        out.extend(torch.full((n,), -1, dtype=torch.int32, device="cuda") for _ in range(3))
+        for p, t in zip((oi, oj, ow), out):
+            p[0] = t.data_ptr()
+        return 0
+
+    n = ctypes.c_int64(0)
+    rc = slg.load().slg_build_alloc(ctypes.byref(dh.struct), 2, 0, None, slg._AllocFn(alloc), None,
+                                    ctypes.byref(n), None)
+    torch.cuda.synchronize()
+    assert rc == 0 and seen == want and n.value == ref[0].numel()
+    assert all(torch.equal(a, b) for a, b in zip(out, ref))
+    got = slg.last_stats()
+    assert all(got[k] == stats[k] for k in ("wedges", "pairs", "rows_active", "rows_bin"))
