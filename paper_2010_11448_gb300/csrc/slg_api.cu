@@ -629,7 +629,11 @@ int run_binned(Call &c, int64_t *result) {
   }
   if (pairs > c.capacity) return SLG_ERR_CAPACITY;
   if (m.stage_overflow == 0) return SLG_OK;
-  // Staging too small: walk again, writing straight to the output.
+  // Staging too small: walk again, writing straight to the output.  The rows'
+  // pairs and cycles are counted anew.
+  SLG_TRY(cudaMemsetAsync(w.meta->pairs_bin, 0, sizeof(w.meta->pairs_bin), c.st));
+  SLG_TRY(cudaMemsetAsync(w.meta->giant_cycles, 0, sizeof(w.meta->giant_cycles), c.st));
+  SLG_TRY(cudaMemsetAsync(w.meta->sparse_cycles, 0, sizeof(w.meta->sparse_cycles), c.st));
   SLG_TRY(cudaMemsetAsync(&w.meta->giant_ticket, 0, sizeof(unsigned int), c.st));
   static_assert(offsetof(Meta, dense_ticket_rest) ==
                     offsetof(Meta, dense_ticket) + sizeof(unsigned int),

@@ -112,3 +112,16 @@ def test_the_callback_may_call_the_library(count, size, extra):
     assert all(torch.equal(a, b) for a, b in zip(out, ref))
     got = slg.last_stats()
     assert all(got[k] == stats[k] for k in ("wedges", "pairs", "rows_active", "rows_bin"))
+
+
+def test_statistics_of_a_list_walked_twice():
+    # warp-sized rows; rows of the dense and the sparse bin
+    for args in ((20_000, 24, 2, 0), (10, 3_000, 2, 0), (10, 3_000, 2, 500_000)):
+        dh = slg.to_device(groups(*args))
+        once = slg.build(dh, 2, capacity=slg.count(dh, 2))
+        want = slg.last_stats()
+        got = slg.build(dh, 2)
+        st = slg.last_stats()
+        assert st["pairs"] == got[0].numel() == once[0].numel()
+        assert sum(st["pairs_bin"]) == st["pairs"] and st["pairs_bin"] == want["pairs_bin"]
+        assert st["rows_bin"] == want["rows_bin"]
