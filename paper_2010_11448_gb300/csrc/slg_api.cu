@@ -168,6 +168,15 @@ struct Pool {
     *p = static_cast<T *>(q);
     return cudaSuccess;
   }
+  template <class T>
+  void give_back(T **p) {
+    const auto it = std::find(ptrs.begin(), ptrs.end(), static_cast<void *>(*p));
+    if (*p && it != ptrs.end()) {
+      cudaFreeAsync(*p, st);
+      ptrs.erase(it);
+    }
+    *p = nullptr;
+  }
   ~Pool() {
     for (void *q : ptrs) cudaFreeAsync(q, st);
   }
@@ -526,24 +535,14 @@ int run_binned(Call &c, int64_t *result) {
   }
   auto stage = [&](int64_t cap) {
     w.stage_cap = 0;  // rows that find no staging room are re-walked directly
-    if (cap > 0 && c.pool->get(&w.stage_j, (size_t)cap) == cudaSuccess &&
-        (c.unweighted || c.pool->get(&w.stage_w, (size_t)cap) == cudaSuccess))
-      w.stage_cap = cap;
+    if (cap <= 0 || c.pool->get(&w.stage_j, (size_t)cap) != cudaSuccess) return;
+    if (c.unweighted || c.pool->get(&w.stage_w, (size_t)cap) == cudaSuccess) w.stage_cap = cap;
+    else c.pool->give_back(&w.stage_j);
   };
   if (c.op == kOpBuild && !c.alloc) stage(c.capacity);
   // Planning totals: the giant bin's scratch is sized by its largest row.
   int rc = read_meta(c);
   if (rc) return rc;
-  if (c.alloc) {
-    // The pairs are not known yet.  Each has at least s wedges; on real
-    // lists an eighth of the wedges at s = 2 is plenty (0.06 to 0.08 on
-    // chung_lu_1m), and a list that is longer is walked again.
-    const int64_t W = (int64_t)c.meta_host->wedges;
-    int64_t cap = W / c.smin;
-    if (c.smin > 1) cap = std::min(cap, std::max<int64_t>(W / 8, (int64_t)1 << 22));
-    if (core.T) cap += (int64_t)core.n_core * core.n_core / 2;
-    stage(std::max<int64_t>(cap, 1));
-  }
   // (core rows may have no wedges but still need a giant CTA; their pairs,
   // staged in the same scratch, also come from up to n_core tile items)
   // (a row of the sparse, flat or rows bin that overflows its table is handed to
@@ -570,6 +569,22 @@ int run_binned(Call &c, int64_t *result) {
                         dense_pairs(mp.dense_huge, mp.max_dense_work[0]),
                         dense_pairs(mp.dense_rest, mp.max_dense_work[1]), mp.max_dense_size,
                         &L));
+  if (c.alloc) {
+    // The pairs are not known yet.  Each has at least s wedges; on real
+    // lists an eighth of the wedges at s = 2 is plenty (0.06 to 0.08 on
+    // chung_lu_1m), and a list that is longer is walked again.  Far more wedges
+    // than pairs (many vertices shared by a few rows) are no reason to take the
+    // device's memory: kMaxGuess at most, 2 GB, and after the scratch.
+    constexpr int64_t kMaxGuess = (int64_t)1 << 28;
+    const int64_t W = (int64_t)mp.wedges;
+    int64_t cap = W / c.smin;
+    if (c.smin > 1) cap = std::min(cap, std::max<int64_t>(W / 8, (int64_t)1 << 22));
+    if (core.T) cap += (int64_t)core.n_core * core.n_core / 2;
+    stage(std::min(std::max<int64_t>(cap, 1), kMaxGuess));
+    L.a.stage_j = w.stage_j;
+    L.a.stage_w = w.stage_w;
+    L.a.stage_cap = w.stage_cap;
+  }
   L.w.r_off = c.sd.r_off;
   L.w.r_idx = c.sd.r_idx;
   L.w.c_idx_s = w.c_idx_s;

@@ -125,3 +125,27 @@ def test_statistics_of_a_list_walked_twice():
         assert st["pairs"] == got[0].numel() == once[0].numel()
         assert sum(st["pairs_bin"]) == st["pairs"] and st["pairs_bin"] == want["pairs_bin"]
         assert st["rows_bin"] == want["rows_bin"]
+
+
+def test_far_more_wedges_than_pairs():
+    """400 rows with the same 40,000 vertices: 3.2e9 wedges, 79,800 pairs.  The
+    staging area does not grow with the wedges."""
+    m, rows, k = 20_000, 400, 40_000
+    ids = torch.arange(rows, device="cuda", dtype=torch.int32) * 50
+    e_off = torch.zeros(m + 1, dtype=torch.int64, device="cuda")
+    e_off[ids.long() + 1] = k
+    dh = slg.DeviceHypergraph(
+        m, k, e_off.cumsum(0).int(), torch.arange(k, device="cuda", dtype=torch.int32).repeat(rows),
+        torch.arange(k + 1, device="cuda", dtype=torch.int32) * rows, ids.repeat(k))
+    want = torch.triu_indices(rows, rows, 1, device="cuda") * 50
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    slg.release_memory()
+    free = torch.cuda.mem_get_info()[0]
+    for s in (1, 2, k):
+        i, j, w = slg.build(dh, s)
+        assert torch.equal(i, want[0].int()) and torch.equal(j, want[1].int())
+        assert bool((w == k).all())
+    torch.cuda.synchronize()
+    assert free - torch.cuda.mem_get_info()[0] < 5 << 30
+    slg.release_memory()
