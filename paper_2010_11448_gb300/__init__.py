@@ -47,6 +47,7 @@ _ALGOS = {"binned": SLG_ALGO_BINNED, "plain": SLG_ALGO_PLAIN,
 _RELABEL = {None: 0, "asc": SLG_RELABEL_ASC, "desc": SLG_RELABEL_DESC}
 
 SLG_ERR_CAPACITY = 2
+SLG_ERR_NOMEM = 3
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 
@@ -288,8 +289,9 @@ def _outputs(capacity, unweighted, device):
 
 def _build_alloc(fn, what, arg, s, flags, unweighted, device, stream, row_ptr=None):
     """One walk, the outputs allocated by the pair count it finds
-    (slg_build_alloc): (i, j, w), i None with `row_ptr`; None when the outputs
-    could not be allocated next to the walk's memory."""
+    (slg_build_alloc): (i, j, w), i None with `row_ptr`; None when the walk's
+    memory or the outputs beside it could not be had: what the library keeps
+    for later calls is given back then, for a build that counts first."""
     import torch
     got = {}
 
@@ -303,7 +305,7 @@ def _build_alloc(fn, what, arg, s, flags, unweighted, device, stream, row_ptr=No
                     p[0] = t.data_ptr()
             return 0
         except torch.cuda.OutOfMemoryError:
-            got["oom"] = True
+            pass
         except BaseException as exc:  # noqa: B902 - raised again below
             got["exc"] = exc
         return 1
@@ -314,7 +316,9 @@ def _build_alloc(fn, what, arg, s, flags, unweighted, device, stream, row_ptr=No
             ctypes.byref(n), _stream(stream))
     if "exc" in got:
         raise got["exc"]
-    if "oom" in got:
+    if rc == SLG_ERR_NOMEM:
+        got.clear()
+        release_memory()
         return None
     if rc != 0:
         raise SlgError(rc, what)

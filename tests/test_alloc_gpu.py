@@ -149,3 +149,42 @@ def test_far_more_wedges_than_pairs():
     torch.cuda.synchronize()
     assert free - torch.cuda.mem_get_info()[0] < 5 << 30
     slg.release_memory()
+
+
+@pytest.mark.parametrize("form", ["build", "graph", "csr"])
+def test_outputs_that_cannot_be_had_beside_the_walk(form, monkeypatch):
+    """torch's allocator refuses while the walk's memory is held: the library's
+    memory is given back before the build is done over, counting first."""
+    h = groups(200, 24, 2, 20_000)
+    dh = slg.to_device(h)
+    want = slg.build(dh, 2, capacity=slg.count(dh, 2))
+    real_out, real_release, log = slg._outputs, slg.release_memory, []
+
+    def outputs(n, unweighted, device):
+        log.append("outputs")
+        if len(log) == 1:
+            raise torch.cuda.OutOfMemoryError("no memory")
+        return real_out(n, unweighted, device)
+
+    def release():
+        log.append("release")
+        real_release()
+
+    monkeypatch.setattr(slg, "_outputs", outputs)
+    monkeypatch.setattr(slg, "release_memory", release)
+    if form == "csr":
+        got = slg.build_csr(dh, 2)[1:]
+    elif form == "graph":
+        with slg.Graph(dh) as g:
+            got = g.build(2)[1:]
+    else:
+        got = slg.build(dh, 2)[1:]
+    assert log == ["outputs", "release", "outputs"]
+    assert all(torch.equal(a, b) for a, b in zip(got, want[1:]))
+
+
+def test_no_memory_in_the_library(monkeypatch):
+    released = []
+    monkeypatch.setattr(slg, "release_memory", lambda: released.append(1))
+    got = slg._build_alloc(lambda *a: 3, "slg_build", None, 2, 0, False, "cuda", None)
+    assert got is None and released == [1]
