@@ -913,7 +913,7 @@ int run(const slg_hypergraph *h, int32_t smin, uint32_t flags, int32_t row_begin
         int32_t *max_row_work = nullptr, long long *row_ptr_out = nullptr,
         int32_t *row_work_out = nullptr, const int32_t *row_fhi = nullptr,
         int32_t *max_row_size = nullptr, slg_alloc_fn alloc = nullptr,
-        void *alloc_ctx = nullptr, bool *flat = nullptr) {
+        void *alloc_ctx = nullptr, Meta *totals = nullptr) {
   int rc = check_args(h, smin, flags);
   if (rc != SLG_OK) return rc;
   if (!result) return SLG_ERR_INVALID;
@@ -1084,7 +1084,7 @@ int run(const slg_hypergraph *h, int32_t smin, uint32_t flags, int32_t row_begin
   stats.pairs_bin[kBinGiant] += (int64_t)m.pairs_bin[kBinDense];
   if (max_row_work) *max_row_work = m.max_row_work;
   if (max_row_size) *max_row_size = m.max_row_size;
-  if (flat) *flat = flat_kernels(m.wedges_bin[kBinFlat], m.wedges_bin[kBinSparse]);
+  if (totals) *totals = m;
   stats.kernel_launches = c.launches;
   stats.core_rows = c.core_rows;
   stats.core_cols = c.core_cols;
@@ -1940,10 +1940,10 @@ extern "C" int slg_plan_create(const slg_hypergraph *hs, const int32_t *s, int32
   // 2. sizes: one counting pass over the union (per-row thresholds)
   int64_t pairs = 0;
   int32_t max_work = 0, max_size = 0;
-  bool flat = false;  // the flat bin has kernels of its own
+  Meta t = {};
   int rc = run(&p->u, 1, flags, 0, p->sd.R, kOpCount, nullptr, nullptr, nullptr, 0, &pairs, st,
                p->sd.row_s, &max_work, nullptr, nullptr, p->sd.row_fhi, &max_size, nullptr, nullptr,
-               &flat);
+               &t);
   if (rc != SLG_OK) return rc;
   p->pairs = pairs;
   // 3. persistent buffers
@@ -1971,9 +1971,10 @@ extern "C" int slg_plan_create(const slg_hypergraph *hs, const int32_t *s, int32
   SLG_TRY(p->mem.get(&p->out_w, (size_t)std::max<int64_t>(pairs, 1)));
   SLG_TRY(p->mem.get(&p->offsets, (size_t)count + 1));
   if (max_work > 0) {
-    const size_t n = scratch_ints(&p->scratch, max_work, max_work, std::min<long long>(max_work, R),
-                                  std::min<long long>(max_work, R), max_size);
-    p->flat = flat;
+    const size_t n = scratch_ints(&p->scratch, max_work, t.plan_sparse,
+                                  std::min<long long>(t.plan_pairs[0], R),
+                                  std::min<long long>(t.plan_pairs[1], R), max_size);
+    p->flat = flat_kernels(t.wedges_bin[kBinFlat], t.wedges_bin[kBinSparse]);
     SLG_TRY(p->mem.get(&p->giant, n));
   }
   // 4. autotuner: bin thresholds, timed on this batch

@@ -184,6 +184,11 @@ struct Meta {
   int32_t max_dense_work[2];           // largest work of a dense-bin row: big instance, other
   int32_t max_dense_size;              // most vertices of a dense-bin row
   int32_t max_row_size;                // most vertices of a row with work
+  // Of a side with thresholds per row (a plan sizes its scratch by these, whatever
+  // its bins): most pairs a dense-bin row can have, big instance and other, and
+  // largest work of a row that the sparse bin could take.
+  int32_t plan_pairs[2];
+  int32_t plan_sparse;
   int32_t max_sparse_work;             // largest work of a sparse- or flat-bin row
   int32_t kept;                        // entries of the filtered CSC
   int32_t max_giant_work;              // largest work of a giant-bin row

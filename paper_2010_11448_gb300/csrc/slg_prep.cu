@@ -270,9 +270,10 @@ __global__ __launch_bounds__(kRowsNT) void k_rows_work(Side s, int32_t smin, int
   if (meta->err) return;
   __shared__ int32_t s_work[kRowsPerBlock];
   // block maxima of the row work (all rows, giant-bin, sparse- or flat-bin, the dense
-  // bin's two instances' rows) and size (dense-bin rows, all rows): one global atomicMax each per
+  // bin's two instances' rows) and size (dense-bin rows, all rows), and a plan's bounds: one
+  // global atomicMax each per
   // block instead of one per row
-  __shared__ int32_t s_max[7];
+  __shared__ int32_t s_max[10];
   __shared__ int32_t s_act;  // active rows (size >= s) of the block
   __shared__ int32_t s_cnt[kNumLists], s_base[kNumLists];
   __shared__ int32_t s_hcnt[4], s_hbase[4];  // giant / sparse / dense / flat rows handed out first
@@ -285,7 +286,7 @@ __global__ __launch_bounds__(kRowsNT) void k_rows_work(Side s, int32_t smin, int
     s_k[threadIdx.x] = 0;
   }
   if (threadIdx.x < 4) s_hcnt[threadIdx.x] = 0;
-  if (threadIdx.x < 7) s_max[threadIdx.x] = 0;
+  if (threadIdx.x < 10) s_max[threadIdx.x] = 0;
   if (threadIdx.x == 0) s_act = 0;
   __syncthreads();
   // eight lanes per row; long rows and core rows by the whole warp
@@ -392,6 +393,11 @@ __global__ __launch_bounds__(kRowsNT) void k_rows_work(Side s, int32_t smin, int
       }
       else if (!forced && my_work <= bins.ctas && se >= 2)
         my_bin = size <= kRowsMaxSize ? kBinRows : kBinCtaS;
+      if (s.row_s) {
+        if (my_work > kDenseMinWork)
+          atomicMax(&s_max[size > kDenseBigSize ? 7 : 8], max(my_work / se, 1));
+        if (se >= 2 && my_work <= kSparseMaxWork) atomicMax(&s_max[9], my_work);
+      }
       if (my_bin == kBinGiant) atomicMax(&s_max[1], my_work);
       if (my_bin == kBinSparse || my_bin == kBinFlat) atomicMax(&s_max[2], my_work);
       if (my_bin == kBinDense) {
@@ -445,6 +451,9 @@ __global__ __launch_bounds__(kRowsNT) void k_rows_work(Side s, int32_t smin, int
     if (s_max[6]) atomicMax(&meta->max_dense_work[1], s_max[6]);
     if (s_max[4]) atomicMax(&meta->max_dense_size, s_max[4]);
     if (s_max[5]) atomicMax(&meta->max_row_size, s_max[5]);
+    if (s_max[7]) atomicMax(&meta->plan_pairs[0], s_max[7]);
+    if (s_max[8]) atomicMax(&meta->plan_pairs[1], s_max[8]);
+    if (s_max[9]) atomicMax(&meta->plan_sparse, s_max[9]);
   }
   if (my_bin >= 0) {
     const int64_t len = row_end - row_begin;

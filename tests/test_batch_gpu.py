@@ -92,3 +92,34 @@ def test_union_beyond_one_super_chunk():
         assert np.array_equal(as_np(st), want), k
     filler = slg.build(dhs[2], ss[2])
     assert all(torch.equal(a, b) for a, b in zip(res[2], filler))
+
+
+def hub_member(k, deg, m=200_000, seed=1):
+    """Row 0 has k vertices of `deg` other rows each; all rows a few more."""
+    rng = np.random.default_rng(seed)
+    far = rng.integers(1, m, (k, deg))
+    r = np.concatenate([np.zeros(k, np.int64), far.ravel(), np.repeat(np.arange(m), 3)])
+    c = np.concatenate([np.arange(k), np.repeat(np.arange(k), deg),
+                        rng.integers(k, k + 4 * m, 3 * m)])
+    return hg.from_pairs(r, c, m, k + 4 * m)
+
+
+def test_plan_scratch_is_sized_by_the_rows_each_bin_can_have():
+    """A row of 120,000 wedges: the giant bin's share is 1,216 ints per wedge; the
+    others', side by side, were 1,976 whatever the row's size and threshold."""
+    hs = [hub_member(30, 4_000), hub_member(400, 20, seed=2)]
+    dhs = [slg.to_device(h) for h in hs]
+    slg.count(dhs[0], 2)
+    torch.cuda.synchronize()
+    slg.release_memory()
+    free = torch.cuda.mem_get_info()[0]
+    plan = slg.Plan(dhs, [2, 3])
+    plan.execute()
+    torch.cuda.synchronize()
+    slg.release_memory()  # what the creation left in the pool
+    used = free - torch.cuda.mem_get_info()[0]
+    for h, got, s in zip(hs, plan.results(), (2, 3)):
+        want = oracle.canonical(*oracle.line_graph_of(h, s, threads=8))
+        assert np.array_equal(np.stack([x.cpu().numpy() for x in got], 1), want)
+    incidences = sum(h.nnz for h in hs)
+    assert used < 4 * 1_300 * 120_000 + 100 * incidences + (64 << 20), used
