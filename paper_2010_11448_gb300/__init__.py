@@ -568,7 +568,12 @@ def filter_pairs(i, j, w, s: int, out=None, stream=None, weights=True):
         lib = load()
         cnt = ctypes.c_int64(0)
         lib.slg_filter_tiles(n, ctypes.byref(cnt))
-        tiles = torch.empty(cnt.value, dtype=torch.int64, device=i.device)
+        # taken from the allocator on the stream that uses them: on another, a
+        # block that is still being written there could be handed out
+        st = (torch.cuda.current_stream() if stream is None else
+              torch.cuda.ExternalStream(stream.cuda_stream, device=i.device))
+        with torch.cuda.stream(st):
+            tiles = torch.empty(cnt.value, dtype=torch.int64, device=i.device)
         rc = lib.slg_filter_count(w.data_ptr(), n, int(s), tiles.data_ptr(), ctypes.byref(cnt),
                                   _stream(stream))
         p = int(cnt.value)
@@ -579,7 +584,7 @@ def filter_pairs(i, j, w, s: int, out=None, stream=None, weights=True):
                                       ow.data_ptr() if ow is not None else None, p,
                                       _stream(stream))
             # done with `tiles` and the inputs, as slg_filter is on return
-            (stream or torch.cuda.current_stream()).synchronize()
+            st.synchronize()
         if rc != 0:
             raise SlgError(rc, "slg_filter")
         return oi[:p], oj[:p], (ow[:p] if ow is not None else None)

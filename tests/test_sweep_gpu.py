@@ -161,3 +161,29 @@ def test_filter_tiles(size, s):
     # an offset of one entry: no alignment is assumed
     a, b, c = slg.filter_pairs(i[1:], i[1:] + 1, w[1:], s)
     assert torch.equal(a, idx[idx > 0])
+
+
+def test_filter_takes_its_scratch_on_the_stream_given(monkeypatch):
+    h = hg.chung_lu(20_000, 40_000, seed=3, size_cap=500)
+    base = slg.build(slg.to_device(h), 1)
+    want = [slg.filter_pairs(*base, s) for s in (2, 3)]
+    torch.cuda.synchronize()
+    real, seen = torch.empty, []
+
+    def empty(*a, **k):
+        if k.get("dtype") == torch.int64:
+            seen.append(torch.cuda.current_stream().cuda_stream)
+        return real(*a, **k)
+
+    monkeypatch.setattr(torch, "empty", empty)
+    class Handle:  # all that a call reads of a stream
+        def __init__(self, st):
+            self.cuda_stream = st.cuda_stream
+
+    side = torch.cuda.Stream()
+    for st in (side, Handle(side), None):
+        for s, ref in zip((2, 3), want):
+            got = slg.filter_pairs(*base, s, stream=st)
+            torch.cuda.synchronize()
+            assert all(torch.equal(a, b) for a, b in zip(got, ref))
+    assert seen == [side.cuda_stream] * 4 + [torch.cuda.current_stream().cuda_stream] * 2
