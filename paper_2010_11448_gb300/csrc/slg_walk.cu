@@ -706,9 +706,19 @@ int giant_ctas() { return giant_ctas_for_device(); }
 
 namespace {
 
-// Two streams beside the caller's for the bins' kernels, and the events that
-// order them: this host thread's, made on first use on a device (one set per
-// thread; given back when the thread ends or turns to another device).
+// Two streams beside the caller's for the bins' kernels, of the same priority, and
+// the events that order them: this host thread's, made on first use on a device
+// (one set per thread and priority; given back when the thread ends or turns to
+// another device).
+constexpr int kPriorities = 8;  // 0 (the least) to -5 on this GPU
+
+// The index of the stream's priority, or -1.
+int priority_index(cudaStream_t st, int *priority) {
+  *priority = 0;
+  if (cudaStreamGetPriority(st, priority) != cudaSuccess) return cudaGetLastError(), -1;
+  return *priority <= 0 && *priority > -kPriorities ? -*priority : -1;
+}
+
 struct SideStreams {
   int dev = -1;
   bool ok = false;
@@ -727,7 +737,7 @@ struct SideStreams {
   // Whether they can be forked from st.  A stream that was forked into a
   // capture stays in it until the capture ends, so in the meantime they serve
   // that capture only.
-  bool ready(cudaStream_t st) {
+  bool ready(cudaStream_t st, int priority) {
     int d = 0;
     if (cudaGetDevice(&d) != cudaSuccess) return false;
     if (d != dev) {
@@ -737,7 +747,7 @@ struct SideStreams {
       cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
       cudaThreadExchangeStreamCaptureMode(&mode);
       for (cudaStream_t &x : s)
-        ok &= cudaStreamCreateWithFlags(&x, cudaStreamNonBlocking) == cudaSuccess;
+        ok &= cudaStreamCreateWithPriority(&x, cudaStreamNonBlocking, priority) == cudaSuccess;
       for (cudaEvent_t *x : {&fork, &done[0], &done[1]})
         ok &= cudaEventCreateWithFlags(x, cudaEventDisableTiming) == cudaSuccess;
       cudaThreadExchangeStreamCaptureMode(&mode);
@@ -785,7 +795,7 @@ cudaError_t launch_walk(const WalkLaunch &L, cudaStream_t st, int32_t *launches,
     if (err == cudaSuccess) err = e;
   };
   auto empty = [&](int bin) { return (L.skip >> bin) & 1u; };
-  static thread_local SideStreams side;
+  static thread_local SideStreams sides[kPriorities];
   constexpr unsigned kSkipSparse =
       kSkipSparseBig | kSkipSparseSmall | kSkipFlatBig | kSkipFlatSmall;
   const bool has_sparse = L.sparse_scratch && (L.skip & kSkipSparse) != kSkipSparse;
@@ -793,7 +803,11 @@ cudaError_t launch_walk(const WalkLaunch &L, cudaStream_t st, int32_t *launches,
   const bool chain = has_sparse || dense_small;
   const bool ctas = !empty(kBinWarp) || !empty(kBinCtaS) || !empty(kBinCtaL) ||
                     !empty(kBinRows);
-  const bool fork = !ev && dense_big && (chain || ctas) && side.ready(st);
+  const bool may_fork = !ev && dense_big && (chain || ctas);
+  int priority = 0;
+  const int pi = may_fork ? priority_index(st, &priority) : -1;
+  SideStreams &side = sides[pi < 0 ? 0 : pi];
+  const bool fork = pi >= 0 && side.ready(st, priority);
   const bool use[2] = {fork && chain, fork && ctas};
   cudaStream_t s1 = use[0] ? side.s[0] : st, s2 = use[1] ? side.s[1] : st;
   if (fork) keep(cudaEventRecord(side.fork, st));

@@ -3,6 +3,7 @@ builds at once (host threads, each with its own stream or two in turn) give the
 oracle's list, and so do a plan and a build under per-bin timing, where the
 kernels follow one another."""
 import threading
+import time
 
 import numpy as np
 import pytest
@@ -82,3 +83,29 @@ def test_plan(case):
         p.execute()
         for got, s in zip(p.results(), (2, 8)):
             assert np.array_equal(as_np(got), want[s])
+
+
+def test_side_streams_have_the_priority_of_the_callers():
+    """A count on a stream of the highest priority does not wait for a kernel of
+    the default one that fills the device: its bins' kernels, on the call's side
+    streams too, go before the blocks still to come."""
+    dh = slg.to_device(hg.chung_lu(100_000, 200_000, seed=8, size_cap=6000))
+    want = slg.count(dh, 4)
+    st = slg.last_stats()
+    assert st["giant_cycles"][3] > 0 and st["rows_bin"][1] > 0  # it forks
+    high = torch.cuda.Stream(priority=-5)
+    assert slg.count(dh, 4, stream=high) == want
+    x = torch.rand(1 << 28, dtype=torch.float64, device="cuda") + 1.5
+    out = torch.empty_like(x)
+    done = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+    torch.cuda.synchronize()
+    done[0].record()
+    torch.special.zeta(x, x, out=out)  # one kernel of a million blocks
+    done[1].record()
+    t = time.perf_counter()
+    got = slg.count(dh, 4, stream=high)
+    waited = (time.perf_counter() - t) * 1e3
+    torch.cuda.synchronize()
+    assert got == want
+    busy = done[0].elapsed_time(done[1])
+    assert busy > 150 and waited < 0.3 * busy, (waited, busy)  # 10 of 616 ms; was 615
