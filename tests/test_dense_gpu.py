@@ -126,3 +126,54 @@ def test_more_tails_than_wedges_per_window():
             st = slg.last_stats()
             assert (st["giant_cycles"][3] > 0) == dense, (tail, s)
             assert np.array_equal(as_np((i, j, w)), want), (tail, s)
+
+
+# 16-bit counters at their largest value, and 32-bit ones, on a side above the
+# short path's 16,384 rows: weights of the row's size
+@pytest.mark.parametrize("k", [65_535, 65_536, 70_000])
+def test_widest_counters(k):
+    h = hub_rows(k, 20_000, n=k + 100)
+    dh = slg.to_device(h)
+    for s in (1, 2, k):
+        want = oracle.canonical(*oracle.line_graph_of(h, s, threads=8))
+        got = as_np(slg.build(dh, s))
+        assert slg.last_stats()["giant_cycles"][3] > 0
+        assert np.array_equal(got, want), s
+        assert (0, 19_999, k) in map(tuple, got[got[:, 0] == 0])
+        i, j, w = slg.build(dh, s, unweighted=True)
+        assert w is None and np.array_equal(
+            np.stack([i.cpu().numpy(), j.cpu().numpy()], 1), want[:, :2])
+        assert slg.count(dh, s) == want.shape[0]
+
+
+# the large-window instance splits its longest tails (1,024 entries per window and
+# more than a sixteenth of the row) over 32 warps: a round of all warps is 1,024
+# entries, a step two rounds.  One entry less and more than a round and a step, 15
+# tails and one too many, in one window and in two, all in a part of the window and
+# spread
+@pytest.mark.parametrize("tails", [(1_025,), (2_047, 2_048), (2_049, 4_097, 3_072, 1_024),
+                                   (30_000,), (33_000, 33_025), (2_000,) * 15, (2_000,) * 17])
+@pytest.mark.parametrize("m,spread", [(90_000, True), (150_000, False)])
+def test_split_tails_of_the_large_windows(tails, m, spread):
+    n, few = 50_000, 300
+    rng = np.random.default_rng(len(tails) + m)
+    r, c = [np.zeros(len(tails) + few, np.int64)], [np.arange(len(tails) + few)]
+    lo, hi = (1, m) if spread else (m // 2, m // 2 + 40_000)
+    for v, deg in enumerate(tails):
+        r.append(rng.choice(np.arange(lo, hi), deg, replace=False))
+        c.append(np.full(deg, v))
+    r.append(rng.integers(1, m, 3 * few))  # short tails beside them
+    c.append(np.repeat(len(tails) + np.arange(few), 3))
+    size = rng.integers(1, 4, m - 1)
+    r.append(np.repeat(np.arange(1, m), size))
+    c.append(rng.integers(1_000, n, int(size.sum())))
+    h = hg.from_pairs(np.concatenate(r), np.concatenate(c), m, n)
+    dh = slg.to_device(h)
+    mm, nn, off, idx = oracle.side(h, False)
+    for s in (1, 2, 3):
+        want = oracle.canonical(*oracle.line_graph(mm, nn, off, idx, s, rows=np.zeros(1, np.int32),
+                                                   threads=8))
+        got = as_np(slg.build_rows(dh, s, 0, 1, capacity=max(want.shape[0], 1)))
+        if sum(tails) > 2 * 2_000 and s <= 2:
+            assert slg.last_stats()["giant_cycles"][3] > 0
+        assert np.array_equal(got, want), s

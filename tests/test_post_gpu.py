@@ -143,3 +143,15 @@ def test_squeeze_of_large_id_spaces(R):
     wi, wj, wold = oracle.squeeze(i, j, R)
     assert np.array_equal(np_(si), wi) and np.array_equal(np_(sj), wj)
     assert np.array_equal(np_(old), wold)
+
+
+# the sort's tile is 4,096 pairs: one less, one, one more, two and one more
+@pytest.mark.parametrize("n", [4_095, 4_096, 4_097, 8_192, 8_193])
+@pytest.mark.parametrize("V", [1_000, 1_500_000])
+def test_adjacency_at_the_tiles_edges(V, n):
+    i, j, w = random_list(V, n, V + n)
+    assert i.size == n
+    off, adj, adj_w = slg.adjacency(*(torch.from_numpy(x).cuda() for x in (i, j, w)), V)
+    woff, wadj, wadjw = oracle.adjacency(i, j, w, V)
+    assert np.array_equal(np_(off), woff) and np.array_equal(np_(adj), wadj)
+    assert np.array_equal(np_(adj_w), wadjw)
