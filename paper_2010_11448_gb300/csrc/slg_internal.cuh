@@ -184,6 +184,7 @@ struct Meta {
   int32_t max_dense_work[2];           // largest work of a dense-bin row: big instance, other
   int32_t max_dense_size;              // most vertices of a dense-bin row
   int32_t max_row_size;                // most vertices of a row with work
+  int32_t longest_row;                 // most vertices of a row (k_validate)
   // Of a side with thresholds per row (a plan sizes its scratch by these, whatever
   // its bins): most pairs a dense-bin row can have, big instance and other, and
   // largest work of a row that the sparse bin could take.
