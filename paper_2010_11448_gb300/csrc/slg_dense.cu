@@ -163,9 +163,9 @@ __device__ __forceinline__ int32_t dn_sweep(const int32_t *__restrict__ c_idx, i
     }
 #pragma unroll
     for (int u = 0; u < UL; ++u) {
-      const int32_t i = en[u].x + lane;
-      f[u][0] = i < en[u].y ? __ldg(c_idx + i) : 0x7fffffff;
-      f[u][1] = i + 32 < en[u].y ? __ldg(c_idx + i + 32) : 0x7fffffff;
+      const uint32_t i = (uint32_t)en[u].x + lane, end = (uint32_t)en[u].y;  // (as above)
+      f[u][0] = i < end ? __ldg(c_idx + i) : 0x7fffffff;
+      f[u][1] = i + 32 < end ? __ldg(c_idx + i + 32) : 0x7fffffff;
     }
 #pragma unroll
     for (int u = 0; u < UL; ++u) {
@@ -178,9 +178,9 @@ __device__ __forceinline__ int32_t dn_sweep(const int32_t *__restrict__ c_idx, i
                           __popc(__ballot_sync(0xffffffffu, v1));
         cur += n;
         if (n < 64) break;
-        const int32_t i = cur + lane;
-        a = i < en[u].y ? __ldg(c_idx + i) : 0x7fffffff;
-        b = i + 32 < en[u].y ? __ldg(c_idx + i + 32) : 0x7fffffff;
+        const uint32_t i = (uint32_t)cur + lane, end = (uint32_t)en[u].y;
+        a = i < end ? __ldg(c_idx + i) : 0x7fffffff;
+        b = i + 32 < end ? __ldg(c_idx + i + 32) : 0x7fffffff;
       }
       if (cur != en[u].x) {
         *any = true;
@@ -200,8 +200,8 @@ __device__ __forceinline__ int32_t dn_sweep(const int32_t *__restrict__ c_idx, i
     }
 #pragma unroll
     for (int u = 0; u < US; ++u) {
-      const int32_t i = en[u].x + l8;
-      f[u] = i < en[u].y ? __ldg(c_idx + i) : 0x7fffffff;
+      const uint32_t i = (uint32_t)en[u].x + l8;
+      f[u] = i < (uint32_t)en[u].y ? __ldg(c_idx + i) : 0x7fffffff;
     }
 #pragma unroll
     for (int u = 0; u < US; ++u) {
@@ -212,8 +212,8 @@ __device__ __forceinline__ int32_t dn_sweep(const int32_t *__restrict__ c_idx, i
         const int32_t n = __popc((__ballot_sync(0xffffffffu, v) >> (sub << 3)) & 0xFFu);
         cur += n;
         if (!__any_sync(0xffffffffu, n == 8)) break;
-        const int32_t i = cur + l8;
-        a = n == 8 && i < en[u].y ? __ldg(c_idx + i) : 0x7fffffff;
+        const uint32_t i = (uint32_t)cur + l8;
+        a = n == 8 && i < (uint32_t)en[u].y ? __ldg(c_idx + i) : 0x7fffffff;
       }
       if (cur != en[u].x) {
         *any = true;

@@ -36,12 +36,13 @@ __global__ __launch_bounds__(kValNT) void k_validate(const int32_t *__restrict__
   bool bad = false;
   int32_t most = 0;
   // ids k, k + step, ... of the row [lo, hi)
-  auto check = [&](int32_t lo, int32_t hi, int32_t k0, int32_t step) {
+  // (unsigned: the last of the four may lie beyond 2^31)
+  auto check = [&](uint32_t lo, uint32_t hi, uint32_t k0, uint32_t step) {
     for (; k0 < hi; k0 += 4 * step) {
       int32_t x[4], y[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
-        const int32_t k = k0 + u * step;
+        const uint32_t k = k0 + u * step;
         x[u] = k < hi ? __ldg(idx + k) : 0;
         y[u] = k < hi && k > lo ? __ldg(idx + k - 1) : -1;
       }
@@ -329,13 +330,13 @@ __global__ __launch_bounds__(kRowsNT) void k_rows_work(Side s, int32_t smin, int
       core_row = core.row_rank && core.row_rank[e + 1] != core.row_rank[e];
     }
     // tail lengths of incidences k0, k0 + step, ... of [.., b)
-    auto sum = [&](int32_t k0, int32_t b, int32_t step) {
+    auto sum = [&](uint32_t k0, uint32_t b, uint32_t step) {
       int32_t n = 0;
       for (; k0 < b; k0 += 4 * step) {
         int32_t tb[4], te[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-          const int32_t k = k0 + u * step;
+          const uint32_t k = k0 + u * step;
           tb[u] = k < b ? tail_beg[k] : 0;
           te[u] = k < b ? tail_end[k] : 0;
         }

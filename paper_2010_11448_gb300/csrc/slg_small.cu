@@ -72,12 +72,12 @@ __global__ __launch_bounds__(kCkNT) void k_small_check(Side s, int32_t smin,
         }
       }
       if (!map) continue;
-      auto check = [&](int32_t a, int32_t b, int32_t k0, int32_t step) {
+      auto check = [&](uint32_t a, uint32_t b, uint32_t k0, uint32_t step) {
         for (; k0 < b; k0 += 4 * step) {
           int32_t v[4], p[4];
 #pragma unroll
           for (int u = 0; u < 4; ++u) {
-            const int32_t k = k0 + u * step;
+            const uint32_t k = k0 + u * step;
             v[u] = k < b ? __ldg(idx + k) : 0;
             p[u] = k < b && k > a ? __ldg(idx + k - 1) : -1;
           }
@@ -208,29 +208,29 @@ __global__ __launch_bounds__(kSwNT) void k_small_walk(SmallWalk w, EmitArgs a) {
       const int32_t n = min(kSwNT, k1 - base);
       const int l8 = lane & 7;
       for (int32_t x0 = tid >> 3; x0 < n; x0 += 4 * (kSwNT / 8)) {
-        int2 t[4];
+        uint2 t[4];  // (unsigned: a place may lie beyond 2^31)
         int32_t f[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
           const int32_t x = x0 + u * (kSwNT / 8);
-          t[u] = x < n ? s_tail[x] : make_int2(0, 0);
-          if (t[u].y - t[u].x > kSwLongMin) t[u].y = t[u].x;
-          t[u].x += l8;
-          f[u] = t[u].x < t[u].y ? __ldg(w.s.c_idx + t[u].x) : -1;
+          const int2 tail = x < n ? s_tail[x] : make_int2(0, 0);
+          t[u] = make_uint2(tail.x, tail.y - tail.x > kSwLongMin ? tail.x : tail.y);
+          f[u] = t[u].x + l8 < t[u].y ? __ldg(w.s.c_idx + t[u].x + l8) : -1;
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
           if (f[u] >= 0) count(f[u]);
-          for (int32_t i = t[u].x + 8; i < t[u].y; i += 8) count(__ldg(w.s.c_idx + i));
+          for (uint32_t i = t[u].x + l8 + 8; i < t[u].y; i += 8) count(__ldg(w.s.c_idx + i));
         }
       }
       for (int32_t x = wq; x < n; x += kSwNW) {
         const int2 t = s_tail[x];
         if (t.y - t.x <= kSwLongMin) continue;
-        for (int32_t i = t.x + lane; i < t.y; i += 128) {
+        const uint32_t end = (uint32_t)t.y;
+        for (uint32_t i = (uint32_t)t.x + lane; i < end; i += 128) {
           int32_t f[4];
 #pragma unroll
-          for (int u = 0; u < 4; ++u) f[u] = i + 32 * u < t.y ? __ldg(w.s.c_idx + i + 32 * u) : -1;
+          for (int u = 0; u < 4; ++u) f[u] = i + 32 * u < end ? __ldg(w.s.c_idx + i + 32 * u) : -1;
 #pragma unroll
           for (int u = 0; u < 4; ++u)
             if (f[u] >= 0) count(f[u]);
