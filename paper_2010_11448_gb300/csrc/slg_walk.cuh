@@ -366,7 +366,7 @@ __device__ __forceinline__ void rank_keys(unsigned long long *k, int32_t n, Fn &
 template <int NT, int SPT, bool RUNS = (NT >= 512)>
 __device__ __forceinline__ int32_t table_collect(unsigned long long *tab, int32_t T, int32_t smin,
                                                  bool sort, int32_t *ws, int32_t *sorted_at,
-                                                 int32_t *used, int32_t sort_cap = 0x7fffffff) {
+                                                 int32_t *used) {
   constexpr int RND = SPT < 8 ? SPT : 8;
   int32_t run = 0;
   for (int32_t r0 = 0; r0 * NT < T; r0 += RND) {
@@ -389,7 +389,6 @@ __device__ __forceinline__ int32_t table_collect(unsigned long long *tab, int32_
     run += total;
   }
   *used = T;
-  if (sort && run > sort_cap) return -1;  // uniform: too many to order in the table
   if (sort && run > 0) {
     __syncthreads();  // compaction writes done
     int32_t u;
