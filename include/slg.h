@@ -438,7 +438,7 @@ int slg_tile_overlap(const uint8_t *A, int32_t rows_pad, int32_t cols_pad,
  *   last execution, if any.
  * slg_plan_info -- the autotuner's choice, in `bins` (6 entries): the warp,
  *   CTA-small and CTA-large work limits, the sparse bin's upper work limit
- *   (0: bin off) and lower limit, and the dense-row ratio of the giant bin;
+ *   (0: bin off) and lower limit, and the scale of the dense bin's threshold;
  *   the tuned build time in ms and the kernels per execution.
  */
 typedef struct slg_plan slg_plan;
@@ -500,7 +500,8 @@ typedef struct slg_stats {
   int64_t pairs;           /* |L_s| */
   int64_t rows_active;     /* rows with size >= s */
   int64_t rows_bin[5];     /* rows per bin: warp, CTA-S (and rows bin),
-                              CTA-L, giant (and dense bin), sparse */
+                              CTA-L, giant (and dense bin), sparse (and
+                              flat bin) */
   int64_t wedges_bin[5];   /* wedges per bin */
   int64_t incid_bin[5];    /* CSR incidences of the rows of each bin */
   int64_t pairs_bin[5];    /* pairs emitted by each bin */
@@ -521,7 +522,7 @@ typedef struct slg_stats {
   int64_t max_row_work;    /* largest wedge count of one row */
   float ms_relabel;        /* SLG_RELABEL_*: building the renumbered side */
   float ms_order;          /* SLG_RELABEL_*: caller ids and (i, j) order */
-  int64_t sparse_cycles[5]; /* sparse bin, SM clock cycles summed over CTAs:
+  int64_t sparse_cycles[5]; /* sparse and flat bins, SM clock cycles summed over CTAs:
                                row set-up, first pass, second pass, collect
                                and order the survivors, emit and clear */
   float ms_tile;           /* the tensor-core tile kernel of the dense core

@@ -1979,7 +1979,7 @@ extern "C" int slg_plan_create(const slg_hypergraph *hs, const int32_t *s, int32
   }
   // 4. autotuner: bin thresholds, timed on this batch
   // candidates: CTA-bin limits, the sparse bin's range (0: off) and the
-  // dense-row ratio
+  // dense bin's threshold
   const Bins cands[] = {Bins{},
                         Bins{64, 1024, 4096},
                         Bins{128, 512, 4096},

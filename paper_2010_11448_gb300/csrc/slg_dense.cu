@@ -12,8 +12,10 @@
 //
 // Counters are as narrow as the row allows: a count |e ∩ f| never exceeds
 // |e|, so rows of at most 15, 255 and 65,535 vertices use 4-, 8- and 16-bit
-// counters packed in 32-bit words (additions never carry into a neighbour),
-// and a window of kDnBytes holds 128K, 64K or 32K ids (16K with 32 bits).
+// counters packed in 32-bit words (additions never carry into a neighbour).
+// A window of the small instance's 10,240 words holds 81,920 ids with 4-bit and
+// 40,960 with 8-bit counters; one of the large instance's 48,128 words 96,256 with
+// 16 bits and 48,128 with 32.
 //
 // A counter that reaches s sets its id's bit in a map of survivors (one more
 // shared atomic per surviving pair), so that the window's end reads one bit
@@ -21,9 +23,8 @@
 // and far-end loads, so several list entries are in flight per warp, and the
 // fewer windows a row has the better: rows of more than kDenseBigSize
 // vertices (short pieces of many tails: 3 to 8 entries of a tail in a window
-// of 26K ids) take an instance with one CTA of 1,024 threads per SM and a
-// window of 96K ids; the others one with four CTAs of 256 threads and windows
-// of 80K (4-bit) or 40K ids (8-bit counters).
+// of 26K ids) take the large instance, one CTA of 1,024 threads per SM; the
+// others the small one, four CTAs of 256 threads.
 //
 // Measured on chung_lu_1m (1M x 2M) against the partitioned hash buckets and
 // dense windows of the giant bin that these rows took before: L_8 of H, giant

@@ -279,7 +279,8 @@ __global__ __launch_bounds__(kRowsNT) void k_tails(int64_t k0, int64_t k1,
   }
 }
 
-// A block handles kRowsPerBlock consecutive rows, one warp per row at a time.
+// A block handles kRowsPerBlock consecutive rows, eight lanes each (long rows and
+// core rows by whole warps).
 // The row's work is the sum of its tail lengths (k_tails; core columns of core
 // rows are set here).  Rows with
 // work > 0 are appended to their bin's list (one global atomic per bin and
