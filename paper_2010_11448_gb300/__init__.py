@@ -570,10 +570,13 @@ def filter_pairs(i, j, w, s: int, out=None, stream=None, weights=True):
         lib.slg_filter_tiles(n, ctypes.byref(cnt))
         # taken from the allocator on the stream that uses them: on another, a
         # block that is still being written there could be handed out
-        st = (torch.cuda.current_stream() if stream is None else
-              torch.cuda.ExternalStream(stream.cuda_stream, device=i.device))
-        with torch.cuda.stream(st):
+        if stream is None:
+            st = torch.cuda.current_stream()
             tiles = torch.empty(cnt.value, dtype=torch.int64, device=i.device)
+        else:
+            st = torch.cuda.ExternalStream(stream.cuda_stream, device=i.device)
+            with torch.cuda.stream(st):
+                tiles = torch.empty(cnt.value, dtype=torch.int64, device=i.device)
         rc = lib.slg_filter_count(w.data_ptr(), n, int(s), tiles.data_ptr(), ctypes.byref(cnt),
                                   _stream(stream))
         p = int(cnt.value)

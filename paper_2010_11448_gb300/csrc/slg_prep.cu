@@ -14,6 +14,12 @@ namespace {
 
 constexpr int kValNT = 256;
 
+// Sides whose longest row matters to the map (k_csr2csc): k_validate notes it for
+// these only, since a maximum over all warps costs it 10 us.
+__host__ __device__ __forceinline__ bool long_rows(const Side &s) {
+  return s.nnz >= 128ll * s.R;
+}
+
 // Offsets monotone inside [0, nnz], ids inside [0, cols), every row strictly
 // ascending.  Eight lanes per row (rows hold 10 to 20 ids on average; a warp
 // per row left two thirds of its lanes idle: 257 us for both sides of 500K x
@@ -91,14 +97,13 @@ __global__ __launch_bounds__(kValNT) void k_validate(const int32_t *__restrict__
 // through the column ids at the same pace and share their sectors (200K rows of 800
 // of 30M columns 2.7 instead of 5.7 ms, 100K of 3,000 of 60M 4.0 instead of 11.8).
 constexpr int kMapK = 8;
-constexpr int kMapRowMean = 128;          // vertices per row from which
 constexpr int64_t kMapRowShare = 5'000;   // incidences per vertex of the longest row
 __global__ __launch_bounds__(kValNT) void k_csr2csc(Side s, int32_t *__restrict__ csr2csc,
                                                     Meta *meta) {
   if (meta->err) return;
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * kValNT + threadIdx.x) >> 5;
-  if (s.nnz >= (int64_t)kMapRowMean * s.R && meta->longest_row * kMapRowShare <= s.nnz) {
+  if (long_rows(s) && meta->longest_row * kMapRowShare <= s.nnz) {
     const int64_t nwarps = ((int64_t)gridDim.x * kValNT) >> 5;
     bool bad = false;
     for (int64_t f = warp; f < s.R; f += nwarps) {
@@ -506,7 +511,7 @@ cudaError_t launch_validate(const Side &s, Meta *meta, cudaStream_t st) {
   const int wpb = kValNT / 8;  // rows per block
   k_validate<<<grid_for(s.R, wpb, 65536), kValNT, 0, st>>>(s.r_off, s.r_idx, s.R, s.C, s.nnz, meta,
                                                           kWhereRowOffsets, kWhereRowIds,
-                                                          &meta->longest_row);
+                                                          long_rows(s) ? &meta->longest_row : nullptr);
   k_validate<<<grid_for(s.C, wpb, 65536), kValNT, 0, st>>>(s.c_off, s.c_idx, s.C, s.R, s.nnz, meta,
                                                           kWhereColOffsets, kWhereColIds,
                                                           nullptr);
