@@ -570,8 +570,8 @@ def filter_pairs(i, j, w, s: int, out=None, stream=None, weights=True):
         lib.slg_filter_tiles(n, ctypes.byref(cnt))
         # taken from the allocator on the stream that uses them: on another, a
         # block that is still being written there could be handed out
+        st = None
         if stream is None:
-            st = torch.cuda.current_stream()
             tiles = torch.empty(cnt.value, dtype=torch.int64, device=i.device)
         else:
             st = torch.cuda.ExternalStream(stream.cuda_stream, device=i.device)
@@ -587,7 +587,7 @@ def filter_pairs(i, j, w, s: int, out=None, stream=None, weights=True):
                                       ow.data_ptr() if ow is not None else None, p,
                                       _stream(stream))
             # done with `tiles` and the inputs, as slg_filter is on return
-            st.synchronize()
+            (st or torch.cuda.current_stream()).synchronize()
         if rc != 0:
             raise SlgError(rc, "slg_filter")
         return oi[:p], oj[:p], (ow[:p] if ow is not None else None)
