@@ -211,19 +211,30 @@ WALK_KERNELS = ["k_walk_warp", "k_walk_rows + k_walk_cta<256,2048>", "k_walk_cta
 NBINS = len(WALK_KERNELS)
 
 
-def recorded_traffic(kernel: str):
-    """DRAM bytes per launch of `kernel` from the committed ncu summary, if
-    it was taken on the current walk source (else None)."""
-    path = os.path.join(ROOT, "profiles", "traffic.txt")
-    src = os.path.join(ROOT, "paper_2010_11448_gb300", "csrc", "slg_walk.cu")
+BINS = ["warp", "cta_small", "cta_large", "giant", "sparse"]
+WALK_SOURCES = ["slg_dense.cu", "slg_internal.cuh", "slg_sparse.cu", "slg_walk.cu", "slg_walk.cuh"]
+
+
+def walk_sources_sha() -> str:
+    h = hashlib.sha256()
+    for name in WALK_SOURCES:
+        with open(os.path.join(ROOT, "paper_2010_11448_gb300", "csrc", name), "rb") as fh:
+            h.update(fh.read())
+    return h.hexdigest()[:16]
+
+
+def recorded_traffic(b: int, path: str | None = None):
+    """DRAM bytes per build of bin b's kernels from the committed ncu summary,
+    if it was taken on the current walk sources (else None)."""
+    path = path or os.path.join(ROOT, "profiles", "traffic.txt")
     if not os.path.exists(path):
         return None
-    sha = hashlib.sha256(open(src, "rb").read()).hexdigest()[:16]
+    sha = walk_sources_sha()
     for ln in open(path):
         kv = dict(x.split("=", 1) for x in ln.split() if "=" in x)
-        if kv.get("kernel") == kernel and kv.get("src_sha") == sha and \
+        if kv.get("bin") == BINS[b] and kv.get("src_sha") == sha and \
                 kv.get("workload") == WORKLOAD:
-            return float(kv["bytes_per_launch"])
+            return float(kv["bytes_per_build"])
     return None
 
 
@@ -434,7 +445,7 @@ def run_ours(args):
     achieved = bytes_l / t_l / 1e9 if t_l > 0 else 0.0
     roofline = {"bound": "hbm", "kernel": WALK_KERNELS[b], "achieved": achieved,
                 "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-                "peak_source": peak_kind, "traffic": recorded_traffic(WALK_KERNELS[b]),
+                "peak_source": peak_kind, "traffic": recorded_traffic(b),
                 "algorithmic_bytes_per_launch": bytes_l, "ms_per_launch": t_l * 1e3,
                 "walk_ms_share": {WALK_KERNELS[i]: stats_acc["ms_walk"][i] / max(ms, 1e-9)
                                   for i in range(NBINS)}}
