@@ -61,11 +61,17 @@ constexpr int32_t kSparseBigWork = SLG_SP_BIG_WORK;
 #define SLG_SPARSE_MAX_WORK 65536
 #endif
 constexpr int32_t kSparseMaxWork = SLG_SPARSE_MAX_WORK;
-// Rows of many vertices whose tails are mostly short: of these, the flat bin
-// takes rows of up to kFlatMaxWork wedges.
+// Rows of the flat bin, of up to kFlatMaxWork wedges: many vertices whose tails are
+// mostly short, or tails alike, of which the longest is no eighth of the row, so that
+// setting it aside gains little (400K rows of 40 vertices with 40 far ends per tail,
+// counting pass 6.0 -> 4.3 ms, of 100 with 50 14.5 -> 10.8).  Larger such rows go to
+// the giant bin: the sparse bin's ranges search every tail (1M rows of 400 with 40
+// 267 -> 221 ms; alike is a 32nd there, to leave the others in the sparse bin).
 constexpr int32_t kFlatMaxWork = 16384;
-__host__ __device__ __forceinline__ bool short_tails(int32_t work, int32_t size) {
-  return size > 48 && work < 32ll * size;
+__host__ __device__ __forceinline__ bool short_tails(int32_t work, int32_t size, int32_t longest) {
+  return (size > 48 && work < 32ll * size) ||
+         (size > 32 && work < 128ll * size &&
+          (work <= kFlatMaxWork ? 8ll : 32ll) * longest <= work);
 }
 // Whether the flat bin's kernels run, by its wedges and the sparse bin's; else
 // its rows are given to the sparse bin (launch_join_flat).  A kernel lasts as long
@@ -73,7 +79,7 @@ __host__ __device__ __forceinline__ bool short_tails(int32_t work, int32_t size)
 // (counting pass of 120K x 240K, host builds of 200K x 400K: 800 and 3,470 us so,
 // 870 and 3,570 with kernels of their own; chung_lu_1m the same both ways).
 __host__ __device__ __forceinline__ bool flat_kernels(long long flat, long long sparse) {
-  return flat > 0 && (2 * flat >= sparse || flat >= 1ll << 26);
+  return flat > 0 && (flat >= 2 * sparse || flat >= 1ll << 28);
 }
 // Rows of more vertices leave the rows bin to the small CTA bin: the kernel lasts
 // as long as its longest row, and a warp there walks 32 tails at a time, a CTA 256

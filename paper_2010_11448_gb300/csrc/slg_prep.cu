@@ -302,7 +302,7 @@ __global__ __launch_bounds__(kRowsNT) void k_rows_work(Side s, int32_t smin, int
                                                        int32_t *__restrict__ bin_rows,
                                                        Meta *meta) {
   if (meta->err) return;
-  __shared__ int32_t s_work[kRowsPerBlock];
+  __shared__ int32_t s_work[kRowsPerBlock], s_longest[kRowsPerBlock];  // wedges, longest tail
   // block maxima of the row work (all rows, giant-bin, sparse- or flat-bin, the dense
   // bin's two instances' rows) and size (dense-bin rows, all rows), and a plan's bounds: one
   // global atomicMax each per
@@ -327,7 +327,7 @@ __global__ __launch_bounds__(kRowsNT) void k_rows_work(Side s, int32_t smin, int
   for (int i0 = warp * 4; i0 < kRowsPerBlock; i0 += kRowsNT / 8) {
     const int i = i0 + (lane >> 3), l8 = lane & 7;
     const int32_t e = r0 + i;
-    int32_t work = 0, lo = 0, hi = 0;
+    int32_t work = 0, longest = 0, lo = 0, hi = 0;
     bool active = false, core_row = false;
     if (e < row_end) {
       lo = __ldg(s.r_off + e);
@@ -335,7 +335,7 @@ __global__ __launch_bounds__(kRowsNT) void k_rows_work(Side s, int32_t smin, int
       active = hi - lo >= s_of(s.row_s, smin, e);
       core_row = core.row_rank && core.row_rank[e + 1] != core.row_rank[e];
     }
-    // tail lengths of incidences k0, k0 + step, ... of [.., b)
+    // tail lengths of incidences k0, k0 + step, ... of [.., b): their sum, the longest
     auto sum = [&](uint32_t k0, uint32_t b, uint32_t step) {
       int32_t n = 0;
       for (; k0 < b; k0 += 4 * step) {
@@ -347,14 +347,20 @@ __global__ __launch_bounds__(kRowsNT) void k_rows_work(Side s, int32_t smin, int
           te[u] = k < b ? tail_end[k] : 0;
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) n += te[u] - tb[u];
+        for (int u = 0; u < 4; ++u) {
+          n += te[u] - tb[u];
+          longest = max(longest, te[u] - tb[u]);
+        }
       }
       return n;
     };
     const bool whole = active && (core_row || hi - lo > kValLong);
     if (active && !whole) work = sum(lo + l8, hi, 8);
 #pragma unroll
-    for (int d = 4; d > 0; d >>= 1) work += __shfl_xor_sync(0xffffffffu, work, d);
+    for (int d = 4; d > 0; d >>= 1) {
+      work += __shfl_xor_sync(0xffffffffu, work, d);
+      longest = max(longest, __shfl_xor_sync(0xffffffffu, longest, d));
+    }
     unsigned big = __ballot_sync(0xffffffffu, l8 == 0 && whole);
     while (big) {
       const int src = __ffs(big) - 1;
@@ -362,6 +368,8 @@ __global__ __launch_bounds__(kRowsNT) void k_rows_work(Side s, int32_t smin, int
       const int32_t x = __shfl_sync(0xffffffffu, e, src);
       const int32_t a = __shfl_sync(0xffffffffu, lo, src), b = __shfl_sync(0xffffffffu, hi, src);
       int32_t n = 0;
+      const int32_t own = longest;  // of this lane's own row
+      longest = 0;
       if (!__shfl_sync(0xffffffffu, (int)core_row, src)) {
         n = sum(a + lane, b, 32);
       } else {
@@ -384,7 +392,12 @@ __global__ __launch_bounds__(kRowsNT) void k_rows_work(Side s, int32_t smin, int
         }
       }
       n = __reduce_add_sync(0xffffffffu, n);
-      if ((lane & 24) == (src & 24)) work = n;
+      const int32_t most = __reduce_max_sync(0xffffffffu, longest);
+      longest = own;
+      if ((lane & 24) == (src & 24)) {
+        work = n;
+        longest = most;
+      }
     }
     if (l8 == 0) {
       if (e < row_end) {
@@ -400,6 +413,7 @@ __global__ __launch_bounds__(kRowsNT) void k_rows_work(Side s, int32_t smin, int
       // core rows take part even without wedges (their tile counts are added
       // by the bin), marked by a negative work entry here
       s_work[i] = e < row_end ? (core_row && active ? -1 - work : work) : 0;
+      s_longest[i] = longest;
     }
   }
   __syncthreads();
@@ -419,10 +433,11 @@ __global__ __launch_bounds__(kRowsNT) void k_rows_work(Side s, int32_t smin, int
       // a row whose far ends are dense in its span takes the dense bin; else
       // one with s >= 2 from bins.bloom up to bins.sparse wedges the sparse or
       // the flat bin
+      const bool sparse = !forced && my_work > bins.bloom && my_work <= bins.sparse && se >= 2;
       if ((forced || my_work > kDenseMinWork) && is_dense(my_work, size, se, span, bins.dense))
         my_bin = kBinDense;
       else if (!forced && my_work > bins.bloom && my_work <= bins.sparse && se >= 2) {
-        if (!bins.flat || !short_tails(my_work, size)) my_bin = kBinSparse;
+        if (!bins.flat || !short_tails(my_work, size, s_longest[threadIdx.x])) my_bin = kBinSparse;
         else if (my_work <= kFlatMaxWork) my_bin = kBinFlat;
       }
       else if (!forced && my_work <= bins.ctas && se >= 2)

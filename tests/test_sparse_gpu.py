@@ -350,3 +350,16 @@ def test_rows_of_many_vertices_are_not_left_to_a_warp():
     finally:
         slg.set_profiling(False)
     assert ms[2] < 1.7 * ms[1], ms
+
+
+# tails alike (the longest no eighth of the row) of 32 to 127 far ends on average, in
+# rows of more than 32 vertices; a longest tail at, below and above that share; above
+# 16,384 wedges
+@pytest.mark.parametrize("k,lens,repeat", [
+    (32, (40,), 3), (33, (40,), 3), (34, (100, 127), 4), (40, (128,), 4), (64, (127,), 5),
+    (33, (60, 60, 60, 60, 60, 60, 60, 60, 60, 60, 267), 3),
+    (33, (60, 60, 60, 60, 60, 60, 60, 60, 60, 60, 600), 3),
+    (130, (126,), 8), (131, (126,), 8), (300, (64,), 10)])
+@pytest.mark.parametrize("mixed", [False, True])
+def test_tails_alike(k, lens, repeat, mixed):
+    test_short_tails(k, lens, repeat, mixed)
