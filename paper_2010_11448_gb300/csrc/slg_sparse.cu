@@ -518,12 +518,11 @@ __global__ __launch_bounds__(C::NT, C::MINB) void k_walk_sparse(
 
 // ------------------------------------------------------------ short tails --
 //
-// The flat bin: rows with s >= 2 of 1,025 to 16,384 wedges whose tails are short
-// (more than 48 vertices, under 32 far ends per tail on average: web-shaped and
-// uniform inputs with a mean of 5 to 25 hyperedges per vertex).  A warp per tail,
-// as in the sparse bin, leaves most of its lanes idle there (58 to 190 instead of
-// 10 to 15 CTA cycles per wedge), and no tail is long enough to be worth setting
-// aside.  The row's wedges are flattened: wedge i's tail is found by a search over
+// The flat bin: rows with s >= 2 of 1,025 to 16,384 wedges whose tails are short or
+// alike (short_tails: web-shaped and uniform inputs).  A warp per tail, as in the
+// sparse bin, leaves most of its lanes idle there (58 to 190 instead of 10 to 15 CTA
+// cycles per wedge), and no tail is long enough to be worth setting aside.  The
+// row's wedges are flattened: wedge i's tail is found by a search over
 // the tails' prefix sums, each warp loads kSpSeg consecutive wedges per step and
 // copies their far ends to the CTA's scratch, so that the second pass reads them
 // in order.  Filters, table and survivors are the sparse bin's; a row that
@@ -532,7 +531,7 @@ __global__ __launch_bounds__(C::NT, C::MINB) void k_walk_sparse(
 // step of chung_lu_1m, which has few such rows, took 107.4 instead of 105.4 ms.)
 //
 // 100K rows of 250 of 1.9M vertices, L_2, whole counting pass: 6.8 -> 2.6 ms; 200K
-// rows of 400 of 9M 19.7 -> 9.3; 4M x 10M lognormal hyperedges with the tile path,
+// rows of 400 of 9M 19.7 -> 8.7; 4M x 10M lognormal hyperedges with the tile path,
 // L_2, L_8, L_32, per build 23.3, 23.9, 22.5 -> 19.1, 18.0, 16.7.  Mean tails of
 // up to 8, 16, 32: 5.0, 2.7, 2.7 ms and (100K rows of 100 of 300K) 2.9, 2.6, 1.7.
 
