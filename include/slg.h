@@ -281,6 +281,8 @@ int slg_wedges(const slg_hypergraph *h, int32_t s, uint32_t flags,
  * stay NULL with row_ptr, out_w with SLG_UNWEIGHTED; nothing is needed for
  * n_pairs = 0).  A counting call before the build, and its walk, are saved.
  * A non-zero return of `alloc` ends the call with SLG_ERR_NOMEM.
+ * `alloc` may call the library itself.  The call's own memory for the pairs is
+ * guessed from the wedges, 2 GB at most; a longer list is walked twice.
  * Binned algorithm only, without relabelling (else SLG_ERR_UNSUPPORTED).
  * slg_graph_build_alloc: the same through a prepared hypergraph.
  */
