@@ -143,13 +143,14 @@ constexpr int kDenseRatio = 16;
 // wedge; so the line is drawn at a number of wedges per window.  A window also
 // visits every tail, which the other bins read once: in the large-window
 // instance, whose rows can have more tails than wedges per window, a visit after
-// the first counts as 2.5 wedges (a quarter at s = 1, where hash tables would
-// count the row).  400K rows of 1,500 of 67M vertices, counting pass at s = 2
+// the first counts as 2.5 wedges (a quarter where hash tables would count the
+// row: at s = 1, and core rows).  400K rows of 1,500 of 67M vertices, counting pass at s = 2
 // 112.7, 95.3, 90.6 ms with 0.25, 1, 2.5 (125.3 without), at s = 1 117.6, 119.6,
 // 121.3; rows of up to 100,000 vertices over 4M ids (web-shaped input with the
 // tile path) 4.6 -> 1.75 ms; step of chung_lu_1m the same all ways.
 __host__ __device__ __forceinline__ bool is_dense(int32_t work, int32_t size, int32_t s,
-                                                  int32_t span, int32_t ratio) {
+                                                  int32_t span, int32_t ratio,
+                                                  bool core = false) {
   const int lw = 5 - dense_lg_bits(size);
   const bool big = size > kDenseBigSize;
   const int32_t nwin = span / ((big ? SLG_DN_BIG_WORDS : SLG_DN_WORDS) << lw) + 1;
@@ -157,7 +158,7 @@ __host__ __device__ __forceinline__ bool is_dense(int32_t work, int32_t size, in
                       : s == 1                                     ? SLG_DENSE_T1
                       : size <= (long long)kDenseFew * (s - 2) ? SLG_DENSE_T4
                                                                    : SLG_DENSE_T2;
-  const long long visits = big ? (nwin - 1ll) * size * (s == 1 ? 4 : 40) : 0;
+  const long long visits = big ? (nwin - 1ll) * size * (s == 1 || core ? 4 : 40) : 0;
   return (long long)work * ratio >= (long long)per * 16 * nwin + visits;
 }
 

@@ -434,7 +434,7 @@ __global__ __launch_bounds__(kRowsNT) void k_rows_work(Side s, int32_t smin, int
       // one with s >= 2 from bins.bloom up to bins.sparse wedges the sparse or
       // the flat bin
       const bool sparse = !forced && my_work > bins.bloom && my_work <= bins.sparse && se >= 2;
-      if ((forced || my_work > kDenseMinWork) && is_dense(my_work, size, se, span, bins.dense))
+      if ((forced || my_work > kDenseMinWork) && is_dense(my_work, size, se, span, bins.dense, forced))
         my_bin = kBinDense;
       else if (!forced && my_work > bins.bloom && my_work <= bins.sparse && se >= 2) {
         if (!bins.flat || !short_tails(my_work, size, s_longest[threadIdx.x])) my_bin = kBinSparse;

@@ -782,7 +782,8 @@ struct SideStreams {
 // 5,777, L_1 of 100K x 200K 2,499 -> 2,287; chung_lu_1m's four lists 105.7 ms
 // both ways.  DnSmall beside the sparse bin costs more than it fills (L_2
 // sweep of 150K x 300K 10,190 -> 10,711 us), as does a fork without DnBig (L_3
-// of a dual of 30K x 60K 1,346 -> 1,362).  With per-bin timing (ev) they run
+// of a dual of 30K x 60K 1,346 -> 1,362), but for the flat bin's kernels, which last
+// as long as their longest rows too.  With per-bin timing (ev) they run
 // one after the other.
 cudaError_t launch_walk(const WalkLaunch &L, cudaStream_t st, int32_t *launches,
                         cudaEvent_t *ev) {
@@ -803,7 +804,9 @@ cudaError_t launch_walk(const WalkLaunch &L, cudaStream_t st, int32_t *launches,
   const bool chain = has_sparse || dense_small;
   const bool ctas = !empty(kBinWarp) || !empty(kBinCtaS) || !empty(kBinCtaL) ||
                     !empty(kBinRows);
-  const bool may_fork = !ev && dense_big && (chain || ctas);
+  const bool has_flat =
+      has_sparse && (L.skip & (kSkipFlatBig | kSkipFlatSmall)) != (kSkipFlatBig | kSkipFlatSmall);
+  const bool may_fork = !ev && (dense_big || (has_flat && ctas)) && (chain || ctas);
   int priority = 0;
   const int pi = may_fork ? priority_index(st, &priority) : -1;
   SideStreams &side = sides[pi < 0 ? 0 : pi];
